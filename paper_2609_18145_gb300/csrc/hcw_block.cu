@@ -192,12 +192,13 @@ __global__ void __launch_bounds__(kRowWarps * 32)
     if (lane == 0) stats[row] = make_float2(mean, rstd);
 }
 
-// One warp per position r = b n + t: z = logits[r] + bh, target v* =
-// ids[b][t + 1]; loss += (logsumexp(z) - z[v*]) / N; dlog[r][v] =
-// bf16((softmax(z)[v] - [v == v*]) / N).
+// One warp per position r = b n + t: z = logits[r] + bh (rows of ldz elements, a
+// multiple of 4), target v* = ids[b][t + 1]; loss += (logsumexp(z) - z[v*]) / N;
+// dlog[r][v] = bf16((softmax(z)[v] - [v == v*]) / N) (rows of ldd elements, a
+// multiple of 4).  Four symbols a lane and access, the last V % 4 one a lane.
 __global__ void __launch_bounds__(kRowWarps * 32)
-    ce_kernel(const float* logits, const float* bh, const int* ids, __nv_bfloat16* dlog,
-              float* loss, int B, int n, int V, float inv_N) {
+    ce_kernel(const float* logits, int ldz, const float* bh, const int* ids, __nv_bfloat16* dlog,
+              int ldd, float* loss, int B, int n, int V, float inv_N) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
     const int lane = threadIdx.x & 31;
@@ -205,35 +206,61 @@ __global__ void __launch_bounds__(kRowWarps * 32)
     if (r >= B * n) return;
     const int b = r / n, t = r % n;
     const int tgt = symbol(ids, b, t + 1, n, V);
-    const float* z = logits + (size_t)r * V;
-    float m = -INFINITY;
-    for (int v = lane; v < V; v += 32) m = fmaxf(m, z[v] + bh[v]);
-    m = warp_max(m);
-    float s = 0.f;
-    for (int v = lane; v < V; v += 32) s += expf(z[v] + bh[v] - m);
-    const float lse = m + logf(warp_sum(s));
-    for (int v = lane; v < V; v += 32) {
-        const float p = expf(z[v] + bh[v] - lse) - (v == tgt ? 1.f : 0.f);
-        dlog[(size_t)r * V + v] = __float2bfloat16_rn(p * inv_N);
+    const float* z = logits + (size_t)r * ldz;
+    __nv_bfloat16* dz = dlog + (size_t)r * ldd;
+    const int v4 = V & ~3, vt = v4 + lane;   // the lane's symbol past the whole fours
+    const bool tail = vt < V;
+    const float zt = tail ? z[vt] + bh[vt] : -INFINITY;
+    float m = zt;
+#pragma unroll 4
+    for (int v = 4 * lane; v < v4; v += 128) {
+        const float4 q = add4(ld4(z, v), ld4(bh, v));
+        m = fmaxf(m, fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)));
     }
+    m = warp_max(m);
+    float s = tail ? expf(zt - m) : 0.f;
+#pragma unroll 2
+    for (int v = 4 * lane; v < v4; v += 128) {
+        const float4 q = add4(ld4(z, v), ld4(bh, v));
+        s += (expf(q.x - m) + expf(q.y - m)) + (expf(q.z - m) + expf(q.w - m));
+    }
+    const float lse = m + logf(warp_sum(s));
+#pragma unroll 2
+    for (int v = 4 * lane; v < v4; v += 128) {
+        const float4 q = add4(ld4(z, v), ld4(bh, v));
+        st4(dz, v,
+            make_float4((expf(q.x - lse) - (v == tgt ? 1.f : 0.f)) * inv_N,
+                        (expf(q.y - lse) - (v + 1 == tgt ? 1.f : 0.f)) * inv_N,
+                        (expf(q.z - lse) - (v + 2 == tgt ? 1.f : 0.f)) * inv_N,
+                        (expf(q.w - lse) - (v + 3 == tgt ? 1.f : 0.f)) * inv_N));
+    }
+    if (tail) dz[vt] = __float2bfloat16_rn((expf(zt - lse) - (vt == tgt ? 1.f : 0.f)) * inv_N);
     if (lane == 0) atomicAdd(loss, (lse - (z[tgt] + bh[tgt])) * inv_N);
 }
 
-// out[c] += sum over a tile of kColRows rows of M[r][c] (bf16 M [T][C]; out
-// zeroed before the launch): grid (ceil(C / 256), ceil(T / kColRows)), a
-// thread per column of its tile, the rows' loads independent of each other
+// out[c] += sum over a tile of kColRows rows of M[r][c] (bf16 M, T rows of ld
+// elements, ld even; out zeroed before the launch): grid (ceil(C / 512), ceil(T /
+// kColRows)), a thread per two columns of its tile, the rows' loads independent of
+// each other
 constexpr int kColRows = 64;
-__global__ void colsum_kernel(const __nv_bfloat16* M, float* out, int T, int C) {
+__global__ void __launch_bounds__(256)
+    colsum_kernel(const __nv_bfloat16* M, int ld, float* out, int T, int C) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (c >= C) return;
     const int r0 = blockIdx.y * kColRows;
     const int r1 = min(T, r0 + kColRows);
-    float s = 0.f;
-#pragma unroll 8
-    for (int r = r0; r < r1; ++r) s += __bfloat162float(M[(size_t)r * C + c]);
-    atomicAdd(out + c, s);
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll 16
+    for (int r = r0; r < r1; ++r) {
+        const float2 f =
+            unpack_bf16x2(*reinterpret_cast<const uint32_t*>(M + (size_t)r * ld + c));
+        s0 += f.x;
+        s1 += f.y;
+    }
+    atomicAdd(out + c, s0);
+    if (c + 1 < C) atomicAdd(out + c + 1, s1);
 }
 
 // W consecutive features at element e (W = 2 or 4; e a multiple of W).
@@ -487,14 +514,18 @@ __global__ void pos_bwd_kernel(const float* dx, float* dP, int B, int n, int d) 
 namespace {
 
 // Row-major C[M][N] (fp32) = op(A) op(B) with bf16 operands and fp32
-// accumulation; A is [M][K] ([K][M] when ta), B is [K][N] ([N][K] when tb).
-// split_ws holds the partial sums when the GEMM splits K.  HCW_OK after
+// accumulation; A is [M][K] ([K][M] when ta), B is [K][N] ([N][K] when tb); lda /
+// ldc elements from one row of A / C to the next (0: dense).  split_ws holds the partial sums when the GEMM splits K.  HCW_OK after
 // counting its launches, else HCW_ERR_CUDA.
 int gemm(float* split_ws, size_t split_bytes, cudaStream_t st, int M, int N, int K, const void* A,
-         bool ta, const void* B, bool tb, float* C) {
+         bool ta, const void* B, bool tb, float* C, int lda = 0, int ldc = 0) {
+    GemmEpi epi = {};
+    epi.kind = EPI_F32;
+    epi.lda = lda;
+    epi.ldc = ldc;
     int launches = 0;
     const cudaError_t e =
-        gemm_bf16_f32(M, N, K, A, ta, B, tb, C, split_ws, split_bytes, st, &launches);
+        gemm_bf16(M, N, K, A, ta, B, tb, C, epi, split_ws, split_bytes, st, &launches);
     return count_launch(e, launches);
 }
 
@@ -504,7 +535,7 @@ int gemm(float* split_ws, size_t split_bytes, cudaStream_t st, int M, int N, int
 int gemm_ffn(cudaStream_t st, int M, int N, int K, const void* A, const void* B, bool tb,
              const float* bias, const __nv_bfloat16* aux, __nv_bfloat16* out,
              float* colsum = nullptr) {
-    GemmEpi epi;
+    GemmEpi epi = {};
     epi.kind = bias ? EPI_BIAS_RELU : EPI_RELU_GRAD;
     epi.bias = bias;
     epi.aux = aux;
@@ -533,8 +564,10 @@ size_t round256(size_t v) { return (v + 255) & ~(size_t)255; }
 //   a    [L][T][h] bf16        relu(u), the FFN's hidden activations
 //   st1, st2 [L][T], stf [T]   LayerNorm (mean, rstd)
 //   m, hf [T][d] bf16          mixing output (per layer), head input
-//   U    [T][max(h, V, d)] fp32  every GEMM output with T rows, in turn
-//   dlog [T][V] bf16; dx [T][d] fp32
+//   U    [T][max(h, V4, d)] fp32  every GEMM output with T rows, in turn; the
+//                              logits' rows are V4 = V rounded up to 4 apart
+//   dlog [T][Vp] bf16          Vp = V rounded up to 64: rows TMA can read for any V
+//   dx [T][d] fp32
 //   dxf  [L][T][d] bf16        each FFN output's gradient (bf16 of dx)
 //   dpre [L][T][h] bf16        each FFN pre-activation gradient
 //   dh [T][d] bf16; the LayerNorm backward's partial sums
@@ -548,9 +581,13 @@ struct BlockWs {
         sws_bytes, split, total;
 };
 
+int logit_ld(int V) { return (V + 3) & ~3; }
+int dlog_ld(int V) { return (V + 63) & ~63; }
+
 BlockWs block_ws(int B, int n, int d, int h, int V, int L) {
     const size_t T = (size_t)B * n;
-    const size_t wide = (size_t)(h > V ? (h > d ? h : d) : (V > d ? V : d));
+    const int zl = logit_ld(V);
+    const size_t wide = (size_t)(h > zl ? (h > d ? h : d) : (zl > d ? zl : d));
     BlockWs w;
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -568,7 +605,7 @@ BlockWs block_ws(int B, int n, int d, int h, int V, int L) {
     w.m = take(T * d * 2);
     w.hf = take(T * d * 2);
     w.U = take(T * wide * 4);
-    w.dlog = take(T * V * 2);
+    w.dlog = take(T * dlog_ld(V) * 2);
     w.dx = take(T * d * 4);
     // per layer: the FFN output's gradient (bf16) and the pre-activation
     // gradient, the operands of the batched FFN weight gradients after the loop
@@ -802,19 +839,25 @@ int block_step(const int* ids, const hcw_block_params& p, const hcw_block_grads&
                           top ? sf : S1(l + 1), T, d),
             1));
     }
-    HCW_GEMM(T, V, d, hf, false, p.Wh, true, U);
+    // V is any size: the logits and their gradient sit in rows padded to what TMA
+    // reads and writes, so that all three head products run on the tensor cores
+    // (dense rows of an odd V sent both gradient products to the plain kernel, 780 us
+    // each at V = 4769, T = 4096, d = 128, and the logits out one scalar store at a
+    // time: the step of 12 such layers took 2,589 us, with padded rows 935 us)
+    const int ldz = logit_ld(V), ldd = dlog_ld(V);
+    HCW_GEMM(T, V, d, hf, false, p.Wh, true, U, 0, ldz);
     HCW_TRY(count_launch(launch_pdl(ce_kernel, dim3(rows_grid), dim3(kRowWarps * 32), 0, st,
-                                    static_cast<const float*>(U), p.bh, ids, dlog, loss, B, n, V,
+                                    static_cast<const float*>(U), ldz, p.bh, ids, dlog, ldd, loss, B, n, V,
                                     1.f / T),
                          1));
 
     // ----------------------------------------------------------- backward
     const unsigned gridT = (unsigned)((T + kColRows - 1) / kColRows);
-    HCW_GEMM(V, d, T, dlog, true, hf, false, gr.Wh);   // dWh = dlog^T hf
-    HCW_TRY(count_launch(launch_pdl(colsum_kernel, dim3((V + 255) / 256, gridT), dim3(256), 0, st,
-                                    static_cast<const __nv_bfloat16*>(dlog), gr.bh, T, V),
+    HCW_GEMM(V, d, T, dlog, true, hf, false, gr.Wh, ldd);   // dWh = dlog^T hf
+    HCW_TRY(count_launch(launch_pdl(colsum_kernel, dim3((V + 511) / 512, gridT), dim3(256), 0, st,
+                                    static_cast<const __nv_bfloat16*>(dlog), ldd, gr.bh, T, V),
                          1));
-    HCW_GEMM(T, d, V, dlog, false, p.Wh, false, U);    // dhf = dlog Wh
+    HCW_GEMM(T, d, V, dlog, false, p.Wh, false, U, ldd);    // dhf = dlog Wh
     // each LayerNorm backward that writes the gradient of x_{l+1} (LNf, then
     // LN1 of layer l + 1) also sums its bf16 copy's columns: db2 of layer l
     int nk = 0;

@@ -30,8 +30,9 @@
 //
 // Every wait is bounded: a CTA that gives up records HCW_ERR_TIMEOUT in the
 // error word, lets its copies and MMAs in flight finish, frees TMEM and
-// returns.  Shapes TMA cannot read (a K-major row not a multiple of 16 bytes,
-// an MN-major one not a multiple of 64 elements) go to a plain tiled kernel.
+// returns.  Shapes TMA cannot read (a K-major row stride not a multiple of 16
+// bytes, an MN-major one not a multiple of 64 elements) go to a plain tiled
+// kernel.
 #include "hcw.h"
 #include "hcw_internal.h"
 #include "hcw_ptx.cuh"
@@ -83,6 +84,7 @@ struct GemmArgs {
     const __nv_bfloat16* aux;   // EPI_RELU_GRAD: [M][N]
     float* colsum;              // EPI_RELU_GRAD: [N] += column sums of the bf16 output, or null
     int M, N, K;
+    int ldc;                    // EPI_F32: elements from one row of C to the next
     int mt, nt;                 // tile counts (256-row tiles, 256-column tiles)
     int splits, kps;            // K splits and K steps per split
     // batched (both operands MN-major, EPI_F32): `splits` counts independent
@@ -445,7 +447,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                 if (row >= a.M || col0 >= a.N) continue;
                 const bool full = a.vec && col0 + 32 <= a.N;
                 if (EPI == EPI_F32) {
-                    float* dst = a.C + (size_t)s * a.M * a.N + (size_t)row * a.N + col0;
+                    float* dst = a.C + ((size_t)s * a.M + row) * a.ldc + col0;
                     if (full) {
 #pragma unroll
                         for (int m = 0; m < 8; ++m)
@@ -581,6 +583,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K,
     __shared__ float Bs[16][65];
     const int tm = blockIdx.y * 64, tn = blockIdx.x * 64;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int lda = e.lda ? e.lda : (ta ? M : K), ldc = e.ldc ? e.ldc : N;
     float acc[4][4] = {};
     for (int k0 = 0; k0 < K; k0 += 16) {
         for (int i = threadIdx.x; i < 16 * 64; i += 256) {
@@ -588,7 +591,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K,
             const int gm = tm + mm, gn = tn + mm, gk = k0 + kk;
             float av = 0.f, bv = 0.f;
             if (gm < M && gk < K)
-                av = __bfloat162float(ta ? A[(size_t)gk * M + gm] : A[(size_t)gm * K + gk]);
+                av = __bfloat162float(ta ? A[(size_t)gk * lda + gm] : A[(size_t)gm * lda + gk]);
             if (gn < N && gk < K)
                 bv = __bfloat162float(tb ? B[(size_t)gn * K + gk] : B[(size_t)gk * N + gn]);
             As[kk][mm] = av;
@@ -611,7 +614,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K,
             if (gm >= M || gn >= N) continue;
             const size_t o = (size_t)gm * N + gn;
             if (e.kind == EPI_F32) {
-                C[o] = acc[i][j];
+                C[(size_t)gm * ldc + gn] = acc[i][j];
             } else if (e.kind == EPI_BIAS_RELU) {
                 const float x = acc[i][j] + e.bias[gn];
                 e.out[o] = __float2bfloat16_rn(x > 0.f ? x : 0.f);
@@ -641,12 +644,13 @@ GemmEncodeFn gemm_encode_fn() {
     return fn;
 }
 
-// A K-major operand [rows][K] bf16 as 64-element rows: box (64, box_rows).
-bool map_kmajor(CUtensorMap* m, const void* base, int rows, int K, int box_rows) {
+// A K-major operand [rows][K] bf16, ld elements from row to row, as 64-element
+// rows: box (64, box_rows).
+bool map_kmajor(CUtensorMap* m, const void* base, int rows, int K, int ld, int box_rows) {
     GemmEncodeFn enc = gemm_encode_fn();
     if (!enc) return false;
     cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)K * 2};
+    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
     cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
@@ -654,14 +658,14 @@ bool map_kmajor(CUtensorMap* m, const void* base, int rows, int K, int box_rows)
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// An MN-major operand, the row-major [K][cols] matrix, as (64 columns, K rows,
-// cols / 64 blocks): box (64, 64, nblk) lands nblk blocks of 64 rows x 64
-// columns one after the other.
-bool map_mnmajor(CUtensorMap* m, const void* base, int K, int cols, int nblk) {
+// An MN-major operand, the row-major [K][cols] matrix with ld elements from row
+// to row (ld holds whole 64-column blocks), as (64 columns, K rows, blocks): box
+// (64, 64, nblk) lands nblk blocks of 64 rows x 64 columns one after the other.
+bool map_mnmajor(CUtensorMap* m, const void* base, int K, int cols, int ld, int nblk) {
     GemmEncodeFn enc = gemm_encode_fn();
     if (!enc) return false;
-    cuuint64_t dims[3] = {64, (cuuint64_t)K, (cuuint64_t)(cols / 64)};
-    cuuint64_t strides[2] = {(cuuint64_t)cols * 2, 128};
+    cuuint64_t dims[3] = {64, (cuuint64_t)K, (cuuint64_t)((cols + 63) / 64)};
+    cuuint64_t strides[2] = {(cuuint64_t)ld * 2, 128};
     cuuint32_t box[3] = {64, 64, (cuuint32_t)nblk};
     cuuint32_t estr[3] = {1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
@@ -685,13 +689,13 @@ bool map_mnmajor_batched(CUtensorMap* m, const void* base, int K, int cols, int 
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// fp32 output [splits][M][N] as (N, M, splits), box (32, 32, 1): 32 x 32
-// patches clipped at each split's M rows; 128-byte swizzle.
-bool map_out_f32(CUtensorMap* m, void* base, int M, int N, int splits) {
+// fp32 output [splits][M][ld], N columns of each row, as (N, M, splits), box
+// (32, 32, 1): 32 x 32 patches clipped at each split's M rows; 128-byte swizzle.
+bool map_out_f32(CUtensorMap* m, void* base, int M, int N, int ld, int splits) {
     GemmEncodeFn enc = gemm_encode_fn();
-    if (!enc || (reinterpret_cast<uintptr_t>(base) & 15) || N % 4) return false;
+    if (!enc || (reinterpret_cast<uintptr_t>(base) & 15) || ld % 4) return false;
     cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)M, (cuuint64_t)splits};
-    cuuint64_t strides[2] = {(cuuint64_t)N * 4, (cuuint64_t)M * N * 4};
+    cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)M * ld * 4};
     cuuint32_t box[3] = {32, 32, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
@@ -821,11 +825,14 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
     }
     if (bad) return cudaErrorInvalidValue;
     const bool a_mn = ta, b_mn = !tb;
+    const int lda = epi.lda ? epi.lda : (a_mn ? M : K), ldb = b_mn ? N : K;
+    const int ldc = epi.ldc ? epi.ldc : N;
     const auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
     // what TMA can read: 16-byte row strides, MN-major operands in whole
-    // 64-column blocks
-    const bool tc = aligned(A) && aligned(B) && (a_mn ? M % 64 == 0 : K % 8 == 0) &&
-                    (b_mn ? N % 64 == 0 : K % 8 == 0) && epi_has_kernel(a_mn, b_mn, epi.kind) &&
+    // 64-column blocks (a padded row may end past the operand's last column:
+    // the columns past it reach only output rows that are not stored)
+    const bool tc = aligned(A) && aligned(B) && (a_mn ? lda % 64 == 0 : lda % 8 == 0) &&
+                    (b_mn ? ldb % 64 == 0 : ldb % 8 == 0) && epi_has_kernel(a_mn, b_mn, epi.kind) &&
                     gemm_encode_fn() != nullptr;
     if (!tc) {
         dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
@@ -837,12 +844,13 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
     }
     // boxes no larger than the operand (the rows / blocks a smaller box leaves
     // in shared memory only reach output rows and columns that are not stored)
-    const int a_box = a_mn ? (M / 64 < kGM / 64 ? M / 64 : kGM / 64) : (M < kGM ? M : kGM);
+    const int a_blk = (M + 63) / 64;
+    const int a_box = a_mn ? (a_blk < kGM / 64 ? a_blk : kGM / 64) : (M < kGM ? M : kGM);
     const int b_box = b_mn ? (N / 64 < kGN / 128 ? N / 64 : kGN / 128) : (N < kGN / 2 ? N : kGN / 2);
     GemmArgs a;
     memset(&a, 0, sizeof(a));
-    if (!(a_mn ? map_mnmajor(&a.mA, A, K, M, a_box) : map_kmajor(&a.mA, A, M, K, a_box)) ||
-        !(b_mn ? map_mnmajor(&a.mB, B, K, N, b_box) : map_kmajor(&a.mB, B, N, K, b_box)))
+    if (!(a_mn ? map_mnmajor(&a.mA, A, K, M, lda, a_box) : map_kmajor(&a.mA, A, M, K, lda, a_box)) ||
+        !(b_mn ? map_mnmajor(&a.mB, B, K, N, ldb, b_box) : map_kmajor(&a.mB, B, N, K, ldb, b_box)))
         return cudaErrorInvalidValue;
     a.stage_tx = (uint32_t)(kGK * 2) * (uint32_t)((a_mn ? 64 * a_box : a_box) +
                                                   (b_mn ? 64 * b_box : b_box));
@@ -854,13 +862,14 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
     const int nkb = (K + kGK - 1) / kGK;
     const int sms = gemm_sms();
     const int splits =
-        split_ws && epi.kind == EPI_F32 ? choose_splits(M, N, K, sms, split_ws_bytes) : 1;
+        split_ws && epi.kind == EPI_F32 && ldc == N ? choose_splits(M, N, K, sms, split_ws_bytes) : 1;
     a.kps = (nkb + splits - 1) / splits;
     a.splits = (nkb + a.kps - 1) / a.kps;   // no empty split
     if (epi.kind == EPI_F32) {
         a.C = a.splits > 1 ? split_ws : C;
-        a.vec = (N % 4 == 0) && aligned(a.C);
-        a.tma_out = map_out_f32(&a.mOut, a.C, M, N, a.splits);
+        a.ldc = ldc;
+        a.vec = (ldc % 4 == 0) && aligned(a.C);
+        a.tma_out = map_out_f32(&a.mOut, a.C, M, N, ldc, a.splits);
     } else {
         a.out = epi.out;
         a.bias = epi.bias;
@@ -940,8 +949,9 @@ cudaError_t gemm_bf16_f32_batched(int M, int N, int K, const void* A, size_t a_b
     a.splits = batch;
     a.kps = (K + kGK - 1) / kGK;
     a.C = C;
+    a.ldc = N;
     a.vec = N % 4 == 0;
-    a.tma_out = map_out_f32(&a.mOut, C, M, N, batch);
+    a.tma_out = map_out_f32(&a.mOut, C, M, N, N, batch);
     a.timeout_ns = kGemmTimeoutNs;
     const int sms = gemm_sms();
     const int units = a.mt * a.nt * batch;

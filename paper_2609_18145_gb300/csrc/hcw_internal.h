@@ -287,7 +287,8 @@ cudaError_t gemm_bf16_f32_batched(int M, int N, int K, const void* A, size_t a_b
                                   cudaStream_t st, int* launches);
 // Epilogues of the GEMM: fp32 C; out = bf16(relu(C + bias[col])); or
 // out = bf16(aux[row][col] > 0 ? C : 0), with colsum[col] (if given) += the
-// column sums of out.  out and aux are [M][N] bf16.
+// column sums of out.  out and aux are [M][N] bf16.  lda / ldc: elements from
+// one row of A (as stored) / C to the next; 0 = dense rows.
 enum GemmEpiKind { EPI_F32 = 0, EPI_BIAS_RELU = 1, EPI_RELU_GRAD = 2 };
 struct GemmEpi {
     int kind;
@@ -295,6 +296,8 @@ struct GemmEpi {
     const __nv_bfloat16* aux;
     __nv_bfloat16* out;
     float* colsum;
+    int lda = 0;
+    int ldc = 0;
 };
 // gemm_bf16_f32 with an epilogue (C unused unless epi.kind is EPI_F32; only
 // fp32 output splits K).

@@ -93,6 +93,7 @@ def check_grads_elementwise(got, ref):
 CASES = [
     # B, n, d, h, V, L
     (2, 16, 64, 128, 11, 3),
+    (3, 16, 128, 256, 389, 2),    # logit rows past whole tiles and whole fours
     (3, 32, 128, 256, 256, 4),
     (1, 64, 192, 136, 37, 2),
 ]
