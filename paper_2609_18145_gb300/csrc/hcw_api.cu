@@ -435,7 +435,11 @@ int fwd_bf16(const Shape& sh, const void* x, const void* Ws, const void* Wn, con
     TcLaunch<1> L;
     memset(&L, 0, sizeof(L));
     if (!fwd_maps(L.maps[0], sh, sh.s, x, Ws, Wn, y)) return HCW_ERR_CUDA;
-    if (xpair && !map_rows(&L.maps[0][5], xpair, sh.tokens, sh.d, 1 << sh.s, 128))
+    // map 5: the row-aligned partner tensor, or the patches of z (never both: the
+    // layer API has no shift layers)
+    if (xpair && (z || !map_rows(&L.maps[0][5], xpair, sh.tokens, sh.d, 1 << sh.s, 128)))
+        return HCW_ERR_CUDA;
+    if (z && !map_rows(&L.maps[0][5], z, sh.tokens, sh.d, 1 << sh.s, 32, epi_patch_cols(BN)))
         return HCW_ERR_CUDA;
     L.layer[0] = {sh.s, 1 << sh.s, bias, mask, static_cast<__nv_bfloat16*>(z), true, nullptr, false};
     L.layer[0].pair_rows = xpair != nullptr;
@@ -591,8 +595,12 @@ int dx_bf16(const Shape& sh, const void* dz, const void* dy, const void* Ws, con
     return launched(launch_tc(MODE_DX, BN, L, grid, st), 1);
 }
 
-// dW: token-contracted, split over token blocks, fixed-order reduction; dbias
-// by a deterministic two-pass column sum.  wws: weight workspace.
+// dW: token-contracted, split over token blocks, fixed-order reduction.  dbias:
+// the self part's units sum dz's columns on the way (their helper warps), per split,
+// and the reduction adds the splits with the weights' (two launches fewer than a
+// column sum of its own, 7.7 us at 16,384 tokens of d = 512); the partials take the
+// column sum's scratch, which holds a row per 64 tokens (256 above 65,536), and a
+// split has at least 256.  wws: weight workspace.
 int dw_bf16(const Shape& sh, const void* x, const void* dz, unsigned flags, float* dWs,
             float* dWn, float* dbias, uint8_t* wws, cudaStream_t st) {
     const int d = sh.d, BN = pick_bn(d), k = 1 << sh.s;
@@ -610,6 +618,10 @@ int dw_bf16(const Shape& sh, const void* x, const void* dz, unsigned flags, floa
         return HCW_ERR_CUDA;
     maps[2] = maps[1];   // unused by the weight gradient
     L.layer[0] = {sh.s, k, nullptr, nullptr, nullptr, false, nullptr, false};
+    float* bpart = reinterpret_cast<float*>(wws + lay.col_off);
+    const bool fused_bias =
+        dbias && (w.splits_self == 1 || (size_t)w.splits_self * d * 4 <= lay.col_bytes);
+    if (fused_bias) L.layer[0].colsum = w.splits_self == 1 ? dbias : bpart;
     TcParams& p = L.p;
     p.d = d;
     p.Mh = (int)(sh.tokens / 2);
@@ -632,11 +644,13 @@ int dw_bf16(const Shape& sh, const void* x, const void* dz, unsigned flags, floa
     if (rc) return rc;
     if (w.splits_max > 1) {
         rc = launched(launch_splitk_reduce(part, w.splits_max, w.splits_self,
-                                           w.splits_nbr, d, dWs, dWn, st),
+                                           w.splits_nbr, d, dWs, dWn, st, 1, 0, 0,
+                                           fused_bias ? bpart : nullptr,
+                                           fused_bias ? dbias : nullptr),
                       1);
         if (rc) return rc;
     }
-    if (dbias)
+    if (dbias && !fused_bias)
         return launched(launch_colsum_bf16(static_cast<const __nv_bfloat16*>(dz), sh.tokens, d,
                                            reinterpret_cast<float*>(wws + lay.col_off), dbias,
                                            st),

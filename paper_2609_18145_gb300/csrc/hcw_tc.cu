@@ -1292,31 +1292,6 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                 if (!wait_acc()) {
                     return false;
                 }
-                // FWD z (layer API only): the pre-activation, row-wise stores; every
-                // lane joins the warp-wide TMEM loads, rows past the end skip the store
-                if (fwd && ly.zout) {
-#pragma unroll 1
-                    for (int h = 0; h < SUB; ++h) {
-                        uint32_t raw[32];
-                        load_acc(h * 32, raw);
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            uint32_t w[4];
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                const int e2 = 8 * m + 2 * i;
-                                w[i] = pack_bf16x2(
-                                    __uint_as_float(raw[e2]) +
-                                        __shfl_sync(0xffffffffu, bias_reg[h], e2),
-                                    __uint_as_float(raw[e2 + 1]) +
-                                        __shfl_sync(0xffffffffu, bias_reg[h], e2 + 1));
-                            }
-                            if (tok_row >= 0)
-                                reinterpret_cast<uint4*>(ly.zout + (size_t)tok_row * p.d + col0 +
-                                                         h * 32)[m] = make_uint4(w[0], w[1], w[2], w[3]);
-                        }
-                    }
-                }
                 if (has_res) {
                     const bool okl = wait_bar(&bars->epi_load[e], ld_phase);
                     ld_phase ^= 1;
@@ -1331,13 +1306,14 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                                      : "memory");
                 }
                 const bool write_out = fwd || ly.out;
+                const bool want_z = fwd && !STACKED && ly.zout != nullptr;
                 uint32_t gw[SUB][16];
                 uint32_t mbits[SUB];
 #pragma unroll
                 for (int h = 0; h < SUB; ++h) {
                     uint32_t raw[32];
                     load_acc(h * 32, raw);
-                    if (h == SUB - 1) release_acc();
+                    if (h == SUB - 1 && !want_z) release_acc();
                     // The arithmetic runs on the FP32 pipe, two columns per instruction
                     // where it can (f32x2): the epilogue of a chained unit sits on the
                     // layer chain, and half-rate integer work (compares, selects, bit
@@ -1527,6 +1503,40 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                         }
                     }
                     if (signal) count(L.counters, 0);
+                }
+                // FWD z (layer API only): the pre-activation, from the accumulator
+                // again (held until now) through the same patch buffer once the y store
+                // has read it: whole rows by TMA.  Row pieces stored from registers took
+                // 24 us of a 16,384-token layer at d = 512, this 20.
+                if (want_z) {
+                    if (lane == 0) bulk_wait_read<0>();
+                    __syncwarp();
+#pragma unroll 1
+                    for (int h = 0; h < SUB; ++h) {
+                        uint32_t raw[32];
+                        load_acc(h * 32, raw);
+                        if (h == SUB - 1) release_acc();
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const int e2 = 8 * m + 2 * i;
+                                w[i] = pack_bf16x2(
+                                    __uint_as_float(raw[e2]) +
+                                        __shfl_sync(0xffffffffu, bias_reg[h], e2),
+                                    __uint_as_float(raw[e2 + 1]) +
+                                        __shfl_sync(0xffffffffu, bias_reg[h], e2 + 1));
+                            }
+                            *patch_piece<RB>(buf, lane, 4 * h + m) =
+                                make_uint4(w[0], w[1], w[2], w[3]);
+                        }
+                    }
+                    publish();
+                    if (lane == 0 && inside) {
+                        tma_store_4d(mE2, buf, col0, lo_w, r.beta, hi_w);
+                        bulk_commit();
+                    }
                 }
                 // FWD: the ReLU mask words, read only by the input gradient (a later
                 // launch), after the signal so that they stay off the layer chain
