@@ -352,6 +352,21 @@ struct WsLayout {
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
+// Partial sums of the fp32 weight gradients of `layers` layers (dw_f32).
+size_t f32_part_bytes(long long tokens, int d, int layers) {
+    size_t most = 0;
+    // launches of kMaxF32Layers layers and the last, shorter one
+    const int counts[2] = {layers < kMaxF32Layers ? layers : kMaxF32Layers,
+                           layers % kMaxF32Layers};
+    for (int cnt : counts) {
+        if (cnt == 0) continue;
+        const int s = f32_dw_splits(tokens, d, cnt, sm_count());
+        const size_t b = s > 1 ? (size_t)cnt * s * (2 * (size_t)d * d + d) * 4 : 0;
+        if (b > most) most = b;
+    }
+    return align256(most);
+}
+
 WsLayout ws_layout(long long tokens, int d, int dtype, unsigned flags) {
     WsLayout l;
     const size_t es = elem_size(dtype);
@@ -366,6 +381,12 @@ WsLayout ws_layout(long long tokens, int d, int dtype, unsigned flags) {
     }
     l.col_off = l.part_bytes;   // relative to w_off
     l.col_bytes = align256(colsum_workspace_bytes(tokens, d));
+    // fp32: the split's partial sums, or the column sums' size where that is larger
+    // (what callers without an allocator were promised to fit stays so)
+    if (dtype != HCW_BF16) {
+        const size_t part = f32_part_bytes(tokens, d, 1);
+        if (part > l.col_bytes) l.col_bytes = part;
+    }
     l.w_bytes = l.part_bytes + l.col_bytes;
     l.total = l.w_off + l.w_bytes;
     return l;
@@ -712,23 +733,45 @@ int fwd_f32(const Shape& sh, const void* x, const void* Ws, const void* Wn, cons
 }
 
 int dx_f32(const Shape& sh, const void* dz, const void* dy, const void* Ws, const void* Wn,
-           unsigned flags, void* dx, cudaStream_t st) {
+           unsigned flags, void* dx, cudaStream_t st, const uint32_t* mprev = nullptr,
+           void* dz_prev = nullptr) {
     return launched(launch_f32_dx(static_cast<const float*>(dz), static_cast<const float*>(dy),
                                   static_cast<const float*>(Ws), static_cast<const float*>(Wn),
-                                  sh.s, sh.B, sh.n, sh.d, flags, static_cast<float*>(dx), st),
+                                  sh.s, sh.B, sh.n, sh.d, flags, static_cast<float*>(dx), mprev,
+                                  static_cast<float*>(dz_prev), st),
                     1);
 }
 
-int dw_f32(const Shape& sh, const void* x, const void* dz, unsigned flags, float* dWs,
-           float* dWn, float* dbias, uint8_t* wws, cudaStream_t st) {
-    const WsLayout lay = ws_layout(sh.tokens, sh.d, HCW_F32, flags);
-    int rc = launched(launch_f32_dw(static_cast<const float*>(x), static_cast<const float*>(dz),
-                                    sh.s, sh.B, sh.n, sh.d, flags, dWs, dWn, st),
-                      1);
-    if (rc || !dbias) return rc;
-    return launched(launch_colsum_f32(static_cast<const float*>(dz), sh.tokens, sh.d,
-                                      reinterpret_cast<float*>(wws + lay.col_off), dbias, st),
-                    2);
+// fp32 weight gradients of L layers with links link(l) at once.  wws: scratch of
+// f32_part_bytes.
+template <class Link>
+int dw_f32(const Shape& sh, int L, Link link, const void* x, const void* acts, const void* dz,
+           unsigned flags, float* dWs, float* dWn, float* dbias, uint8_t* wws, cudaStream_t st) {
+    const size_t dd = (size_t)sh.d * sh.d;
+    for (int l0 = 0; l0 < L; l0 += kMaxF32Layers) {
+        const int cnt = L - l0 < kMaxF32Layers ? L - l0 : kMaxF32Layers;
+        F32DwArgs a;
+        a.act_elems = sh.tokens * sh.d;
+        a.rows = sh.tokens;
+        const float* in = static_cast<const float*>(acts);
+        a.x = l0 == 0 ? static_cast<const float*>(x) : in + (l0 - 1) * a.act_elems;
+        a.acts = in ? in + l0 * a.act_elems : nullptr;
+        a.dz = static_cast<const float*>(dz) + l0 * a.act_elems;
+        a.dWs = dWs + l0 * dd;
+        a.dWn = dWn + l0 * dd;
+        a.dbias = dbias ? dbias + (size_t)l0 * sh.d : nullptr;
+        a.part = reinterpret_cast<float*>(wws);
+        for (int i = 0; i < cnt; ++i) a.s[i] = link(l0 + i);
+        a.n = sh.n;
+        a.d = sh.d;
+        a.flags = flags;
+        int nk = 0;
+        const cudaError_t e =
+            launch_f32_dw(a, cnt, f32_dw_splits(sh.tokens, sh.d, cnt, sm_count()), st, &nk);
+        const int rc = launched(e, nk);
+        if (rc) return rc;
+    }
+    return HCW_OK;
 }
 
 int layer_fwd_impl(const Shape& sh, int dtype, const void* x, const void* Ws, const void* Wn,
@@ -759,7 +802,8 @@ int layer_dw_impl(const Shape& sh, int dtype, const void* x, const void* dz, uns
                   float* dWs, float* dWn, float* dbias, uint8_t* wws, cudaStream_t st) {
     if (sh.tokens == 0) return zero_weight_grads(sh, dWs, dWn, dbias, st);
     return dtype == HCW_BF16 ? dw_bf16(sh, x, dz, flags, dWs, dWn, dbias, wws, st)
-                             : dw_f32(sh, x, dz, flags, dWs, dWn, dbias, wws, st);
+                             : dw_f32(sh, 1, [&](int) { return sh.s; }, x, nullptr, dz, flags, dWs, dWn,
+                                      dbias, wws, st);
 }
 
 int layer_bwd_impl(const Shape& sh, int dtype, const void* x, const void* z, const void* dy,
@@ -845,7 +889,10 @@ size_t split_dw_ws(const Shape& sh, unsigned flags, int cnt) {
 // partials] when that is larger
 size_t stack_weight_ws(const Shape& sh, int dtype, unsigned flags, int L) {
     const WsLayout w = ws_layout(sh.tokens, sh.d, dtype, flags);
-    if (dtype != HCW_BF16) return w.w_bytes;
+    if (dtype != HCW_BF16) {
+        const size_t part = f32_part_bytes(sh.tokens, sh.d, L);
+        return part > w.w_bytes ? part : w.w_bytes;
+    }
     size_t body = align256(w.w_bytes) + align256(sh.act_bytes);
     // the launches of kMaxStackLayers layers and the last, shorter one
     const int counts[2] = {L < kMaxStackLayers ? L : kMaxStackLayers, L % kMaxStackLayers};
@@ -1344,41 +1391,28 @@ int stack_data_f32(const Shape& sh, const StackData& a, cudaStream_t st) {
         rc = cuda_status(cudaMemcpyAsync(dz(L - 1), a.dy, ab, cudaMemcpyDeviceToDevice, st));
     }
     if (rc) return rc;
+    // a layer's launch also writes the dz of the layer below: with the ReLU through
+    // its mask (and the unmasked g only where the residual needs it), else dz is g
     const void* cur_g = a.dy;
     for (int l = L - 1; l >= 0; --l) {
+        const bool below = relu && l > 0;
+        void* out = l == 0 ? a.dx
+                           : (!relu ? dz(l - 1)
+                                    : ((a.flags & HCW_RESIDUAL) ? (void*)g[l & 1] : nullptr));
         Shape shl = sh;
         shl.s = a.sc.dim(sh, l);
-        void* out = l == 0 ? a.dx : (relu ? (void*)g[l & 1] : dz(l - 1));
-        rc = layer_dx_impl(shl, HCW_F32, dz(l), cur_g, a.Ws + l * wb, a.Wn + l * wb, a.flags, out,
-                           st);
+        rc = dx_f32(shl, dz(l), cur_g, a.Ws + l * wb, a.Wn + l * wb, a.flags, out, st,
+                    below ? mask(l - 1) : nullptr, below ? dz(l - 1) : nullptr);
         if (rc) return rc;
-        if (l == 0) break;
-        if (relu) {
-            rc = launched(launch_relu_grad_mask_f32(static_cast<const float*>(out), mask(l - 1),
-                                                    static_cast<float*>(dz(l - 1)), sh.tokens, d,
-                                                    st),
-                          1);
-            if (rc) return rc;
-        }
         cur_g = out;
     }
     return HCW_OK;
 }
 
-// fp32 weight gradients, layer by layer.
+// fp32 weight gradients, all layers at once.
 int stack_weight_f32(const Shape& sh, const StackWeight& a, cudaStream_t st) {
-    const int d = sh.d;
-    const size_t ab = sh.act_bytes;
-    for (int l = 0; l < a.L; ++l) {
-        Shape shl = sh;
-        shl.s = a.sc.dim(sh, l);
-        const void* in = l == 0 ? a.x : static_cast<const uint8_t*>(a.acts) + (size_t)(l - 1) * ab;
-        const int rc = layer_dw_impl(shl, HCW_F32, in, a.dz + (size_t)l * ab, a.flags,
-                                     a.dWs + (size_t)l * d * d, a.dWn + (size_t)l * d * d,
-                                     a.dbias ? a.dbias + (size_t)l * d : nullptr, a.ws, st);
-        if (rc) return rc;
-    }
-    return HCW_OK;
+    return dw_f32(sh, a.L, [&](int l) { return a.sc.dim(sh, l); }, a.x, a.acts, a.dz, a.flags,
+                  a.dWs, a.dWn, a.dbias, a.ws, st);
 }
 
 // Argument checks of the two halves (sizes, pointers, alignment, overlaps).

@@ -250,9 +250,19 @@ cudaError_t launch_decode(const DecodeLaunch& p, cudaStream_t st);
 // Read the decode kernel's error word and reset it to 0 (synchronous).
 cudaError_t decode_error_word_read_clear(int* word);
 
+// Programmatic dependent launch (a launch with the programmatic stream
+// serialization attribute may start before the kernel before it in the stream
+// has finished): pdl_wait blocks until that kernel has completed and its
+// memory is visible -- a no-op in a launch without the attribute -- and
+// pdl_trigger lets the next such launch begin its prologue.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Launch `kern` with programmatic stream serialization: it may start while the
 // kernel before it in the stream finishes, and must call pdl_wait()
-// (hcw_ptx.cuh) before it touches memory that kernel reads or writes.
+// before it touches memory that kernel reads or writes.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t st, Args... args) {
@@ -330,9 +340,27 @@ cudaError_t launch_relu_grad_mask_bf16(const __nv_bfloat16* dy, const uint32_t* 
                                        cudaStream_t st);
 cudaError_t launch_f32_dx(const float* dz, const float* dy, const float* Ws, const float* Wn,
                           int s, int B, int n, int d, unsigned flags, float* dx,
-                          cudaStream_t st);
-cudaError_t launch_f32_dw(const float* x, const float* dz, int s, int B, int n, int d,
-                          unsigned flags, float* dWs, float* dWn, cudaStream_t st);
+                          const uint32_t* mprev, float* dz_prev, cudaStream_t st);
+// The fp32 weight and bias gradients of up to kMaxF32Layers layers (layer l's input
+// is x for l = 0, acts[l - 1] above, activations act_elems apart): one launch, and
+// one that adds the splits' partial sums `part` (splits (2 d d + d) floats a layer)
+// when there are several.
+constexpr int kMaxF32Layers = 64;
+struct F32DwArgs {
+    const float* x;
+    const float* acts;
+    const float* dz;
+    long long act_elems, rows, rows_per_split;
+    float* dWs;
+    float* dWn;
+    float* dbias;   // or null
+    float* part;
+    int s[kMaxF32Layers];   // links, as for the other fp32 kernels
+    int n, d, splits;
+    unsigned flags;
+};
+int f32_dw_splits(long long rows, int d, int layers, int sms);
+cudaError_t launch_f32_dw(F32DwArgs& a, int layers, int splits, cudaStream_t st, int* launches);
 // dz = dy * (z > 0), elementwise over count elements (T = float or bf16)
 cudaError_t launch_relu_grad_f32(const float* dy, const float* z, float* dz, size_t count,
                                  cudaStream_t st);
@@ -340,8 +368,6 @@ cudaError_t launch_relu_grad_bf16(const __nv_bfloat16* dy, const __nv_bfloat16* 
                                   __nv_bfloat16* dz, size_t count, cudaStream_t st);
 // dbias[o] = sum_t dz[t][o], deterministic two-pass column sum.
 size_t colsum_workspace_bytes(long long rows, int d);
-cudaError_t launch_colsum_f32(const float* dz, long long rows, int d, float* partial,
-                              float* out, cudaStream_t st);
 cudaError_t launch_colsum_bf16(const __nv_bfloat16* dz, long long rows, int d, float* partial,
                                float* out, cudaStream_t st);
 // The same for `batch` consecutive [rows][d] matrices: out [batch][d], partial

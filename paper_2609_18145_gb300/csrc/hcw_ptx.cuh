@@ -25,16 +25,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// Programmatic dependent launch (a launch with the programmatic stream
-// serialization attribute may start before the kernel before it in the stream
-// has finished): pdl_wait blocks until that kernel has completed and its
-// memory is visible -- a no-op in a launch without the attribute -- and
-// pdl_trigger lets the next such launch begin its prologue.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

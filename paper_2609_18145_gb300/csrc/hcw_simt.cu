@@ -32,36 +32,63 @@ __device__ __forceinline__ int reader_of(int i, int s, int n, unsigned flags) {
 
 constexpr int T = 32;   // tile edge of the fp32 kernels
 
+// The fp32 kernels: 32 x 32 output tiles, 32 x 8 threads, 4 outputs per thread,
+// the contraction in steps of 32 through shared memory, the next step's operands
+// loaded into registers while one is computed.  Their users' sizes are small
+// (checks and first experiments, d in the tens): they are bound by launches and by
+// the latency of a step, so every launch is a programmatic dependent of the one
+// before it, the input gradient writes the layer below's dz itself, and one launch
+// computes the weight and bias gradients of a whole stack (four layers forward and
+// backward at 64 rows of d = 32: 24 launches, 127 us, now 10, 48 us; seven layers
+// at 3,968 rows of d = 91, whose gradient blocks each walked all rows: 2,493 us,
+// now 402).
+
 // z[r][o] = sum_k Ws[o][k] x[r][k] + m_r sum_k Wn[o][k] x[p(r)][k] + bias[o]
-// Block: 32 rows x 32 outputs, 32 x 8 threads, 4 outputs per thread.
 // mout (optional): ReLU mask words [rows][ceil(d/32)], bit o%32 of word o/32 = (z > 0).
-__global__ void f32_fwd_kernel(const float* __restrict__ x, const float* __restrict__ Ws,
-                               const float* __restrict__ Wn, const float* __restrict__ bias,
-                               int s, int n, int d, long long rows, unsigned flags,
-                               float* __restrict__ y, float* __restrict__ z,
-                               uint32_t* __restrict__ mout) {
+__global__ void __launch_bounds__(256)
+    f32_fwd_kernel(const float* __restrict__ x, const float* __restrict__ Ws,
+                   const float* __restrict__ Wn, const float* __restrict__ bias, int s, int n,
+                   int d, long long rows, unsigned flags, float* __restrict__ y,
+                   float* __restrict__ z, uint32_t* __restrict__ mout) {
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
     __shared__ float xs[T][T + 1], xp[T][T + 1], ws[T][T + 1], wn[T][T + 1];
     const long long r0 = (long long)blockIdx.y * T;
     const int o0 = blockIdx.x * T;
     const int tx = threadIdx.x, ty = threadIdx.y;
+    // this thread's rows ty, ty + 8, ... of the tile: row, partner row (or null)
+    const float *xr[4], *pr[4], *wsr[4], *wnr[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const long long r = r0 + ty + 8 * q;
+        const int i = (int)(r & (n - 1)), o = o0 + ty + 8 * q;
+        xr[q] = r < rows ? x + r * d : nullptr;
+        pr[q] = r < rows && receives(i, s, flags) ? x + (r - i + partner_of(i, s)) * d : nullptr;
+        wsr[q] = o < d ? Ws + (long long)o * d : nullptr;
+        wnr[q] = o < d ? Wn + (long long)o * d : nullptr;
+    }
+    float a[4], b[4], u[4], v4[4];
+    auto load = [&](int k) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            a[q] = xr[q] && k < d ? xr[q][k] : 0.f;
+            b[q] = pr[q] && k < d ? pr[q][k] : 0.f;
+            u[q] = wsr[q] && k < d ? wsr[q][k] : 0.f;
+            v4[q] = wnr[q] && k < d ? wnr[q][k] : 0.f;
+        }
+    };
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    load(tx);
     for (int k0 = 0; k0 < d; k0 += T) {
-        for (int rr = ty; rr < T; rr += 8) {
-            const long long r = r0 + rr;
-            const int k = k0 + tx;
-            float a = 0.f, b = 0.f;
-            if (r < rows && k < d) {
-                const int i = (int)(r % n);
-                a = x[r * d + k];
-                b = receives(i, s, flags) ? x[(r - i + partner_of(i, s)) * d + k] : 0.f;
-            }
-            xs[rr][tx] = a;
-            xp[rr][tx] = b;
-            const int o = o0 + rr;
-            ws[rr][tx] = (o < d && k < d) ? Ws[(long long)o * d + k] : 0.f;
-            wn[rr][tx] = (o < d && k < d) ? Wn[(long long)o * d + k] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            xs[ty + 8 * q][tx] = a[q];
+            xp[ty + 8 * q][tx] = b[q];
+            ws[ty + 8 * q][tx] = u[q];
+            wn[ty + 8 * q][tx] = v4[q];
         }
         __syncthreads();
+        if (k0 + T < d) load(k0 + T + tx);
 #pragma unroll 8
         for (int kk = 0; kk < T; ++kk) {
 #pragma unroll
@@ -93,34 +120,55 @@ __global__ void f32_fwd_kernel(const float* __restrict__ x, const float* __restr
     }
 }
 
-// dx[r][k] = sum_o dz[r][o] Ws[o][k] + m_{p(r)} sum_o dz[p(r)][o] Wn[o][k] (+ dy[r][k])
-__global__ void f32_dx_kernel(const float* __restrict__ dz, const float* __restrict__ dy,
-                              const float* __restrict__ Ws, const float* __restrict__ Wn, int s,
-                              int n, int d, long long rows, unsigned flags,
-                              float* __restrict__ dx) {
+// dx[r][k] = sum_o dz[r][o] Ws[o][k] + m_{p(r)} sum_o dz[p(r)][o] Wn[o][k] (+ dy[r][k]),
+// written to dx (if given) and, where the mask bits mprev of the layer below are set
+// (else 0), to dz_prev (if given).
+__global__ void __launch_bounds__(256)
+    f32_dx_kernel(const float* __restrict__ dz, const float* __restrict__ dy,
+                  const float* __restrict__ Ws, const float* __restrict__ Wn, int s, int n, int d,
+                  long long rows, unsigned flags, float* __restrict__ dx,
+                  const uint32_t* __restrict__ mprev, float* __restrict__ dz_prev) {
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
     __shared__ float gs[T][T + 1], gp[T][T + 1], ws[T][T + 1], wn[T][T + 1];
     const long long r0 = (long long)blockIdx.y * T;
     const int k0 = blockIdx.x * T;
     const int tx = threadIdx.x, ty = threadIdx.y;
+    const int k = k0 + tx;
+    const float *gr[4], *pr[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const long long r = r0 + ty + 8 * q;
+        const int i = (int)(r & (n - 1));
+        const int j = reader_of(i, s, n, flags);
+        gr[q] = r < rows ? dz + r * d : nullptr;
+        pr[q] = r < rows && j >= 0 ? dz + (r - i + j) * d : nullptr;
+    }
+    float a[4], b[4], u[4], v4[4];
+    auto load = [&](int o0) {
+        const int o = o0 + tx;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int oo = o0 + ty + 8 * q;
+            const bool w = oo < d && k < d;
+            a[q] = gr[q] && o < d ? gr[q][o] : 0.f;
+            b[q] = pr[q] && o < d ? pr[q][o] : 0.f;
+            u[q] = w ? Ws[(long long)oo * d + k] : 0.f;
+            v4[q] = w ? Wn[(long long)oo * d + k] : 0.f;
+        }
+    };
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    load(0);
     for (int o0 = 0; o0 < d; o0 += T) {
-        for (int rr = ty; rr < T; rr += 8) {
-            const long long r = r0 + rr;
-            const int o = o0 + tx;
-            float a = 0.f, b = 0.f;
-            if (r < rows && o < d) {
-                const int i = (int)(r % n);
-                const int j = reader_of(i, s, n, flags);
-                a = dz[r * d + o];
-                b = j >= 0 ? dz[(r - i + j) * d + o] : 0.f;
-            }
-            gs[rr][tx] = a;
-            gp[rr][tx] = b;
-            const int oo = o0 + rr, k = k0 + tx;
-            ws[rr][tx] = (oo < d && k < d) ? Ws[(long long)oo * d + k] : 0.f;
-            wn[rr][tx] = (oo < d && k < d) ? Wn[(long long)oo * d + k] : 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            gs[ty + 8 * q][tx] = a[q];
+            gp[ty + 8 * q][tx] = b[q];
+            ws[ty + 8 * q][tx] = u[q];
+            wn[ty + 8 * q][tx] = v4[q];
         }
         __syncthreads();
+        if (o0 + T < d) load(o0 + T);
 #pragma unroll 8
         for (int oo = 0; oo < T; ++oo) {
 #pragma unroll
@@ -132,64 +180,121 @@ __global__ void f32_dx_kernel(const float* __restrict__ dz, const float* __restr
         }
         __syncthreads();
     }
-    const int k = k0 + tx;
     if (k >= d) return;
+    const int wpr = (d + 31) >> 5;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const long long r = r0 + ty + 8 * q;
         if (r >= rows) continue;
         float v = acc[q];
         if (flags & 2u) v += dy[r * d + k];
-        dx[r * d + k] = v;
+        if (dx) dx[r * d + k] = v;
+        // (the tile's 32 columns are one mask word)
+        if (dz_prev) dz_prev[r * d + k] = (mprev[r * wpr + (k0 >> 5)] >> tx) & 1u ? v : 0.f;
     }
 }
 
-// dWs[o][k] = sum_r dz[r][o] x[r][k];  dWn[o][k] = sum_r m_r dz[r][o] x[p(r)][k]
-// Block: 32 o x 32 k; the token loop is sequential (fixed order).
-__global__ void f32_dw_kernel(const float* __restrict__ x, const float* __restrict__ dz, int s,
-                              int n, int d, long long rows, unsigned flags,
-                              float* __restrict__ dWs, float* __restrict__ dWn) {
+// Per layer l and split sp of the rows,
+//   dWs[o][k] = sum_r dz[r][o] x[r][k];  dWn[o][k] = sum_r m_r dz[r][o] x[p(r)][k];
+//   dbias[o] = sum_r dz[r][o]
+// A block per 32 o x 32 k and (l, sp) = blockIdx.z; its rows in order.  One split
+// writes the gradients, several their partial sums [l][sp][2 d d + d], which
+// f32_dw_reduce_kernel adds in split order: the same bits every time.
+__global__ void __launch_bounds__(256) f32_dw_kernel(const __grid_constant__ F32DwArgs A) {
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
     __shared__ float gz[T][T + 1], xs[T][T + 1], xp[T][T + 1];
+    const int l = blockIdx.z / A.splits, sp = blockIdx.z - l * A.splits;
+    const int n = A.n, d = A.d, s = A.s[l];
+    const unsigned flags = A.flags;
+    const float* __restrict__ x = l == 0 ? A.x : A.acts + (l - 1) * A.act_elems;
+    const float* __restrict__ dz = A.dz + l * A.act_elems;
+    const long long rb = (long long)sp * A.rows_per_split;
+    const long long re = rb + A.rows_per_split < A.rows ? rb + A.rows_per_split : A.rows;
     const int o0 = blockIdx.y * T, k0 = blockIdx.x * T;
     const int tx = threadIdx.x, ty = threadIdx.y;
-    float as[4] = {0.f, 0.f, 0.f, 0.f}, an[4] = {0.f, 0.f, 0.f, 0.f};
-    for (long long r0 = 0; r0 < rows; r0 += T) {
-        for (int rr = ty; rr < T; rr += 8) {
-            const long long r = r0 + rr;
-            float g = 0.f, a = 0.f, b = 0.f;
-            if (r < rows) {
-                const int i = (int)(r % n);
-                if (o0 + tx < d) g = dz[r * d + o0 + tx];
-                if (k0 + tx < d) {
-                    a = x[r * d + k0 + tx];
-                    b = receives(i, s, flags) ? x[(r - i + partner_of(i, s)) * d + k0 + tx] : 0.f;
-                }
-            }
-            gz[rr][tx] = g;
-            xs[rr][tx] = a;
-            xp[rr][tx] = b;
+    float g[4], a[4], b[4];
+    auto load = [&](long long r0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const long long r = r0 + ty + 8 * q;
+            const int i = (int)(r & (n - 1));
+            g[q] = r < re && o0 + tx < d ? dz[r * d + o0 + tx] : 0.f;
+            a[q] = r < re && k0 + tx < d ? x[r * d + k0 + tx] : 0.f;
+            b[q] = r < re && k0 + tx < d && receives(i, s, flags)
+                       ? x[(r - i + partner_of(i, s)) * d + k0 + tx]
+                       : 0.f;
+        }
+    };
+    float as[4] = {0.f, 0.f, 0.f, 0.f}, an[4] = {0.f, 0.f, 0.f, 0.f}, cs = 0.f;
+    load(rb);
+    for (long long r0 = rb; r0 < re; r0 += T) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            gz[ty + 8 * q][tx] = g[q];
+            xs[ty + 8 * q][tx] = a[q];
+            xp[ty + 8 * q][tx] = b[q];
+            cs += g[q];
         }
         __syncthreads();
+        if (r0 + T < re) load(r0 + T);
 #pragma unroll 8
         for (int rr = 0; rr < T; ++rr) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const float g = gz[rr][ty + 8 * q];
-                as[q] = fmaf(g, xs[rr][tx], as[q]);
-                an[q] = fmaf(g, xp[rr][tx], an[q]);
+                const float gv = gz[rr][ty + 8 * q];
+                as[q] = fmaf(gv, xs[rr][tx], as[q]);
+                an[q] = fmaf(gv, xp[rr][tx], an[q]);
             }
         }
         __syncthreads();
     }
+    const size_t dd = (size_t)d * d;
+    float* part = A.part + ((size_t)l * A.splits + sp) * (2 * dd + d);
+    float* ws = A.splits > 1 ? part : A.dWs + l * dd;
+    float* wn = A.splits > 1 ? part + dd : A.dWn + l * dd;
     const int k = k0 + tx;
-    if (k >= d) return;
+    if (k < d) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int o = o0 + ty + 8 * q;
-        if (o >= d) continue;
-        dWs[(long long)o * d + k] = as[q];
-        dWn[(long long)o * d + k] = an[q];
+        for (int q = 0; q < 4; ++q) {
+            const int o = o0 + ty + 8 * q;
+            if (o >= d) continue;
+            ws[(size_t)o * d + k] = as[q];
+            wn[(size_t)o * d + k] = an[q];
+        }
     }
+    if (blockIdx.x == 0 && A.dbias) {
+        // the eight row lanes' column sums, in order
+        gz[ty][tx] = cs;
+        __syncthreads();
+        if (ty == 0 && o0 + tx < d) {
+            float t = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) t += gz[q][tx];
+            (A.splits > 1 ? part + 2 * dd : A.dbias + (size_t)l * d)[o0 + tx] = t;
+        }
+    }
+}
+
+// The split sums of f32_dw_kernel, in split order: a thread per output of layer
+// blockIdx.y.
+__global__ void __launch_bounds__(256) f32_dw_reduce_kernel(const __grid_constant__ F32DwArgs A) {
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
+    const int l = blockIdx.y;
+    const size_t dd = (size_t)A.d * A.d, tot = 2 * dd + A.d;
+    const size_t e = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (e >= tot || (e >= 2 * dd && !A.dbias)) return;
+    const float* p = A.part + (size_t)l * A.splits * tot + e;
+    float t = 0.f;
+#pragma unroll 8
+    for (int sp = 0; sp < A.splits; ++sp) t += p[sp * tot];
+    if (e < dd)
+        A.dWs[l * dd + e] = t;
+    else if (e < 2 * dd)
+        A.dWn[l * dd + e - dd] = t;
+    else
+        A.dbias[(size_t)l * A.d + e - 2 * dd] = t;
 }
 
 template <typename V>
@@ -239,6 +344,8 @@ __global__ void __launch_bounds__(256)
 __global__ void relu_grad_mask_f32_kernel(const float* __restrict__ dy,
                                           const uint32_t* __restrict__ mask,
                                           float* __restrict__ dz, long long rows, int d) {
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
     const int wpr = (d + 31) >> 5;
     const size_t count = (size_t)rows * d;
     for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < count;
@@ -282,27 +389,8 @@ __global__ void relu_grad_mask_kernel(const V* __restrict__ dy, const uint32_t* 
 // fill the GPU), 256 above (the partials stay small)
 inline long long col_rows(long long rows) { return rows <= 65536 ? 64 : 256; }
 
-// partial[c][o] = sum_{r in chunk c} dz[r][o] for any d (block: 32 columns x
-// 8 row lanes).
-__global__ void colsum_partial_f32_kernel(const float* __restrict__ dz, long long rows, int d,
-                                          int crows, float* __restrict__ partial) {
-    __shared__ float red[8][33];
-    const int o = blockIdx.x * 32 + threadIdx.x;
-    const long long r0 = (long long)blockIdx.y * crows;
-    const long long r1 = min(rows, r0 + crows);
-    float acc = 0.f;
-    if (o < d)
-        for (long long r = r0 + threadIdx.y; r < r1; r += 8) acc += dz[r * d + o];
-    red[threadIdx.y][threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.y == 0 && o < d) {
-        float s = 0.f;
-        for (int q = 0; q < 8; ++q) s += red[q][threadIdx.x];
-        partial[(long long)blockIdx.y * d + o] = s;
-    }
-}
-
-// The same for bf16 rows (d a multiple of 64), 16-byte loads.  Block: 64
+// partial[c][o] = sum_{r in chunk c} dz[r][o] for bf16 rows (d a multiple of 64),
+// 16-byte loads.  Block: 64
 // column groups of 16 bytes x 4 row lanes; each thread sums its group over every 4th row of
 // the chunk, then the 4 row lanes are added in a fixed order.
 template <typename V>
@@ -446,16 +534,14 @@ cudaError_t launch_f32_fwd(const float* x, const float* Ws, const float* Wn, con
                            uint32_t* mout, cudaStream_t st) {
     const long long rows = (long long)B * n;
     dim3 grid((d + T - 1) / T, (unsigned)((rows + T - 1) / T));
-    f32_fwd_kernel<<<grid, dim3(T, 8), 0, st>>>(x, Ws, Wn, bias, s, n, d, rows, flags, y, z,
-                                                 mout);
-    return cudaGetLastError();
+    return launch_pdl(f32_fwd_kernel, grid, dim3(T, 8), 0, st, x, Ws, Wn, bias, s, n, d, rows,
+                      flags, y, z, mout);
 }
 
 cudaError_t launch_relu_grad_mask_f32(const float* dy, const uint32_t* mask, float* dz,
                                       long long rows, int d, cudaStream_t st) {
-    relu_grad_mask_f32_kernel<<<blocks_for((size_t)rows * d, 256), 256, 0, st>>>(dy, mask, dz,
-                                                                              rows, d);
-    return cudaGetLastError();
+    return launch_pdl(relu_grad_mask_f32_kernel, dim3(blocks_for((size_t)rows * d, 256)), dim3(256),
+                      0, st, dy, mask, dz, rows, d);
 }
 
 cudaError_t launch_relu_grad_mask_bf16(const __nv_bfloat16* dy, const uint32_t* mask,
@@ -468,19 +554,39 @@ cudaError_t launch_relu_grad_mask_bf16(const __nv_bfloat16* dy, const uint32_t* 
 
 cudaError_t launch_f32_dx(const float* dz, const float* dy, const float* Ws, const float* Wn,
                           int s, int B, int n, int d, unsigned flags, float* dx,
-                          cudaStream_t st) {
+                          const uint32_t* mprev, float* dz_prev, cudaStream_t st) {
     const long long rows = (long long)B * n;
     dim3 grid((d + T - 1) / T, (unsigned)((rows + T - 1) / T));
-    f32_dx_kernel<<<grid, dim3(T, 8), 0, st>>>(dz, dy, Ws, Wn, s, n, d, rows, flags, dx);
-    return cudaGetLastError();
+    return launch_pdl(f32_dx_kernel, grid, dim3(T, 8), 0, st, dz, dy, Ws, Wn, s, n, d, rows, flags,
+                      dx, mprev, dz_prev);
 }
 
-cudaError_t launch_f32_dw(const float* x, const float* dz, int s, int B, int n, int d,
-                          unsigned flags, float* dWs, float* dWn, cudaStream_t st) {
-    const long long rows = (long long)B * n;
-    dim3 grid((d + T - 1) / T, (d + T - 1) / T);
-    f32_dw_kernel<<<grid, dim3(T, 8), 0, st>>>(x, dz, s, n, d, rows, flags, dWs, dWn);
-    return cudaGetLastError();
+// Splits of the rows: enough blocks for two an SM, at least 128 rows (four steps)
+// each.  One split at 49 tiles (d = 200) leaves 103 SMs idle and walks all rows in
+// one block.
+int f32_dw_splits(long long rows, int d, int layers, int sms) {
+    const long long tiles = (long long)((d + T - 1) / T) * ((d + T - 1) / T) * layers;
+    long long s = (2ll * sms + tiles - 1) / tiles;
+    if (s > rows / 128) s = rows / 128;
+    return s < 1 ? 1 : (int)s;
+}
+
+cudaError_t launch_f32_dw(F32DwArgs& a, int layers, int splits, cudaStream_t st, int* launches) {
+    *launches = 0;
+    const long long steps = (a.rows + T - 1) / T;
+    a.rows_per_split = (steps + splits - 1) / splits * T;
+    a.splits = (int)((a.rows + a.rows_per_split - 1) / a.rows_per_split);   // no empty split
+    const unsigned t = (unsigned)((a.d + T - 1) / T);
+    cudaError_t e = launch_pdl(f32_dw_kernel, dim3(t, t, (unsigned)(layers * a.splits)),
+                               dim3(T, 8), 0, st, a);
+    if (e != cudaSuccess) return e;
+    *launches = 1;
+    if (a.splits == 1) return e;
+    const size_t tot = 2 * (size_t)a.d * a.d + a.d;
+    e = launch_pdl(f32_dw_reduce_kernel, dim3((unsigned)((tot + 255) / 256), (unsigned)layers),
+                   dim3(256), 0, st, a);
+    if (e == cudaSuccess) *launches = 2;
+    return e;
 }
 
 cudaError_t launch_relu_grad_f32(const float* dy, const float* z, float* dz, size_t count,
@@ -510,14 +616,9 @@ static cudaError_t colsum(const V* dz, long long rows, int d, float* partial, fl
         cudaError_t e = cudaMemsetAsync(out, 0, (size_t)batch * d * sizeof(float), st);
         return e;
     }
-    if (sizeof(V) == 4) {
-        colsum_partial_f32_kernel<<<dim3((d + 31) / 32, (unsigned)chunks, 1), dim3(32, 8), 0, st>>>(
-            reinterpret_cast<const float*>(dz), rows, d, crows, partial);
-    } else {
-        constexpr int VEC = 16 / sizeof(V);
-        dim3 grid((d / VEC + 63) / 64, (unsigned)chunks, (unsigned)batch);
-        colsum_partial_kernel<V><<<grid, dim3(64, 4), 0, st>>>(dz, rows, d, crows, partial);
-    }
+    constexpr int VEC = 16 / sizeof(V);
+    dim3 grid((d / VEC + 63) / 64, (unsigned)chunks, (unsigned)batch);
+    colsum_partial_kernel<V><<<grid, dim3(64, 4), 0, st>>>(dz, rows, d, crows, partial);
     colsum_final_kernel<<<dim3((d + 31) / 32, batch), 1024, 0, st>>>(partial, (int)chunks, d, out);
     return cudaGetLastError();
 }
@@ -525,11 +626,6 @@ static cudaError_t colsum(const V* dz, long long rows, int d, float* partial, fl
 cudaError_t launch_colsum_bf16_batched(const __nv_bfloat16* dz, int batch, long long rows, int d,
                                        float* partial, float* out, cudaStream_t st) {
     return colsum<__nv_bfloat16>(dz, rows, d, partial, out, st, batch);
-}
-
-cudaError_t launch_colsum_f32(const float* dz, long long rows, int d, float* partial,
-                              float* out, cudaStream_t st) {
-    return colsum<float>(dz, rows, d, partial, out, st);
 }
 
 cudaError_t launch_colsum_bf16(const __nv_bfloat16* dz, long long rows, int d, float* partial,

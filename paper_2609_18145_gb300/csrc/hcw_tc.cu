@@ -1507,7 +1507,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                 // FWD z (layer API only): the pre-activation, from the accumulator
                 // again (held until now) through the same patch buffer once the y store
                 // has read it: whole rows by TMA.  Row pieces stored from registers took
-                // 24 us of a 16,384-token layer at d = 512, this 20.
+                // 24 us of a 16,384-token layer at d = 512, this 19.
                 if (want_z) {
                     if (lane == 0) bulk_wait_read<0>();
                     __syncwarp();

@@ -416,6 +416,31 @@ def test_stack_with_a_schedule_array(H, case):
         H.hcw_set_stack_kernels(prev)
 
 
+@pytest.mark.parametrize("B, n, d, L, flags", [
+    (5, 64, 33, 3, CAUSAL | RESIDUAL | RELU),   # two row splits, the second ragged; d past a tile
+    (13, 32, 32, 2, RELU),                      # no residual: no unmasked gradient is kept
+    (1, 256, 100, 2, RESIDUAL),                 # 4 x 4 tiles, two splits
+    (3, 2, 5, 66, CAUSAL | RESIDUAL),           # more layers than one launch takes
+])
+def test_fp32_stack_gradients_in_one_launch(H, B, n, d, L, flags):
+    """The fp32 weight and bias gradients of all layers in one launch, with and without
+    row splits, and the dz chain written by the input-gradient launches, against the
+    oracle on the oracle's own activations."""
+    pr = synth.problem(B, n, d, L=L, seed=31, w_std=(1 / (2 * d)) ** 0.5 / L ** 0.5)
+    x, x64 = dev(pr.x, torch.float32)
+    Ws, Ws64 = dev(pr.W_self, torch.float32)
+    Wn, Wn64 = dev(pr.W_nbr, torch.float32)
+    dy, dy64 = dev(pr.dy, torch.float32)
+    _, racts, rzs = O.stack_fwd(x64, Ws64, Wn64, pr.bias.astype(np.float64), 0, L, -1, flags)
+    o_acts = torch.from_numpy(racts[1:]).float().cuda()
+    o_masks = masks_from_z(rzs).cuda() if flags & RELU else None
+    got = H.hcw_stack_bwd(x, o_acts, o_masks, dy, Ws, Wn, 0, -1, flags)
+    torch.cuda.synchronize()
+    ref = O.stack_bwd(racts, rzs, dy64, Ws64, Wn64, 0, L, -1, flags)
+    for a, r, what in zip(got, ref, ("dx", "dW_self", "dW_nbr", "dbias")):
+        assert rel(host(a), r) <= TOL_F32, what
+
+
 @pytest.mark.parametrize("flags", [CAUSAL | RESIDUAL | RELU, 0])
 def test_shift_schedule_fp32(H, flags):
     """The fp32 path (CUDA-core kernels) on a schedule of near, jump and shift
