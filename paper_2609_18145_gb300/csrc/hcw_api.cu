@@ -2277,11 +2277,17 @@ int hcw_decode_step(const void* x_t, const void* W_self, const void* W_nbr, cons
         p.prow[l] = recv ? (int)(slot(l, t + 1) / d) : -1;   // the slot of t - k_l
         p.out[l] = l == L - 1 ? static_cast<__nv_bfloat16*>(y_t) : ring + slot(l + 1, t);
     }
-    if (!map_tiles_sw128(&p.mWs, W_self, (long long)L * d, d, geo.oc, geo.kc / 64) ||
+    p.tc = g_decode_kernel.load(std::memory_order_relaxed) == HCW_DECODE_TCGEN05;
+    if (p.tc &&
+        (!map_tiles_sw128(&p.mWs, W_self, (long long)L * d, d, geo.oc, geo.kc / 64) ||
         !map_tiles_sw128(&p.mWn, W_nbr, (long long)L * d, d, geo.oc, geo.kc / 64) ||
         !map_tiles_sw128(&p.mCache, cache, (long long)(off[L] / d), d, 16, d / 64) ||
-        !map_tiles_sw128(&p.mX, x_t, B, d, 16, d / 64))
+        !map_tiles_sw128(&p.mX, x_t, B, d, 16, d / 64)))
         return HCW_ERR_CUDA;
+    p.Ws = static_cast<const __nv_bfloat16*>(W_self);
+    p.Wn = static_cast<const __nv_bfloat16*>(W_nbr);
+    p.x = static_cast<const __nv_bfloat16*>(x_t);
+    p.cache = ring;
     p.bias = bias;
     p.ring0 = ring + slot(0, t);
     p.g = geo;
@@ -2289,7 +2295,6 @@ int hcw_decode_step(const void* x_t, const void* W_self, const void* W_nbr, cons
     p.B = B;
     p.flags = flags;
     p.timeout_ns = g_timeout_ns;
-    p.tc = g_decode_kernel.load(std::memory_order_relaxed) == HCW_DECODE_TCGEN05;
     return launched(launch_decode(p, st), 1);
 }
 

@@ -15,43 +15,36 @@
 // one earlier position of the same sequence), so one position of the whole
 // stack splits into independent blocks of 16 rows.  A thread-block cluster of
 // C CTAs (C <= 16) runs one row block through all L layers; CTA q of the
-// cluster owns output columns [q OC, (q + 1) OC), OC = d / C.  Per layer:
-//   - a producer thread streams the CTA's weight rows (OC rows of W_nbr, then
-//     of W_self, in K chunks) into a ring of shared-memory stages, and the
-//     partner rows (16 x d, inputs of earlier positions) into a partner
-//     buffer, running ahead of the layers.  Each moves as ONE TMA copy, a
-//     3-D box (64 features, rows, K tiles) with the 128-byte swizzle that lands
-//     as consecutive 64-feature tiles; one tensor map over the whole cache
-//     serves every ring slot;
-//   - eight MMA warps contract the partner part first (it does not depend on
-//     the previous layer), then the self part once the layer input is
-//     complete: [16 x d] x [d x OC] twice, fp32 accumulation;
-//   - the epilogue (bias, ReLU, residual, bf16) writes the CTA's 16 x OC slice
-//     to the next layer's ring slot in global memory and pushes it into every
-//     cluster CTA's input buffer of the next layer with asynchronous remote
-//     stores (distributed shared memory) that count their bytes on that CTA's
-//     "input ready" mbarrier: the layer input is complete when all 16 x d x 2
-//     bytes have landed, with no fence or barrier between the CTAs.
-// No layer boundary goes through global memory or a grid-wide barrier.
+// cluster owns output columns [q OC, (q + 1) OC), OC = d / C, and contracts the
+// partner part first (it does not depend on the previous layer), then the self
+// part once the layer input is complete: [16 x d] x [d x OC] twice, fp32
+// accumulation.  The epilogue (bias, ReLU, residual, bf16) writes the CTA's 16 x
+// OC slice to the next layer's ring slot in global memory and sends it into every
+// cluster CTA's input buffer of the next layer (distributed shared memory: bulk
+// copies, or in decode_tc_kernel asynchronous remote stores) with its bytes
+// counted on that CTA's "input ready" mbarrier: the layer input is complete when
+// every slice has landed, with no fence or barrier between the CTAs.  No layer boundary
+// goes through global memory or a grid-wide barrier.
 //
-// Two contractions (decode_kernel<TC>, chosen with hcw_set_decode_kernel):
-//   - TC = false (the default): eight warps share the K range with the
-//     warp-level bf16 MMA (m16n8k16) and add their 16 x 8 blocks into the
-//     CTA's row sums;
-//   - TC = true: one thread issues tcgen05.mma.  A tile holds 16 rows, below
-//     the 64-row minimum, so the MMA runs with M = 64 on the 16 rows (its
-//     other 48 rows read whatever follows in shared memory; only D's rows
-//     0..15, TMEM lanes 0..15, are used) and N = OC.  The operands are already
-//     in the MMA's K-major 128-byte-swizzled layout.  Warp 7 issues, warp 0
-//     drains D into the row sums, and a layer's partner part is contracted
-//     into the other of two accumulators while the layer before is drained.
-// A layer is a chain (input in, contraction, epilogue, pushes out).  Issuing
-// a layer's 32 partner-part MMAs (N = OC = 32 at d = 512, K = 16) only after
-// its input arrived costs 0.75 us a layer, so one thread's tcgen05.mma run
-// about 45 cycles each in sequence, where the eight warps' MMAs run side by
-// side; the commit, the TMEM drain and a proxy fence (the remote stores are
-// generic writes that the MMA reads through the async proxy) add to the chain.
-// So the tensor-core version is the slower of the two here.
+// Two contractions (hcw_set_decode_kernel):
+//   - decode_mma_kernel (the default): eight warps share the K range with the
+//     warp-level bf16 MMA (m16n8k16), weights and partner rows straight from
+//     global memory into registers;
+//   - decode_tc_kernel: one thread issues tcgen05.mma over weights that a
+//     producer warp streams into a ring of shared-memory stages by TMA (3-D boxes
+//     of 64 features, rows, K tiles, 128-byte swizzle), running ahead of the
+//     layers; the partner rows come the same way.  A tile holds 16 rows, below
+//     the 64-row minimum, so the MMA runs with M = 64 on the 16 rows (its other
+//     48 rows read whatever follows in shared memory; only D's rows 0..15, TMEM
+//     lanes 0..15, are used) and N = OC.  Warp 7 issues, warp 0 drains D into the
+//     row sums, and a layer's partner part is contracted into the other of two
+//     accumulators while the layer before is drained.  Issuing a layer's 32
+//     partner-part MMAs (N = OC = 32 at d = 512, K = 16) only after its input
+//     arrived costs 0.75 us a layer, so one thread's tcgen05.mma run about 45
+//     cycles each in sequence; the commit, the TMEM drain and a proxy fence (the
+//     remote stores are generic writes that the MMA reads through the async
+//     proxy) add to the chain.  So the tensor-core version is the slower of the
+//     two here.
 #include "hcw_internal.h"
 #include "hcw_ptx.cuh"
 
@@ -60,10 +53,10 @@ namespace hcw {
 namespace {
 
 constexpr int kRows = 16;          // rows of a row block
-constexpr int kMmaWarps = 8;       // warps 0..7: MMA + epilogue (TC: warp 7 issues, warps
-                                   // 0..6 run the epilogue); warp 8: producer
+constexpr int kMmaWarps = 8;       // warps 0..7: MMA + epilogue (decode_tc_kernel: warp 7
+                                   // issues, warps 0..6 run the epilogue; warp 8: producer)
 constexpr int kThreads = (kMmaWarps + 1) * 32;
-// TC: accumulators a layer's K tiles alternate over, for each layer parity (64
+// decode_tc_kernel: accumulators a layer's K tiles alternate over, for each layer parity (64
 // columns each); four in turn measured no faster than one
 constexpr int kNAcc = 1;
 constexpr uint32_t kTmemCols = 2 * kNAcc * 64 < 32 ? 32 : 2 * kNAcc * 64;
@@ -83,21 +76,21 @@ struct DecodeArgs {
     unsigned long long timeout_ns;
 };
 
-// barrier slots
+// barrier slots of decode_tc_kernel
 enum : int {
     B_FULL = 0,                       // [kMaxStages] stage filled (tx bytes)
-    B_EMPTY = kMaxStages,             // [kMaxStages] stage consumed (8 MMA warps, or a commit)
+    B_EMPTY = kMaxStages,             // [kMaxStages] stage consumed (a commit)
     B_XS_READY = 2 * kMaxStages,      // [2] layer input complete (tx bytes from every cluster CTA)
     B_X0 = 2 * kMaxStages + 2,        // x_t rows loaded
     B_XP_FULL = 2 * kMaxStages + 3,   // [2] partner rows loaded
-    B_XP_FREE = 2 * kMaxStages + 5,   // [2] partner buffer consumed (8 MMA warps, or a commit)
-    B_DFULL = 2 * kMaxStages + 7,     // TC: [2] a layer's accumulator complete (commit)
-    B_TFREE = 2 * kMaxStages + 9,     // TC: [2] a layer's accumulator drained by warp 0
-    B_DRAIN = 2 * kMaxStages + 11,    // TC: the issuer's last MMAs completed
+    B_XP_FREE = 2 * kMaxStages + 5,   // [2] partner buffer consumed (a commit)
+    B_DFULL = 2 * kMaxStages + 7,     // [2] a layer's accumulator complete (commit)
+    B_TFREE = 2 * kMaxStages + 9,     // [2] a layer's accumulator drained by warp 0
+    B_DRAIN = 2 * kMaxStages + 11,    // the issuer's last MMAs completed
     B_COUNT = 2 * kMaxStages + 12
 };
 
-// Shared memory (1024-byte aligned): Xs[2] (layer inputs) and Xp[2] (partner
+// Shared memory of decode_tc_kernel (1024-byte aligned): Xs[2] (layer inputs) and Xp[2] (partner
 // rows), each d / 64 tiles of 16 rows x 128 bytes; stages[S], each kc / 64
 // tiles of OC rows x 128 bytes; all bf16 in the 128-byte swizzle (16-byte
 // chunk c of row r at chunk c ^ (r & 7)).  Then red[2][16][OC] fp32 (the
@@ -128,18 +121,6 @@ struct Smem {
 __device__ __forceinline__ uint32_t sw_off(int r, int col, uint32_t tile_bytes) {
     const int ch = (col >> 3) & 7;
     return (uint32_t)(col >> 6) * tile_bytes + r * 128 + ((ch ^ (r & 7)) << 4);
-}
-
-__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1,
-                                            uint32_t& r2, uint32_t& r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(addr));
-}
-__device__ __forceinline__ void ldmatrix_x2(uint32_t addr, uint32_t& r0, uint32_t& r1) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];"
-                 : "=r"(r0), "=r"(r1)
-                 : "r"(addr));
 }
 
 // D (16 x 8, fp32) += A (16 x 16 bf16, row-major) * B (16 x 8 bf16, column-major)
@@ -207,7 +188,7 @@ __device__ __forceinline__ void decode_epilogue(const DecodeArgs& a, const Smem&
     }
 }
 
-// The MMA and epilogue warps of decode_kernel<true>: warp 7 issues the
+// The MMA and epilogue warps of decode_tc_kernel: warp 7 issues the
 // tcgen05 MMAs, warp 0 drains each layer's accumulator into the row sums, and
 // warps 0..6 run the epilogue (bias, ReLU, residual, bf16, pushes).
 __device__ __forceinline__ void decode_tc_body(const DecodeArgs& a, const Smem& sm, int warp,
@@ -361,8 +342,8 @@ __device__ __forceinline__ void decode_tc_body(const DecodeArgs& a, const Smem& 
     }
 }
 
-template <bool TC>
-__global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_constant__ DecodeArgs a) {
+__global__ void __launch_bounds__(kThreads, 1)
+    decode_tc_kernel(const __grid_constant__ DecodeArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -375,29 +356,27 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
     const int vr = a.B - row0 < kRows ? a.B - row0 : kRows;   // valid rows
     const int d = g.d, oc = g.oc, col0 = q * oc;
     const int nch = g.nchunks;
-    const uint32_t xtile = kRows * 128, wtile = (uint32_t)oc * 128;
     volatile int* abort = sm.abort_word();
 
-    for (int i = threadIdx.x; i < 2 * kRows * oc; i += kThreads) sm.red(0)[i] = 0.f;
     if (threadIdx.x == 0) {
         *abort = 0;
         for (int s = 0; s < g.stages; ++s) {
             mbar_init(&bars[B_FULL + s], 1);
-            mbar_init(&bars[B_EMPTY + s], TC ? 1 : kMmaWarps);
+            mbar_init(&bars[B_EMPTY + s], 1);
         }
         mbar_init(&bars[B_XS_READY + 0], 1);
         mbar_init(&bars[B_XS_READY + 1], 1);
         mbar_init(&bars[B_X0], 1);
         for (int b = 0; b < 2; ++b) {
             mbar_init(&bars[B_XP_FULL + b], 1);
-            mbar_init(&bars[B_XP_FREE + b], TC ? 1 : kMmaWarps);
+            mbar_init(&bars[B_XP_FREE + b], 1);
             mbar_init(&bars[B_DFULL + b], 1);
             mbar_init(&bars[B_TFREE + b], 1);
         }
         mbar_init(&bars[B_DRAIN], 1);
         fence_mbar_init();
     }
-    if (TC && warp == 0) {
+    if (warp == 0) {
         tmem_alloc(sm.tmem_slot(), kTmemCols);
         tmem_relinquish();
     }
@@ -466,130 +445,447 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(const __grid_consta
             }
         }
         __syncwarp();
-    } else if (TC) {
-        decode_tc_body(a, sm, warp, lane, q, row0, vr);
     } else {
-        // ---------------------------------------------------- MMA + epilogue
-        const int nb_count = oc / 8;               // n8 blocks: 2, 4 or 8
-        const int ksplit = kMmaWarps / nb_count;   // warps sharing an n8 block
-        const int nb = warp % nb_count, kh = warp / nb_count;
-        const int gr = lane >> 2, gc = (lane & 3) * 2;
-        // ldmatrix lanes: A rows lane & 15, feature chunk + (lane >> 4); B
-        // (weight) rows nb 8 + (lane & 7), feature chunk + ((lane >> 3) & 1)
-        const int ar = lane & 15, ahi = lane >> 4;
-        const int br = nb * 8 + (lane & 7), bhi = (lane >> 3) & 1;
-        uint32_t it = 0;
-        int xp_uses[2] = {0, 0};
-        bool ok = true;
-        // every lane waits (each gets the acquire); the outcome is made
-        // warp-uniform so that the aligned MMAs never run divergent
-        auto wait = [&](uint64_t* bar, uint32_t parity, bool cluster) {
-            bool r = ok && (cluster ? mbar_wait_cluster(bar, parity, abort, a.timeout_ns)
-                                    : mbar_wait(bar, parity, abort, a.timeout_ns));
-            ok = __all_sync(0xffffffffu, r);
-        };
-        const int packs = kRows * oc / 8;   // epilogue: a thread per 8 columns of a row
-        const int pr = threadIdx.x / (oc / 8), pc8 = (threadIdx.x % (oc / 8)) * 8;
-        const uint32_t poff = sw_off(pr, col0 + pc8, xtile);
-        for (int l = 0; l < a.L; ++l) {
-            const int xb = l & 1;
-            const bool recv = a.prow[l] >= 0;
-            // the next layer's input arrives as 16 x d x 2 bytes from the cluster
-            if (threadIdx.x == 0 && l + 1 < a.L)
-                mbar_arrive_expect_tx(&bars[B_XS_READY + (xb ^ 1)], (uint32_t)kRows * d * 2);
-            // this thread's bias values, loaded while the layer runs
-            float4 bv0 = make_float4(0.f, 0.f, 0.f, 0.f), bv1 = bv0;
-            if (a.bias && (int)threadIdx.x < packs) {
-                const float4* bl =
-                    reinterpret_cast<const float4*>(a.bias + (size_t)l * d + col0 + pc8);
-                bv0 = __ldg(bl);
-                bv1 = __ldg(bl + 1);
-            }
-            // four independent accumulators: consecutive MMAs do not wait on each other
-            float acc[4][4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) acc[u][e] = 0.f;
-            for (int part = recv ? 1 : 0; part >= 0; --part) {
-                uint32_t X;
-                if (part) {
-                    wait(&bars[B_XP_FULL + xb], xp_uses[xb]++ & 1, false);
-                    X = smem_u32(sm.xpart(xb));
-                } else {
-                    if (l == 0)
-                        wait(&bars[B_X0], 0, false);
-                    else
-                        wait(&bars[B_XS_READY + xb], ((l - 1) >> 1) & 1, true);
-                    X = smem_u32(sm.xs(xb));
-                }
-                for (int c = 0; c < nch; ++c, ++it) {
-                    const int s = (int)(it % (uint32_t)g.stages);
-                    wait(&bars[B_FULL + s], (it / g.stages) & 1, false);
-                    if (ok) {
-                        const uint32_t W = smem_u32(sm.stage(s));
-                        const int ks_n = chunk_len(g, c) / 16;
-                        const int kc0 = c * g.kc;
-                        int ks = kh;
-                        for (; ks + 3 * ksplit < ks_n; ks += 4 * ksplit) {
-                            uint32_t af[4][4], bf[4][2];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                const int kl = (ks + u * ksplit) * 16;
-                                ldmatrix_x4(X + sw_off(ar, kc0 + kl + ahi * 8, xtile), af[u][0],
-                                            af[u][1], af[u][2], af[u][3]);
-                                ldmatrix_x2(W + sw_off(br, kl + bhi * 8, wtile), bf[u][0],
-                                            bf[u][1]);
-                            }
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) mma_16816(acc[u], af[u], bf[u][0], bf[u][1]);
-                        }
-                        for (; ks < ks_n; ks += ksplit) {
-                            const int kl = ks * 16;
-                            uint32_t af[4], b0, b1;
-                            ldmatrix_x4(X + sw_off(ar, kc0 + kl + ahi * 8, xtile), af[0], af[1],
-                                        af[2], af[3]);
-                            ldmatrix_x2(W + sw_off(br, kl + bhi * 8, wtile), b0, b1);
-                            mma_16816(acc[0], af, b0, b1);
-                        }
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&bars[B_EMPTY + s]);
-                }
-                if (part && lane == 0) mbar_arrive(&bars[B_XP_FREE + xb]);
-            }
-            // this warp's partial 16 x 8 block into the CTA's sums of this layer
-            float* red = sm.red(xb);
-            const int cb = nb * 8 + gc;
-            atomicAdd(&red[gr * oc + cb], acc[0][0] + acc[1][0] + acc[2][0] + acc[3][0]);
-            atomicAdd(&red[gr * oc + cb + 1], acc[0][1] + acc[1][1] + acc[2][1] + acc[3][1]);
-            atomicAdd(&red[(gr + 8) * oc + cb], acc[0][2] + acc[1][2] + acc[2][2] + acc[3][2]);
-            atomicAdd(&red[(gr + 8) * oc + cb + 1], acc[0][3] + acc[1][3] + acc[2][3] + acc[3][3]);
-            // every thread past this point has finished the previous layer's
-            // epilogue, so the other partial-sum buffer is free again
-            named_bar_sync(1, kMmaWarps * 32);
-            if ((int)threadIdx.x < packs) {
-                const uint4 xin = *reinterpret_cast<const uint4*>(sm.xs(xb) + poff);
-                float* rr = red + pr * oc + pc8;
-                const float bvals[8] = {bv0.x, bv0.y, bv0.z, bv0.w, bv1.x, bv1.y, bv1.z, bv1.w};
-                float v[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    v[e] = rr[e] + bvals[e];
-                    rr[e] = 0.f;
-                }
-                decode_epilogue(a, sm, v, xin, l, xb, q, row0, vr, pr, pc8, poff);
-            }
-        }
+        decode_tc_body(a, sm, warp, lane, q, row0, vr);
     }
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();   // no CTA leaves while a peer may still write its shared memory
-    if (TC && warp == 0) {
+    if (warp == 0) {
         __syncwarp();
         tc_fence_after();
         tmem_dealloc(*sm.tmem_slot(), kTmemCols);
     }
+}
+
+// ------------------------------------------------------------ warp-level MMA
+struct DecodeMmaArgs {
+    const __nv_bfloat16 *Ws, *Wn;   // [L d][d]
+    const __nv_bfloat16* x;         // x_t [B][d]
+    const __nv_bfloat16* cache;     // the rings as [rows][d]
+    const float* bias;              // [L][d] or null
+    __nv_bfloat16* ring0;           // layer 0's ring slot of position t
+    int prow[kMaxDecodeLayers];             // cache row of the partner slot, or -1
+    __nv_bfloat16* out[kMaxDecodeLayers];   // [B][d] next layer's ring slot, or y_t
+    int d, csize, L, B;
+    unsigned flags;
+    unsigned long long timeout_ns;
+};
+
+// A layer-input buffer holds the cluster's slices one after the other, each 16 rows of
+// OC features, as a CTA sends its slice: one copy a peer.  Bytes of a row, of a slice as
+// copied, and from slice to slice; the odd 16 bytes put the 16-byte reads of a
+// fragment's rows on different banks (for OC = 16 on two a bank).
+__host__ __device__ constexpr int mma_row_bytes(int oc) { return 2 * oc + (oc == 64 ? 16 : 0); }
+__host__ __device__ constexpr int mma_slice_bytes(int oc) { return kRows * mma_row_bytes(oc); }
+__host__ __device__ constexpr int mma_slice_step(int oc) {
+    return mma_slice_bytes(oc) + (oc == 64 ? 0 : 16);
+}
+// floats per row of a warp's block of sums (OC + 8: the fragments' rows on different banks)
+__host__ __device__ constexpr int mma_sum_row(int oc) { return oc + 8; }
+
+// whether the partner parts have warps of their own (kPWarps), and the threads of a CTA
+constexpr int kPWarps = 4;
+__host__ __device__ constexpr bool mma_split(int oc) { return oc < 64; }
+__host__ __device__ constexpr int mma_threads(int oc) {
+    return (kMmaWarps + (mma_split(oc) ? kPWarps : 0)) * 32;
+}
+constexpr int kMmaBars = 2 + 4 * kPWarps;
+
+// bytes from this CTA's shared memory into a cluster CTA's; they complete on that CTA's
+// mbarrier (destination and barrier as shared::cluster addresses)
+__device__ __forceinline__ void copy_to_peer(uint32_t dst, uint32_t src, uint32_t bytes,
+                                             uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, "
+        "[%3];" ::"r"(dst),
+        "r"(src), "r"(bytes), "r"(bar)
+        : "memory");
+}
+
+// 16 features of a row
+struct Feat16 {
+    uint32_t r[8];
+};
+// one 32-byte load of a 32-byte aligned piece (W32), else two of 16 bytes.  (Not the
+// read-only path: the kernel before this one, which this one's start overlaps, may
+// have written the ring slot.)
+template <bool W32>
+__device__ __forceinline__ Feat16 ldg_stream(const void* p) {
+    Feat16 v;
+    if constexpr (W32) {
+        asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(v.r[0]), "=r"(v.r[1]), "=r"(v.r[2]), "=r"(v.r[3]), "=r"(v.r[4]),
+                       "=r"(v.r[5]), "=r"(v.r[6]), "=r"(v.r[7])
+                     : "l"(p));
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            asm volatile("ld.global.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(v.r[4 * h]), "=r"(v.r[4 * h + 1]), "=r"(v.r[4 * h + 2]),
+                           "=r"(v.r[4 * h + 3])
+                         : "l"(static_cast<const uint8_t*>(p) + 16 * h));
+    }
+    return v;
+}
+__device__ __forceinline__ Feat16 lds16(const uint8_t* p) {
+    const uint4 a = *reinterpret_cast<const uint4*>(p), b = *reinterpret_cast<const uint4*>(p + 16);
+    return Feat16{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+}
+
+// Warp w (of eight) contracts the K groups (64 features) w GP .. w GP + GP - 1 with all OC
+// columns.  Inside a group the contraction may take the features in any order, as long
+// as both operands do: lane (g = lane / 4, c = lane % 4) takes features 16 c .. 16 c + 15
+// of rows g and g + 8 of the input and of weight rows 8 u + g, one 32-byte load each
+// (a warp's load: eight whole 128-byte lines), and those are the fragments of the
+// group's four MMAs (MMA m takes the pieces' words 2 m and 2 m + 1).  So the weights and the partner rows go from global
+// memory (L2) straight into the registers the MMA reads; as a group has been
+// contracted, its registers are reloaded for the next part.  The sums of the eight
+// warps meet in shared memory in warp order (deterministic).
+//
+// OC < 64 (SPLIT): warps 8 .. 11 contract the partner parts (a quarter of the K groups
+// each), up to two layers ahead of warps 0 .. 7, and hand their accumulators to warps 0
+// .. 3 to start the self part with.  Warps 0 .. 7 hold the self weights of two layers:
+// a layer's are requested a whole layer before they are needed, between its pushes
+// and the next input's arrival, where issuing loads costs the chain nothing.  At OC =
+// 64 (d > 512) a part takes 128 registers a lane: eight warps contract both parts in
+// turn and reload a group as it has been contracted.
+//
+// What bounds it: the bytes an SM takes in, and a chain per layer (input landed, self
+// MMAs, sums, epilogue, slices sent and landed).  64 KB of weights and 16 KB of slices a
+// layer at d = 512 are 2,000 cycles at the 39 bytes a cycle an SM gets from L2; the
+// chain alone is about 1,500, of which the MMAs take 260.  So it holds no wait but the
+// input's, no address arithmetic that could be set up before, no constant-cache line
+// first touched there and no global load (the layer table and the biases are copied to
+// shared memory first: a bias load queued behind the weights' took 800 cycles), no
+// float atomics in shared memory (a compare-and-swap loop, 110 cycles each), and one
+// bulk copy a peer (1,024 remote 16-byte stores waited behind the weight loads, 850).
+// Microseconds a position at 64 sequences, 16 layers, d = 512, and cycles a layer:
+//   weights staged in shared memory by TMA, atomics, remote stores     52    6,900
+//   no atomics, whole parts staged (one wait a part)                   33    4,350
+//   weights in registers, eight warps for both parts                   30    4,200
+//   partner warps                                                      27    3,300
+//   self weights two layers deep, biases in shared memory              25    3,200
+//   slices sent as bulk copies (this)                                  23    2,600
+template <int OC, int GP, bool W32>
+__global__ void __launch_bounds__(mma_threads(OC), 1)
+    decode_mma_kernel(const __grid_constant__ DecodeMmaArgs a) {
+    constexpr bool SPLIT = mma_split(OC);
+    constexpr int NB = OC / 8;                               // n8 blocks
+    constexpr int RS = mma_sum_row(OC);
+    constexpr int kPacks = kRows * OC / 8;                   // 8-column pieces of the slice
+    constexpr int kGroups = kMmaWarps * 8;                   // groups of four threads
+    constexpr int kPer = (kPacks + kGroups - 1) / kGroups;   // pieces a group
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int d = a.d, L = a.L;
+    constexpr uint32_t RB = mma_row_bytes(OC), SB = mma_slice_bytes(OC), SS = mma_slice_step(OC);
+    const uint32_t xbuf = a.csize * SS;
+    uint8_t* xs = smem;                                      // [2][csize] slices
+    uint8_t* slice = smem + 2 * xbuf;                        // [2] this CTA's, as sent
+    float* sums = reinterpret_cast<float*>(slice + 2 * SB);  // [8 warps][16][RS]
+    // SPLIT: the partner warps' accumulators, [2][4 warps][NB][32 lanes]
+    float4* pacc = reinterpret_cast<float4*>(sums + kMmaWarps * kRows * RS);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(pacc + (SPLIT ? 2 * kPWarps * NB * 32 : 0));
+    uint64_t* const xs_bar = bars;                   // [2] layer input complete
+    uint64_t* const pfull = bars + 2;                // [2][4] accumulators handed over
+    uint64_t* const pfree = pfull + 2 * kPWarps;     // [2][4] ... and taken
+    __nv_bfloat16** outp = reinterpret_cast<__nv_bfloat16**>(bars + kMmaBars);
+    int* prow = reinterpret_cast<int*>(outp + kMaxDecodeLayers);
+    volatile int* abort = prow + kMaxDecodeLayers;
+    float* bias_s = const_cast<float*>(reinterpret_cast<volatile float*>(abort + 4));   // [L][OC]
+    const bool partner_warp = SPLIT && threadIdx.x >= kMmaWarps * 32;
+    const int warp = (threadIdx.x >> 5) - (partner_warp ? kMmaWarps : 0);
+    const int lane = threadIdx.x & 31;
+    const int q = (int)cluster_ctarank();
+    const int row0 = (int)(blockIdx.x / a.csize) * kRows;     // this cluster's row block
+    const int vr = a.B - row0 < kRows ? a.B - row0 : kRows;   // valid rows
+    const int col0 = q * OC, g = lane >> 2, c = lane & 3;
+
+    if (threadIdx.x < L) {
+        outp[threadIdx.x] = a.out[threadIdx.x];
+        prow[threadIdx.x] = a.prow[threadIdx.x];
+    }
+    if (threadIdx.x == 0) {
+        *abort = 0;
+        for (int i = 0; i < kMmaBars; ++i) mbar_init(&bars[i], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    cluster_sync_all();   // barriers initialised in every CTA of the cluster
+    // nothing above touched global memory: it overlaps the end of the kernel before
+    // this one (the position before, in a decode loop)
+    pdl_wait();
+    pdl_trigger();
+
+    for (int i = threadIdx.x; i < L * OC; i += mma_threads(OC))
+        bias_s[i] = a.bias ? a.bias[(size_t)(i / OC) * d + col0 + i % OC] : 0.f;
+    // K groups of this warp: [warp gw, warp gw + gw) clipped to d / 64
+    const int gw = partner_warp ? GP * kMmaWarps / kPWarps : GP;
+    const int k0 = warp * gw * 64 + 16 * c;   // the lane's features of group 0
+    const int ng = d / 64 - warp * gw;       // groups of this warp: min(ng, gw)
+    const size_t wlane = ((size_t)(col0 + g) * d + k0) * 2, wlayer = (size_t)d * d * 2;
+    const size_t ublk = (size_t)16 * d;      // bytes of 8 weight rows
+    const uint8_t* const ws = reinterpret_cast<const uint8_t*>(a.Ws) + wlane;
+    const uint8_t* const wn = reinterpret_cast<const uint8_t*>(a.Wn) + wlane;
+    float acc[NB][4];
+    auto load_group = [&](Feat16 (&w)[NB], const uint8_t* p, int i) {
+        if (i < ng) {
+#pragma unroll
+            for (int u = 0; u < NB; ++u) w[u] = ldg_stream<W32>(p + u * ublk + i * 128);
+        }
+    };
+    // partner rows g, g + 8 of layer l, group i
+    auto load_partner = [&](Feat16 (&xp)[2], int l, int i) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int row = g + 8 * h;
+            if (i < ng && row < vr)
+                xp[h] = ldg_stream<W32>(a.cache + (size_t)(prow[l] + row0 + row) * d + k0 + i * 64);
+            else
+                xp[h] = Feat16{};
+        }
+    };
+    // group i of a part: rows lo (g) and hi (g + 8) against w
+    auto contract = [&](const Feat16& lo, const Feat16& hi, const Feat16 (&w)[NB], int i) {
+        if (i < ng) {
+#pragma unroll
+            for (int m = 0; m < 8; m += 2) {
+                const uint32_t af[4] = {lo.r[m], hi.r[m], lo.r[m + 1], hi.r[m + 1]};
+#pragma unroll
+                for (int u = 0; u < NB; ++u) mma_16816(acc[u], af, w[u].r[m], w[u].r[m + 1]);
+            }
+        }
+    };
+    auto clear = [&]() {
+#pragma unroll
+        for (int u = 0; u < NB; ++u)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[u][e] = 0.f;
+    };
+    // every lane waits (each gets the acquire); the outcome is made warp-uniform so
+    // that the aligned MMAs never run divergent
+    bool ok = true;
+    auto wait = [&](uint64_t* bar, uint32_t parity, bool cluster) {
+        const bool r = ok && (cluster ? mbar_wait_cluster(bar, parity, abort, a.timeout_ns)
+                                      : mbar_wait(bar, parity, abort, a.timeout_ns));
+        ok = __all_sync(0xffffffffu, r);
+    };
+    auto next_recv = [&](int l) {   // the next layer from l on that has a partner part
+        while (l < L && prow[l] < 0) ++l;
+        return l;
+    };
+
+    if (partner_warp) {
+        constexpr int GW = GP * kMmaWarps / kPWarps;
+        Feat16 w[GW][NB], xp[GW][2];   // weights and rows of the next layer with a partner part
+        int l = next_recv(0);
+        if (l < L) {
+#pragma unroll
+            for (int i = 0; i < GW; ++i) {
+                load_group(w[i], wn + l * wlayer, i);
+                load_partner(xp[i], l, i);
+            }
+        }
+        __syncthreads();   // (x_t and the biases in place)
+        for (uint32_t use = 0; l < L; ++use) {
+            const int nl = next_recv(l + 1);
+            const uint32_t slot = (use & 1) * kPWarps + warp;
+            clear();
+#pragma unroll
+            for (int i = 0; i < GW; ++i) {
+                contract(xp[i][0], xp[i][1], w[i], i);
+                if (nl < L) {
+                    load_group(w[i], wn + nl * wlayer, i);
+                    load_partner(xp[i], nl, i);
+                }
+            }
+            if (use >= 2) wait(&pfree[slot], ((use >> 1) - 1) & 1, false);
+            float4* dst = pacc + (size_t)slot * NB * 32 + lane;
+#pragma unroll
+            for (int u = 0; u < NB; ++u)
+                dst[u * 32] = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&pfull[slot]);
+            l = nl;
+        }
+    } else {
+        // weights of the part contracted next, and (SPLIT) of the layer after
+        Feat16 w[GP][NB], w2[SPLIT ? GP : 1][NB], xp[GP][2];
+        // the first part this warp contracts of layer l
+        auto first_part = [&](int l) {
+            return (!SPLIT && prow[l] >= 0 ? wn : ws) + l * wlayer;
+        };
+#pragma unroll
+        for (int i = 0; i < GP; ++i) {
+            if (SPLIT)
+                load_group(w2[i], ws, i);
+            else
+                load_group(w[i], first_part(0), i);
+            if (!SPLIT && prow[0] >= 0) load_partner(xp[i], 0, i);
+        }
+        // x_t, layer 0's input
+        for (int p = threadIdx.x; p < kRows * (d / 8); p += kMmaWarps * 32) {
+            const int row = p / (d / 8), pc = p - row * (d / 8);
+            uint4 v = make_uint4(0, 0, 0, 0);
+            if (row < vr)
+                v = *reinterpret_cast<const uint4*>(a.x + (size_t)(row0 + row) * d + pc * 8);
+            *reinterpret_cast<uint4*>(xs + pc / NB * SS + row * RB + pc % NB * 16) = v;
+        }
+        // epilogue: thread c of a group of four has columns 2 c, 2 c + 1 of the group's
+        // pieces; lanes 0 and 1 of warp w send the slice to CTAs w and w + 8 of the cluster
+        const int group = threadIdx.x >> 2;
+        const int to = warp + kMmaWarps * lane;
+        const bool sends = lane < 2 && to < a.csize;
+        // shared::cluster offset from this CTA to that one
+        const uint32_t peer = sends ? mapa_shared(smem, to) - smem_u32(smem) : 0u;
+        // every piece of a group has the same columns: kGroups is a multiple of NB
+        const int ecol = (group % NB) * 8;
+        const float* const bias = bias_s + ecol + 2 * c;
+        float* const mine = sums + warp * (kRows * RS) + g * RS + 2 * c;
+        const uint8_t* const xa = xs + k0 / OC * SS + g * RB + k0 % OC * 2;
+        const bool relu = (a.flags & 4u) != 0, residual = (a.flags & 2u) != 0;
+        uint32_t use = 0;
+        __syncthreads();   // x_t and the biases in place
+
+        for (int l = 0; l < L; ++l) {
+            const uint32_t xb = l & 1;
+            const bool recv = prow[l] >= 0;
+            // the next layer's input arrives as a slice from every CTA of the cluster
+            if (threadIdx.x == 0 && l + 1 < L)
+                mbar_arrive_expect_tx(&xs_bar[xb ^ 1], a.csize * SB);
+            const float2 bv = *reinterpret_cast<const float2*>(bias + l * OC);
+            if (SPLIT) {
+#pragma unroll
+                for (int i = 0; i < GP; ++i) {
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) w[i][u] = w2[i][u];
+                    if (l + 1 < L) load_group(w2[i], ws + (l + 1) * wlayer, i);
+                }
+            }
+            if (SPLIT && recv && warp < kPWarps) {
+                const uint32_t slot = (use & 1) * kPWarps + warp;
+                wait(&pfull[slot], (use >> 1) & 1, false);
+                const float4* src = pacc + (size_t)slot * NB * 32 + lane;
+#pragma unroll
+                for (int u = 0; u < NB; ++u) {
+                    const float4 t = src[u * 32];
+                    acc[u][0] = t.x;
+                    acc[u][1] = t.y;
+                    acc[u][2] = t.z;
+                    acc[u][3] = t.w;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&pfree[slot]);
+                ++use;
+            } else {
+                clear();
+            }
+            if (!SPLIT) {
+                if (recv) {
+#pragma unroll
+                    for (int i = 0; i < GP; ++i) {
+                        contract(xp[i][0], xp[i][1], w[i], i);
+                        load_group(w[i], ws + l * wlayer, i);
+                    }
+                }
+                if (l + 1 < L && prow[l + 1] >= 0) {
+#pragma unroll
+                    for (int i = 0; i < GP; ++i) load_partner(xp[i], l + 1, i);
+                }
+            }
+            const uint8_t* xl = xa + xb * xbuf;
+            if (l > 0) wait(&xs_bar[xb], ((l - 1) >> 1) & 1, true);
+#pragma unroll
+            for (int i = 0; i < GP; ++i)
+                if (i < ng) {
+                    const uint8_t* xg = xl + i * (64 / OC * SS);
+                    contract(lds16(xg), lds16(xg + 8 * RB), w[i], i);
+                    if (!SPLIT && l + 1 < L) load_group(w[i], first_part(l + 1), i);
+                }
+            // A warp writes its block of sums again only once the next layer's input is
+            // complete, which this CTA has sent after every thread's reads.
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+                *reinterpret_cast<float2*>(mine + u * 8) = make_float2(acc[u][0], acc[u][1]);
+                *reinterpret_cast<float2*>(mine + 8 * RS + u * 8) =
+                    make_float2(acc[u][2], acc[u][3]);
+            }
+            named_bar_sync(1, kMmaWarps * 32);
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                const int pk = group + i * kGroups;
+                if (pk >= kPacks) break;   // warp-uniform
+                const int row = pk / NB;
+                const float* sum = sums + row * RS + ecol + 2 * c;
+                float2 p[kMmaWarps];
+#pragma unroll
+                for (int k = 0; k < kMmaWarps; ++k)
+                    p[k] = *reinterpret_cast<const float2*>(sum + k * (kRows * RS));
+                const uint32_t off = row * RB + ecol * 2;   // the piece in a slice
+                const uint32_t xin =
+                    *reinterpret_cast<const uint32_t*>(xs + xb * xbuf + q * SS + off + 4 * c);
+                float2 v = p[0];
+#pragma unroll
+                for (int k = 1; k < kMmaWarps; ++k) {
+                    v.x += p[k].x;
+                    v.y += p[k].y;
+                }
+                v.x += bv.x;
+                v.y += bv.y;
+                if (relu) {
+                    v.x = v.x > 0.f ? v.x : 0.f;
+                    v.y = v.y > 0.f ? v.y : 0.f;
+                }
+                if (residual) {
+                    const float2 f = unpack_bf16x2(xin);
+                    v.x += f.x;
+                    v.y += f.y;
+                }
+                const uint32_t out = pack_bf16x2(v.x, v.y);
+                uint4 p4;
+                p4.x = __shfl_sync(0xffffffffu, out, 0, 4);
+                p4.y = __shfl_sync(0xffffffffu, out, 1, 4);
+                p4.z = __shfl_sync(0xffffffffu, out, 2, 4);
+                p4.w = __shfl_sync(0xffffffffu, out, 3, 4);
+                if (c == 0) *reinterpret_cast<uint4*>(slice + (xb ^ 1) * SB + off) = p4;
+                if (row < vr) {
+                    const size_t at = (size_t)(row0 + row) * d + col0 + ecol;
+                    if (l == 0)   // position t's layer-0 input into layer 0's ring
+                        *reinterpret_cast<uint32_t*>(a.ring0 + at + 2 * c) = xin;
+                    if (c == 0) *reinterpret_cast<uint4*>(outp[l] + at) = p4;
+                }
+            }
+            if (l + 1 < L) {
+                // the slice to every CTA of the cluster, this one included.  (Its buffer is
+                // free: the copies of two layers ago were part of inputs since used.)
+                fence_proxy_async_smem();
+                named_bar_sync(1, kMmaWarps * 32);
+                if (ok && sends)
+                    copy_to_peer(smem_u32(xs) + (xb ^ 1) * xbuf + q * SS + peer,
+                                 smem_u32(slice) + (xb ^ 1) * SB, SB,
+                                 smem_u32(xs_bar) + 8 * (xb ^ 1) + peer);
+                __syncwarp();
+            }
+        }
+    }
+    // Normally every copy has been waited for as part of an input.  After an abort the
+    // ones in flight, from and to this CTA, get ample time to land before it leaves.
+    auto settle = [&]() {
+        if (*abort)
+            for (const uint64_t t0 = globaltimer_ns(); globaltimer_ns() - t0 < 100000;) {
+            }
+    };
+    settle();
+    __syncwarp();
+    cluster_sync_all();   // no CTA leaves while a peer may still write its shared memory
+    settle();
+}
+
+size_t decode_mma_smem(int d, int oc, int L) {
+    return (size_t)2 * (d / oc) * mma_slice_step(oc) + 2 * mma_slice_bytes(oc) +
+           (size_t)kMmaWarps * kRows * mma_sum_row(oc) * 4 +
+           (mma_split(oc) ? (size_t)2 * kPWarps * kRows * oc * 4 : 0) + kMmaBars * 8 +
+           kMaxDecodeLayers * 12 + 16 + (size_t)L * oc * 4;
 }
 
 }  // namespace
@@ -618,49 +914,87 @@ size_t decode_smem_bytes(const DecodeGeo& g) {
            (size_t)2 * kRows * g.oc * 4 + B_COUNT * 8 + 16;
 }
 
-cudaError_t launch_decode(const DecodeLaunch& p, cudaStream_t st) {
-    if (p.L < 1 || p.L > kMaxDecodeLayers) return cudaErrorInvalidValue;
-    DecodeArgs a;
-    a.mWs = p.mWs;
-    a.mWn = p.mWn;
-    a.mCache = p.mCache;
-    a.mX = p.mX;
-    for (int l = 0; l < p.L; ++l) {
-        a.prow[l] = p.prow[l];
-        a.out[l] = p.out[l];
-    }
-    a.bias = p.bias;
-    a.ring0 = p.ring0;
-    a.g = p.g;
-    a.L = p.L;
-    a.B = p.B;
-    a.flags = p.flags;
-    a.timeout_ns = p.timeout_ns;
-    const size_t smem = decode_smem_bytes(p.g);
-    auto kern = p.tc ? decode_kernel<true> : decode_kernel<false>;
+// Clusters of csize CTAs, one per 16 rows; pdl: as a programmatic dependent.
+template <typename Args>
+static cudaError_t launch_clusters(void (*kern)(Args), const Args& a, int threads, size_t smem,
+                                   bool pdl, cudaStream_t st, int csize) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
-    if (e == cudaSuccess && p.g.csize > 8)
+    if (e == cudaSuccess && csize > 8)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    const int blocks = (p.B + kRows - 1) / kRows;
+    const int blocks = (a.B + kRows - 1) / kRows;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(blocks * p.g.csize));
-    cfg.blockDim = dim3(kThreads);
+    cfg.gridDim = dim3((unsigned)(blocks * csize));
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)p.g.csize;
+    attr[0].val.clusterDim.x = (unsigned)csize;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int clusters = 0;
     e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
     if (e != cudaSuccess) return e;
     if (clusters < 1) return cudaErrorInvalidConfiguration;
+    cfg.numAttrs = pdl ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+cudaError_t launch_decode(const DecodeLaunch& p, cudaStream_t st) {
+    if (p.L < 1 || p.L > kMaxDecodeLayers) return cudaErrorInvalidValue;
+    if (p.tc) {
+        DecodeArgs a;
+        a.mWs = p.mWs;
+        a.mWn = p.mWn;
+        a.mCache = p.mCache;
+        a.mX = p.mX;
+        for (int l = 0; l < p.L; ++l) {
+            a.prow[l] = p.prow[l];
+            a.out[l] = p.out[l];
+        }
+        a.bias = p.bias;
+        a.ring0 = p.ring0;
+        a.g = p.g;
+        a.L = p.L;
+        a.B = p.B;
+        a.flags = p.flags;
+        a.timeout_ns = p.timeout_ns;
+        return launch_clusters(decode_tc_kernel, a, kThreads, decode_smem_bytes(p.g), false, st,
+                               p.g.csize);
+    }
+    DecodeMmaArgs a;
+    a.Ws = p.Ws;
+    a.Wn = p.Wn;
+    a.x = p.x;
+    a.cache = p.cache;
+    a.bias = p.bias;
+    a.ring0 = p.ring0;
+    for (int l = 0; l < p.L; ++l) {
+        a.prow[l] = p.prow[l];
+        a.out[l] = p.out[l];
+    }
+    a.d = p.g.d;
+    a.csize = p.g.csize;
+    a.L = p.L;
+    a.B = p.B;
+    a.flags = p.flags;
+    a.timeout_ns = p.timeout_ns;
+    // K groups of 64 features a warp: OC = 16 up to d = 256, 32 up to 512, then 64
+    const bool w32 = ((reinterpret_cast<uintptr_t>(p.Ws) | reinterpret_cast<uintptr_t>(p.Wn) |
+                       reinterpret_cast<uintptr_t>(p.cache)) & 31) == 0;
+    auto kern = p.g.oc == 16
+                    ? (w32 ? decode_mma_kernel<16, 1, true> : decode_mma_kernel<16, 1, false>)
+                : p.g.oc == 32
+                    ? (w32 ? decode_mma_kernel<32, 1, true> : decode_mma_kernel<32, 1, false>)
+                    : (w32 ? decode_mma_kernel<64, 2, true> : decode_mma_kernel<64, 2, false>);
+    return launch_clusters(kern, a, mma_threads(p.g.oc), decode_mma_smem(p.g.d, p.g.oc, p.L), true, st,
+                           p.g.csize);
 }
 
 cudaError_t decode_error_word_read_clear(int* word) {

@@ -232,9 +232,10 @@ size_t decode_smem_bytes(const DecodeGeo& g);
 // x_t is also copied to ring0.  Maps (128-byte swizzle, matrices viewed as
 // (64 features, rows, 64-feature tiles)): mWs / mWn over [L d][d] with box
 // (64, oc, kc / 64), mCache over the rings as [rows][d] and mX over x_t [B][d]
-// with box (64, 16, d / 64).
+// with box (64, 16, d / 64); the maps are set and used only with tc.
 struct DecodeLaunch {
     CUtensorMap mWs, mWn, mCache, mX;
+    const __nv_bfloat16 *Ws, *Wn, *x, *cache;
     int prow[kMaxDecodeLayers];
     __nv_bfloat16* out[kMaxDecodeLayers];
     const float* bias;

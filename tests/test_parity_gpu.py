@@ -552,6 +552,41 @@ def test_decode_steps_reproduce_the_window_forward(H, case, decode_kernel):
     assert rel(host(ys), host(y)) <= TOL_BF16, name
 
 
+@pytest.mark.parametrize("B, d, L", [(5, 320, 4), (18, 576, 3), (2, 64, 5)])
+def test_decode_operands_at_16_byte_alignment(H, B, d, L):
+    """Weights and rings at the 16-byte alignment the ABI asks for (the decode loads
+    32-byte aligned ones in wider pieces) give the same bits, equal to the window
+    forward at the bf16 tolerance; clusters of 10, 9 and 4 CTAs with K groups that do not
+    go round the warps."""
+    n, flags = 16, CAUSAL | RESIDUAL | RELU
+    pr = synth.problem(B, n, d, L=L, seed=37, w_std=(1 / (2 * d)) ** 0.5)
+    x, _ = dev(pr.x, torch.bfloat16)
+    Ws, _ = dev(pr.W_self, torch.bfloat16)
+    Wn, _ = dev(pr.W_nbr, torch.bfloat16)
+    bias = torch.from_numpy(pr.bias).cuda()
+    nb = H.hcw_decode_cache_bytes(L, B, n, d)
+
+    def at_16(t):
+        buf = torch.empty(t.numel() + 8, dtype=t.dtype, device="cuda")
+        buf[8:].copy_(t.flatten())
+        out = buf[8:].view(t.shape)
+        assert out.data_ptr() % 32 == 16
+        return out
+
+    def window(Ws, Wn, cache):
+        ys = [H.hcw_decode_step(x[:, t].contiguous(), Ws, Wn, bias, t, n, cache, flags)
+              for t in range(n)]
+        return torch.stack(ys, 1)
+
+    a = window(Ws, Wn, torch.empty(nb, dtype=torch.uint8, device="cuda"))
+    for args in ((at_16(Ws), Wn, torch.empty(nb, dtype=torch.uint8, device="cuda")),
+                 (Ws, Wn, torch.empty(nb + 16, dtype=torch.uint8, device="cuda")[16:])):
+        assert torch.equal(window(*args), a)
+    assert H.hcw_sync_status() == H.HCW_OK
+    y, _, _ = H.hcw_stack_fwd(x, Ws, Wn, bias, 0, -1, flags)
+    assert rel(host(a), host(y)) <= TOL_BF16
+
+
 def test_decode_full_size_window(H, decode_kernel):
     """The decode shape bench.py times (64 sequences, window 256, d = 512, 16
     rotated causal layers): every position of every sequence equals the
