@@ -45,6 +45,8 @@
 //     remote stores are generic writes that the MMA reads through the async
 //     proxy) add to the chain.  So the tensor-core version is the slower of the
 //     two here.
+#include <atomic>
+
 #include "hcw_internal.h"
 #include "hcw_ptx.cuh"
 
@@ -914,15 +916,32 @@ size_t decode_smem_bytes(const DecodeGeo& g) {
            (size_t)2 * kRows * g.oc * 4 + B_COUNT * 8 + 16;
 }
 
-// Clusters of csize CTAs, one per 16 rows; pdl: as a programmatic dependent.
+// Clusters of csize CTAs, one per 16 rows; pdl: as a programmatic dependent.  The
+// kernel's attributes are set once per device and a cluster that does not fit is the
+// launch's own error: with two attributes and an occupancy query a call, windows of
+// short steps were bound by the host (32 positions of 22 layers at d = 64: 614 us, 583
+// without; 256 of 16 layers at d = 512: 5,993 us, 5,860).
 template <typename Args>
-static cudaError_t launch_clusters(void (*kern)(Args), const Args& a, int threads, size_t smem,
-                                   bool pdl, cudaStream_t st, int csize) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e == cudaSuccess && csize > 8)
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+using ClusterKernel = void (*)(Args);
+template <typename Args, ClusterKernel<Args> kern>
+static cudaError_t launch_clusters(const Args& a, int threads, size_t smem, bool pdl,
+                                   cudaStream_t st, int csize) {
+    static std::atomic<bool> configured[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    auto configure = [&]() {
+        int most = 0;
+        cudaError_t r = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (r == cudaSuccess)
+            r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (r == cudaSuccess)
+            r = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (r == cudaSuccess && dev < 64) configured[dev].store(true, std::memory_order_release);
+        return r;
+    };
+    const bool cached = dev < 64 && configured[dev].load(std::memory_order_acquire);
+    if (!cached && (e = configure()) != cudaSuccess) return e;
     const int blocks = (a.B + kRows - 1) / kRows;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(blocks * csize));
@@ -937,13 +956,13 @@ static cudaError_t launch_clusters(void (*kern)(Args), const Args& a, int thread
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (clusters < 1) return cudaErrorInvalidConfiguration;
     cfg.numAttrs = pdl ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kern, a);
+    e = cudaLaunchKernelEx(&cfg, kern, a);
+    if (e == cudaSuccess || !cached) return e;
+    // the attributes do not outlive a device reset: set them again, once
+    cudaGetLastError();
+    e = configure();
+    return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, kern, a) : e;
 }
 
 cudaError_t launch_decode(const DecodeLaunch& p, cudaStream_t st) {
@@ -965,8 +984,8 @@ cudaError_t launch_decode(const DecodeLaunch& p, cudaStream_t st) {
         a.B = p.B;
         a.flags = p.flags;
         a.timeout_ns = p.timeout_ns;
-        return launch_clusters(decode_tc_kernel, a, kThreads, decode_smem_bytes(p.g), false, st,
-                               p.g.csize);
+        return launch_clusters<DecodeArgs, decode_tc_kernel>(a, kThreads, decode_smem_bytes(p.g),
+                                                             false, st, p.g.csize);
     }
     DecodeMmaArgs a;
     a.Ws = p.Ws;
@@ -988,13 +1007,15 @@ cudaError_t launch_decode(const DecodeLaunch& p, cudaStream_t st) {
     // K groups of 64 features a warp: OC = 16 up to d = 256, 32 up to 512, then 64
     const bool w32 = ((reinterpret_cast<uintptr_t>(p.Ws) | reinterpret_cast<uintptr_t>(p.Wn) |
                        reinterpret_cast<uintptr_t>(p.cache)) & 31) == 0;
-    auto kern = p.g.oc == 16
-                    ? (w32 ? decode_mma_kernel<16, 1, true> : decode_mma_kernel<16, 1, false>)
-                : p.g.oc == 32
-                    ? (w32 ? decode_mma_kernel<32, 1, true> : decode_mma_kernel<32, 1, false>)
-                    : (w32 ? decode_mma_kernel<64, 2, true> : decode_mma_kernel<64, 2, false>);
-    return launch_clusters(kern, a, mma_threads(p.g.oc), decode_mma_smem(p.g.d, p.g.oc, p.L), true, st,
-                           p.g.csize);
+    auto launch =
+        p.g.oc == 16 ? (w32 ? launch_clusters<DecodeMmaArgs, decode_mma_kernel<16, 1, true>>
+                            : launch_clusters<DecodeMmaArgs, decode_mma_kernel<16, 1, false>>)
+        : p.g.oc == 32 ? (w32 ? launch_clusters<DecodeMmaArgs, decode_mma_kernel<32, 1, true>>
+                              : launch_clusters<DecodeMmaArgs, decode_mma_kernel<32, 1, false>>)
+                       : (w32 ? launch_clusters<DecodeMmaArgs, decode_mma_kernel<64, 2, true>>
+                              : launch_clusters<DecodeMmaArgs, decode_mma_kernel<64, 2, false>>);
+    return launch(a, mma_threads(p.g.oc), decode_mma_smem(p.g.d, p.g.oc, p.L), true, st,
+                  p.g.csize);
 }
 
 cudaError_t decode_error_word_read_clear(int* word) {

@@ -116,6 +116,8 @@ class HcwError(RuntimeError):
 def lib() -> ctypes.CDLL:
     """Load libhcw.so (built in-tree by build()); raise if it is missing."""
     global _lib
+    if _lib is not None:   # set once, under the lock, when complete
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -141,13 +143,13 @@ def _check(rc: int, what: str):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
     if stream is None:
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 def _dtype_code(t: torch.Tensor) -> int:
