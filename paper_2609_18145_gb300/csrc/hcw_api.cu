@@ -487,8 +487,25 @@ size_t stack_counter_bytes(long long tokens, int L) {
 // (tcgen05 cta_group::2, 256-row tiles): 256-column tiles and at least two
 // row blocks.  Each SM of a pair loads its own rows and half of the weight
 // tile per stage.
-bool use_pairs(const Shape& sh) {
-    return pick_bn(sh.d) == 256 && sh.tokens / 2 > 128;
+bool use_pairs(const Shape& sh, int BN) { return BN == 256 && sh.tokens / 2 > 128; }
+
+// Column tile of a stacked forward / input-gradient launch.  With few tokens the
+// launch is the layer chain, not throughput: a unit's operands come at what one SM
+// takes in, so narrower tiles, spread over more SMs, shorten every step (each output
+// element sums the same products in the same order).  64 columns while every unit of
+// a layer has an SM of its own, 128 up to 1.75 waves, else 256 on pairs.  Microseconds a
+// layer of an 8-layer causal stack, forward / input gradient, at 64 | 128 | 256 columns:
+//   d = 256:  2048 tokens  6.3/6.8 | 6.9/7.3 | 8.6/8.9;   16384  12.2/13.9 | 8.6/9.7 | 9.6/9.9
+//   d = 512:   256 tokens  8.2/9.3 | 8.8/9.6 | 11.1/11.6;  2048  8.5/9.6 | 9.1/10.0 | 11.0/11.5
+//             4096 tokens  9.8/10.9 | 9.3/10.8 | 11.2/11.9;  8192  17.0/18.5 | 11.1/12.2 | 11.9/13.1
+//            16384 tokens  32.5/34.2 | 19.6/21.1 | 14.3/15.3
+//   d = 1024: 1024 tokens  12.8/15.1 | 13.6/15.0 | 15.5/16.5;  4096  27.3/29.8 | 16.8/18.3 | 17.0/18.3
+int stack_bn(const Shape& sh) {
+    const long long row_units = 2 * ((sh.tokens / 2 + 127) / 128);
+    const int sms = sm_count();
+    if (row_units * (sh.d / 64) <= sms) return 64;
+    if (sh.d % 128 == 0 && 4 * row_units * (sh.d / 128) <= 7ll * sms) return 128;
+    return pick_bn(sh.d);
 }
 
 // Whether a bf16 stacked forward / input gradient runs on the resident
@@ -526,9 +543,9 @@ template <class In, class Out, class Mask>
 int stack_fwd_group(const Shape& sh, int l0, int n, const Sched& sc,
                     const uint8_t* Ws, const uint8_t* Wn, const float* bias, unsigned flags,
                     In in_ptr, Out out_ptr, Mask mask_ptr, int* counters, cudaStream_t st) {
-    const int d = sh.d, BN = pick_bn(d);
+    const int d = sh.d, BN = stack_bn(sh);
     const size_t wb = (size_t)d * d * 2;
-    const bool pair = use_pairs(sh);
+    const bool pair = use_pairs(sh, BN);
     static thread_local TcLaunch<kMaxStackLayers> L;
     memset(&L, 0, sizeof(L));
     for (int i = 0; i < n; ++i) {
@@ -536,7 +553,7 @@ int stack_fwd_group(const Shape& sh, int l0, int n, const Sched& sc,
         const int sl = sc.dim(sh, l);
         // a shift layer: rows in runs of 128 positions, its input as positions
         const int s = sl >= 0 ? sl : kShiftStackDim;
-        if (!fwd_maps(L.maps[i], sh, s, in_ptr(l), Ws + l * wb, Wn + l * wb, out_ptr(l), pair) ||
+        if (!fwd_maps(L.maps[i], sh, s, in_ptr(l), Ws + l * wb, Wn + l * wb, out_ptr(l), pair, BN) ||
             (sl < 0 && !map_positions(&L.maps[i][0], in_ptr(l), sh.tokens, sh.n, d, 128)))
             return HCW_ERR_CUDA;
         L.layer[i] = {s, 1 << s, bias ? bias + (size_t)l * d : nullptr, mask_ptr(l), nullptr,
@@ -1052,7 +1069,7 @@ int stack_data_bf16(const Shape& sh, const StackData& a, cudaStream_t st) {
     if (a.sc.has_shift(a.L) && (!shift_stackable(sh) || use_resident(sh)))
         return stack_data_layers_bf16(sh, a, st);
     if (use_resident(sh)) return stack_data_resident(sh, a, st);
-    const int d = sh.d, BN = pick_bn(d), L = a.L;
+    const int d = sh.d, BN = stack_bn(sh), L = a.L;
     const bool relu = (a.flags & HCW_ACT_RELU) != 0;
     const bool resid = (a.flags & HCW_RESIDUAL) != 0;
     const bool keep_g = relu && resid;
@@ -1077,7 +1094,7 @@ int stack_data_bf16(const Shape& sh, const StackData& a, cudaStream_t st) {
     // the top layer's dz = dy * act'(z) is written by the first launch itself
     int* counters = reinterpret_cast<int*>(a.ws + stack_g_region(sh, a.flags, L));
     const int n_chunks = (int)((sh.tokens + 127) / 128);
-    const bool pair = use_pairs(sh);
+    const bool pair = use_pairs(sh, BN);
     const int pw = epi_patch_cols(BN);
     static thread_local TcLaunch<kMaxStackLayers> T;
     for (int top = L - 1; top >= 0; top -= kMaxStackLayers) {
@@ -1670,7 +1687,7 @@ size_t step_counter_bytes(long long tokens, int L) {
 bool step_fused(const Shape& sh, int dtype, const Sched& sc, int L) {
     // 256- or 128-column tiles on pairs (d = 128 takes the latter), at least
     // two row blocks
-    const bool pairs = use_pairs(sh) || (pick_bn(sh.d) == 128 && sh.tokens / 2 > 128);
+    const bool pairs = use_pairs(sh, pick_bn(sh.d)) || (pick_bn(sh.d) == 128 && sh.tokens / 2 > 128);
     return dtype == HCW_BF16 && (!sc.has_shift(L) || shift_stackable(sh)) && !use_resident(sh) &&
            pairs && L <= kMaxStackLayers && sh.tokens > 0;
 }
