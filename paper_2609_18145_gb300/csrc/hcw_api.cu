@@ -210,6 +210,21 @@ bool map_tiles_sw128(CUtensorMap* m, const void* base, long long rows, int d, in
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// bf16 [layers][tokens][d] as (features, tokens, layers), box (64, 128, 1), 128-byte
+// swizzle: 128 tokens' 64-feature tiles of one layer, clipped at the tokens.
+bool map_layers(CUtensorMap* m, const void* base, long long tokens, int d, int layers) {
+    EncodeTiledFn enc = encode_fn();
+    if (!enc || !base) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)tokens, (cuuint64_t)layers};
+    cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)tokens * d * 2};
+    cuuint32_t box[3] = {64, 128, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
+               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // fp32 matrix [rows][d], box (32 columns, 32 rows), 128-byte swizzle: the
 // patches the weight-gradient epilogue stores.
 bool map_f32_patches(CUtensorMap* m, const void* base, long long rows, int d) {
@@ -520,6 +535,42 @@ bool use_resident(const Shape& sh) {
     // measured on GB300 (char-LM shapes, d = 512): the streaming kernels are
     // faster, so they are the automatic choice
     return mode == HCW_STACK_RESIDENT;
+}
+
+// Whether a bf16 stack runs on the kernel that keeps 128 tokens on chip through all
+// layers (hcw_small.cu): narrow layers, short windows, no kernel family asked for.
+bool use_small(const Shape& sh, int L) {
+    return g_stack_kernels.load(std::memory_order_relaxed) == HCW_STACK_AUTO &&
+           small_supported(sh.d, sh.n, sh.tokens, L);
+}
+
+// The forward (y given) and / or the input gradient (dx given) of a stack there.
+int small_launch(const Shape& sh, const Sched& sc, int L, unsigned flags, const void* x,
+                 const void* Ws, const void* Wn, const float* bias, void* y, void* acts,
+                 void* masks, const void* dy, void* dx, void* dz, cudaStream_t st) {
+    const int d = sh.d;
+    SmallLaunch S;
+    memset(&S, 0, sizeof(S));
+    if (!map_tiles_sw128(&S.mWs, Ws, (long long)L * d, d, d, d / 64) ||
+        !map_tiles_sw128(&S.mWn, Wn, (long long)L * d, d, d, d / 64) ||
+        (y && L > 1 && !map_layers(&S.mActs, acts, sh.tokens, d, L - 1)) ||
+        (dx && !map_layers(&S.mDz, dz, sh.tokens, d, L)))
+        return HCW_ERR_CUDA;
+    S.x = static_cast<const __nv_bfloat16*>(x);
+    S.dy = static_cast<const __nv_bfloat16*>(dy);
+    S.bias = bias;
+    S.y = static_cast<__nv_bfloat16*>(y);
+    S.dx = static_cast<__nv_bfloat16*>(dx);
+    S.masks = static_cast<uint32_t*>(masks);
+    for (int l = 0; l < L; ++l) S.link[l] = sc.dim(sh, l);
+    S.n_layers = L;
+    S.n = sh.n;
+    S.tokens = (int)sh.tokens;
+    S.fwd = y != nullptr;
+    S.bwd = dx != nullptr;
+    S.flags = flags;
+    S.timeout_ns = g_timeout_ns;
+    return launched(launch_small(S, d, sm_count(), st), 1);
 }
 
 // Row-unit geometry of a pair launch: units count row-block pairs.
@@ -1066,6 +1117,9 @@ int stack_data_layers_bf16(const Shape& sh, const StackData& a, cudaStream_t st)
 }
 
 int stack_data_bf16(const Shape& sh, const StackData& a, cudaStream_t st) {
+    if (use_small(sh, a.L))
+        return small_launch(sh, a.sc, a.L, a.flags, nullptr, a.Ws, a.Wn, nullptr, nullptr, nullptr,
+                            const_cast<void*>(a.masks), a.dy, a.dx, a.dz, st);
     if (a.sc.has_shift(a.L) && (!shift_stackable(sh) || use_resident(sh)))
         return stack_data_layers_bf16(sh, a, st);
     if (use_resident(sh)) return stack_data_resident(sh, a, st);
@@ -1574,6 +1628,9 @@ int stack_fwd_impl(const Shape& sh, const void* x, const void* W_self, const voi
         return want_mask ? reinterpret_cast<uint32_t*>(static_cast<uint8_t*>(masks) + (size_t)l * mb)
                          : nullptr;
     };
+    if (dtype == HCW_BF16 && use_small(sh, L))
+        return small_launch(sh, sc, L, flags, x, W_self, W_nbr, bias, y, acts,
+                            want_mask ? masks : nullptr, nullptr, nullptr, nullptr, st);
     if (dtype == HCW_BF16 && sc.has_shift(L) && (!shift_stackable(sh) || use_resident(sh))) {
         // layer by layer; a shift layer reads its partner rows S_k x, materialised
         // row-aligned behind the counters of the workspace
@@ -1878,13 +1935,18 @@ int train_step_impl(const Shape& sh, const void* x, const void* W_self, const vo
         overlaps(dx, ab, dbias, dbias ? (size_t)L * d * 4 : 0) ||
         overlaps(dy, ab, y, ab) || overlaps(dy, ab, acts, acts_b) || overlaps(dy, ab, masks, m_b))
         return HCW_ERR_ALIASING;
-    rc = step_fused_launch(sh, x, static_cast<const uint8_t*>(W_self),
-                           static_cast<const uint8_t*>(W_nbr), bias, dy, sc, L, flags, y, acts,
-                           masks, dx, ws, ws + zb, reinterpret_cast<int*>(ws + bwd), st,
-                           want_dw ? dw_early_pairs(sh, flags, L) : 0);
+    const bool small = use_small(sh, L);
+    if (small)
+        rc = small_launch(sh, sc, L, flags, x, W_self, W_nbr, bias, y, acts,
+                          (flags & HCW_ACT_RELU) ? masks : nullptr, dy, dx, ws, st);
+    else
+        rc = step_fused_launch(sh, x, static_cast<const uint8_t*>(W_self),
+                               static_cast<const uint8_t*>(W_nbr), bias, dy, sc, L, flags, y, acts,
+                               masks, dx, ws, ws + zb, reinterpret_cast<int*>(ws + bwd), st,
+                               want_dw ? dw_early_pairs(sh, flags, L) : 0);
     if (rc || !want_dw) return rc;
     StackWeight wa{x, acts, ws, sc, L, flags, dW_self, dW_nbr, dbias, ws + zb + db,
-                   reinterpret_cast<const int*>(ws + bwd)};
+                   small ? nullptr : reinterpret_cast<const int*>(ws + bwd)};
     return stack_weight_bf16(sh, wa, st);
 }
 
@@ -2336,8 +2398,9 @@ unsigned long long hcw_launch_count(void) { return g_launches.load(); }
 
 int hcw_sync_status(void* stream) {
     if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return HCW_ERR_CUDA;
-    int word = 0, word_res = 0, word_dec = 0, word_blk = 0, word_gemm = 0;
+    int word = 0, word_res = 0, word_dec = 0, word_blk = 0, word_gemm = 0, word_small = 0;
     if (error_word_read_clear(&word) != cudaSuccess ||
+        small_error_word_read_clear(&word_small) != cudaSuccess ||
         res_error_word_read_clear(&word_res) != cudaSuccess ||
         decode_error_word_read_clear(&word_dec) != cudaSuccess ||
         block_error_word_read_clear(&word_blk) != cudaSuccess ||
@@ -2347,6 +2410,7 @@ int hcw_sync_status(void* stream) {
     if (!word) word = word_dec;
     if (!word) word = word_blk;
     if (!word) word = word_gemm;
+    if (!word) word = word_small;
     if (word == HCW_ERR_INVALID_ARG) return HCW_ERR_INVALID_ARG;
     if (word) return word == HCW_ERR_TIMEOUT ? HCW_ERR_TIMEOUT : HCW_ERR_CUDA;
     return HCW_OK;

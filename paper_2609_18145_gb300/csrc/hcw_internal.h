@@ -215,6 +215,31 @@ cudaError_t launch_res(int mode, const ResLaunch& L, cudaStream_t stream);
 // Read the resident kernels' error word and reset it to 0 (synchronous).
 cudaError_t res_error_word_read_clear(int* word);
 
+// ---- Stacks of narrow layers over short windows (hcw_small.cu) ----
+constexpr int kMaxSmallLayers = 64;   // layers of one launch
+// The forward (fwd) and / or the input gradient (bwd) of a whole bf16 stack, d = 64 or
+// 128, n <= 128: acts and masks as hcw_stack_fwd writes them (masks may be null), dz and
+// dx as hcw_stack_bwd_data does; a backward alone reads masks (ReLU).  Maps, all 128-byte
+// swizzle: weights [L d][d] as 64-feature tiles, box (64, d, d / 64); acts and dz as
+// (features, tokens, layers), box (64, 128, 1).
+struct SmallLaunch {
+    CUtensorMap mWs, mWn, mActs, mDz;
+    const __nv_bfloat16* x;
+    const __nv_bfloat16* dy;
+    const float* bias;   // [L][d] or null
+    __nv_bfloat16* y;
+    __nv_bfloat16* dx;
+    uint32_t* masks;     // [L][tokens][d / 32]
+    int link[kMaxSmallLayers];
+    int n_layers, n, tokens, fwd, bwd;
+    unsigned flags;
+    unsigned long long timeout_ns;
+};
+bool small_supported(int d, int n, long long tokens, int L);
+cudaError_t launch_small(const SmallLaunch& L, int d, int sms, cudaStream_t st);
+// Read the kernel's error word and reset it to 0 (synchronous).
+cudaError_t small_error_word_read_clear(int* word);
+
 // ---- One-token decode (hcw_decode.cu) ----
 constexpr int kMaxDecodeLayers = 64;   // layers of one decode step
 // Split of one decode layer over a cluster: CTA q of csize owns output columns

@@ -310,68 +310,6 @@ __device__ __forceinline__ void red_relaxed_gpu_add(int* p, int v) {
     asm volatile("red.relaxed.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Two fp32 values in one 64-bit register pair, and the packed fp32 arithmetic
-// of the FP32 pipe (each instruction rounds both lanes like its scalar form).
-__device__ __forceinline__ uint64_t f32x2_pack(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 f32x2_unpack(uint64_t r) {
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
-    return make_float2(a, b);
-}
-__device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t f32x2_mul(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ float mul_sat_f32(float a, float b) {
-    float r;
-    asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-// (2^100, 2^100) as a packed pair
-constexpr uint64_t kF32x2Pow100 = 0x7180000071800000ull;
-// bf16 pair -> fp32 pair (exact: the bf16 bits are the high half of each float)
-__device__ __forceinline__ uint64_t bf16x2_to_f32x2(uint32_t w) {
-    return f32x2_pack(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
-}
-
-// 32 ReLU mask bits (bit c = column c) -> the AND-masks of 16 bf16 column
-// pairs: pair q keeps its low half iff bit 2q is set, its high half iff bit
-// 2q + 1 is.  t[k] = mw << (7 - k) puts bits k, k + 8, k + 16, k + 24 at the
-// sign positions of its four bytes; prmt in sign-replicate mode (selector
-// nibble 8 | byte) turns a selected byte into 0xFF or 0x00 by its sign bit, so
-// each pair's mask is one prmt of t[2i] and t[2i + 1] (the pair's two bits sit
-// in the same byte b = q / 4 of both).
-struct PairMasks {
-    uint32_t t[8];
-    __device__ __forceinline__ explicit PairMasks(uint32_t mw) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) t[k] = mw << (7 - k);
-    }
-    __device__ __forceinline__ uint32_t operator()(int q) const {
-        const int i = q & 3, b = q >> 2;
-        const uint32_t sel = (uint32_t)(8 | b) | (uint32_t)(8 | b) << 4 |
-                             (uint32_t)(12 | b) << 8 | (uint32_t)(12 | b) << 12;
-        uint32_t r;
-        asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(t[2 * i]), "r"(t[2 * i + 1]), "r"(sel));
-        return r;
-    }
-};
-
 // Adds v to the shared int *p with acquire-release semantics at CTA scope and
 // returns the previous value.
 __device__ __forceinline__ int atom_add_acq_rel_cta_shared(int* p, int v) {

@@ -522,6 +522,49 @@ def test_column_tile_choice_of_the_stack_keeps_the_bits(H, B, n, d):
     assert H.hcw_sync_status() == H.HCW_OK
 
 
+@pytest.mark.parametrize("B, n, d, L, flags, dims", [
+    (1, 2, 64, 1, CAUSAL | RESIDUAL | RELU, None),            # the smallest
+    (3, 64, 128, 6, RESIDUAL | RELU, None),                   # a ragged tile of 128 tokens
+    (5, 16, 64, 5, CAUSAL | RELU, None),                      # no residual
+    (9, 128, 128, 3, CAUSAL | RESIDUAL, None),                # no ReLU, links across the tile
+    (4, 32, 128, 4, 0, None),                                 # plain Eq. (1)
+    (9, 64, 128, 7, CAUSAL | RESIDUAL | RELU, [-1, 5, -7, 0, -63, 3, -1]),
+    (7, 128, 64, 4, RESIDUAL | RELU, [-64, 6, -127, 0]),
+    (320, 64, 128, 3, CAUSAL | RESIDUAL | RELU, None),        # more tiles than SMs
+    (700, 64, 64, 17, RESIDUAL | RELU, None),                 # the same at d = 64
+])
+def test_on_chip_stack_equals_the_streaming_one(H, B, n, d, L, flags, dims):
+    """Narrow layers over short windows run on the kernel that keeps 128 tokens on chip
+    (forward, input gradient, and both in the training step): every output is bit for
+    bit that of the streaming launches."""
+    g = torch.Generator(device="cuda").manual_seed(B)
+    x, dy = (torch.randn(B, n, d, generator=g, device="cuda").bfloat16() for _ in range(2))
+    Ws, Wn = ((torch.randn(L, d, d, generator=g, device="cuda") / (2 * d) ** 0.5).bfloat16()
+              for _ in range(2))
+    bias = torch.randn(L, d, generator=g, device="cuda") * 0.1
+    sched = dict(dims=dims) if dims else dict(layer0=2)
+
+    def both():
+        f = H.hcw_stack_fwd(x, Ws, Wn, bias, flags=flags, **sched)
+        b = H.hcw_stack_bwd(x, f[1], f[2], dy, Ws, Wn, flags=flags, **sched)
+        s = H.hcw_stack_train_step(x, Ws, Wn, bias, dy, flags=flags, **sched)
+        out = [t for t in (*f, *b, *s) if t is not None]
+        if not dims:
+            out += H.hcw_stack_bwd_data(f[2], dy, Ws, Wn, flags=flags, **sched)
+        assert H.hcw_sync_status() == H.HCW_OK
+        return out
+
+    got = both()
+    prev = H.hcw_set_stack_kernels(H.HCW_STACK_STREAMING)
+    try:
+        ref = both()
+    finally:
+        H.hcw_set_stack_kernels(prev)
+    assert len(got) == len(ref)
+    for i, (a, r) in enumerate(zip(got, ref)):
+        assert torch.equal(a, r), i
+
+
 DECODE_CASES = [
     # name, B, n, d, flags, dims (None = rot), layer0, L
     ("rot_n64", 4, 64, 128, CAUSAL | RESIDUAL | RELU, None, 0, 12),
