@@ -58,22 +58,6 @@ __device__ __forceinline__ int symbol(const int* ids, int b, int t, int n, int V
     return v;
 }
 
-// x[b n + t][c] = E[ids[b][t]][c] + P[t][c]   (fp32 out)
-__global__ void embed_fwd_kernel(const int* ids, const __nv_bfloat16* E, const __nv_bfloat16* P,
-                                 float* x, int B, int n, int d, int V) {
-    pdl_wait();   // until the kernel before it in the stream has finished
-    pdl_trigger();
-    const size_t total = (size_t)B * n * d;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % d);
-        const size_t r = i / d;
-        const int t = (int)(r % n), b = (int)(r / n);
-        const int v = symbol(ids, b, t, n, V);
-        x[i] = __bfloat162float(E[(size_t)v * d + c]) + __bfloat162float(P[(size_t)t * d + c]);
-    }
-}
-
 // One warp per row: x = x_in (+ add1 bf16) (+ add2 fp32) (+ badd[c]); x_out = x
 // when given; y = bf16((x - mean) rstd g + b); stats = (mean, rstd).  d <= 1024.
 __global__ void __launch_bounds__(kRowWarps * 32)
@@ -139,6 +123,38 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b) {
 }
 __device__ __forceinline__ float sum4(float4 a) { return a.x + a.y + a.z + a.w; }
 
+// fp32 buffers that later kernels of the step add into, zeroed by the first one
+constexpr int kZeroRanges = 4;
+struct ZeroRanges {
+    float* p[kZeroRanges];
+    size_t n[kZeroRanges];
+};
+
+// x[b n + t][c] = E[ids[b][t]][c] + P[t][c]   (fp32 out), a warp per row and four
+// features a lane and access (bound by the 33 MB it writes at 16,384 tokens of d =
+// 512: one element a thread with its own row arithmetic took 30 us); and the zero
+// ranges, which took a memset each.
+__global__ void __launch_bounds__(kRowWarps * 32)
+    embed_fwd_kernel(const int* ids, const __nv_bfloat16* E, const __nv_bfloat16* P, float* x,
+                     int B, int n, int d, int V, const __grid_constant__ ZeroRanges Z) {
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
+    const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+#pragma unroll
+    for (int k = 0; k < kZeroRanges; ++k)
+        for (size_t i = t0; i < Z.n[k]; i += stride) Z.p[k][i] = 0.f;
+    const int lane = threadIdx.x & 31;
+    for (long long r = (long long)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+         r < (long long)B * n; r += (long long)gridDim.x * kRowWarps) {
+        const int b = (int)(r / n), t = (int)(r & (n - 1));   // n is a power of two
+        const int v = symbol(ids, b, t, n, V);
+        for (int c = 4 * lane; c < d; c += 128)
+            st4(x, (size_t)r * d + c,
+                add4(ld4(E, (size_t)v * d + c), ld4(P, (size_t)t * d + c)));
+    }
+}
+
 // ln_fwd_kernel for d a multiple of 128: lane holds features 4 (i 32 + lane) ..
 // + 3 for i < d / 128 <= NV4.
 template <int NV4>
@@ -195,47 +211,61 @@ __global__ void __launch_bounds__(kRowWarps * 32)
 // One warp per position r = b n + t: z = logits[r] + bh (rows of ldz elements, a
 // multiple of 4), target v* = ids[b][t + 1]; loss += (logsumexp(z) - z[v*]) / N;
 // dlog[r][v] = bf16((softmax(z)[v] - [v == v*]) / N) (rows of ldd elements, a
-// multiple of 4).  Four symbols a lane and access, the last V % 4 one a lane.
+// multiple of 4).  Four symbols a lane and access, the last V % 4 one a lane; bound by
+// the exponentials' instructions at large V.
 __global__ void __launch_bounds__(kRowWarps * 32)
     ce_kernel(const float* logits, int ldz, const float* bh, const int* ids, __nv_bfloat16* dlog,
               int ldd, float* loss, int B, int n, int V, float inv_N) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
+    __shared__ float row_loss[kRowWarps];
     const int lane = threadIdx.x & 31;
     const int r = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
-    if (r >= B * n) return;
-    const int b = r / n, t = r % n;
-    const int tgt = symbol(ids, b, t + 1, n, V);
-    const float* z = logits + (size_t)r * ldz;
-    __nv_bfloat16* dz = dlog + (size_t)r * ldd;
-    const int v4 = V & ~3, vt = v4 + lane;   // the lane's symbol past the whole fours
-    const bool tail = vt < V;
-    const float zt = tail ? z[vt] + bh[vt] : -INFINITY;
-    float m = zt;
+    if (lane == 0) row_loss[threadIdx.x >> 5] = 0.f;
+    if (r < B * n) {
+        const int b = r / n, t = r & (n - 1);
+        const int tgt = symbol(ids, b, t + 1, n, V);
+        const float* z = logits + (size_t)r * ldz;
+        __nv_bfloat16* dz = dlog + (size_t)r * ldd;
+        const int v4 = V & ~3, vt = v4 + lane;   // the lane's symbol past the whole fours
+        const bool tail = vt < V;
+        const float zt = tail ? z[vt] + bh[vt] : -INFINITY;
+        // running maximum m (finite, so that a logit of -inf adds 0) and sum s of exp(z - m)
+        // of the lane's symbols, in one pass
+        float m = fmaxf(zt, -3.4e38f), s = expf(zt - m);
 #pragma unroll 4
-    for (int v = 4 * lane; v < v4; v += 128) {
-        const float4 q = add4(ld4(z, v), ld4(bh, v));
-        m = fmaxf(m, fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)));
+        for (int v = 4 * lane; v < v4; v += 128) {
+            const float4 q = add4(ld4(z, v), ld4(bh, v));
+            const float mx = fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w));
+            if (mx > m) {
+                s *= expf(m - mx);
+                m = mx;
+            }
+            s += (expf(q.x - m) + expf(q.y - m)) + (expf(q.z - m) + expf(q.w - m));
+        }
+        const float mw = warp_max(m);
+        const float lse = mw + logf(warp_sum(s * expf(m - mw)));
+#pragma unroll 4
+        for (int v = 4 * lane; v < v4; v += 128) {
+            const float4 q = add4(ld4(z, v), ld4(bh, v));
+            st4(dz, v, make_float4(expf(q.x - lse) * inv_N, expf(q.y - lse) * inv_N,
+                                   expf(q.z - lse) * inv_N, expf(q.w - lse) * inv_N));
+        }
+        if (tail) dz[vt] = __float2bfloat16_rn(expf(zt - lse) * inv_N);
+        // the target's own entry, over the one the same lane has just written
+        const float ztgt = z[tgt] + bh[tgt];
+        if (lane == (tgt < v4 ? (tgt >> 2) & 31 : tgt - v4))
+            dz[tgt] = __float2bfloat16_rn((expf(ztgt - lse) - 1.f) * inv_N);
+        if (lane == 0) row_loss[threadIdx.x >> 5] = (lse - ztgt) * inv_N;
     }
-    m = warp_max(m);
-    float s = tail ? expf(zt - m) : 0.f;
-#pragma unroll 2
-    for (int v = 4 * lane; v < v4; v += 128) {
-        const float4 q = add4(ld4(z, v), ld4(bh, v));
-        s += (expf(q.x - m) + expf(q.y - m)) + (expf(q.z - m) + expf(q.w - m));
+    // one addition a CTA: an addition a row, all to one address, took 20 us at 16,384
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < kRowWarps; ++w) t += row_loss[w];
+        atomicAdd(loss, t);
     }
-    const float lse = m + logf(warp_sum(s));
-#pragma unroll 2
-    for (int v = 4 * lane; v < v4; v += 128) {
-        const float4 q = add4(ld4(z, v), ld4(bh, v));
-        st4(dz, v,
-            make_float4((expf(q.x - lse) - (v == tgt ? 1.f : 0.f)) * inv_N,
-                        (expf(q.y - lse) - (v + 1 == tgt ? 1.f : 0.f)) * inv_N,
-                        (expf(q.z - lse) - (v + 2 == tgt ? 1.f : 0.f)) * inv_N,
-                        (expf(q.w - lse) - (v + 3 == tgt ? 1.f : 0.f)) * inv_N));
-    }
-    if (tail) dz[vt] = __float2bfloat16_rn((expf(zt - lse) - (vt == tgt ? 1.f : 0.f)) * inv_N);
-    if (lane == 0) atomicAdd(loss, (lse - (z[tgt] + bh[tgt])) * inv_N);
 }
 
 // out[c] += sum over a tile of kColRows rows of M[r][c] (bf16 M, T rows of ld
@@ -312,7 +342,7 @@ __device__ __forceinline__ void stv(__nv_bfloat16* p, size_t e, const float (&v)
 // summing per feature dy xhat (the scale gradient), dy (the shift gradient)
 // and, with ncol = 3, bf16(dx) (the column sums of dxb); the CTA adds its
 // warps' sums in warp order into row blockIdx.x of part [gridDim.x][ncol d],
-// which ln_part_reduce_kernel adds up in row order.
+// which ln_part_reduce_batched_kernel adds up in a fixed order.
 template <int NV, int W, typename DY>
 __global__ void __launch_bounds__(kRowWarps * 32)
     ln_bwd_fused_kernel(const DY* dy, const float* x, const float2* stats, const float* g,
@@ -393,47 +423,12 @@ __global__ void __launch_bounds__(kRowWarps * 32)
     }
 }
 
-// Sum of the nblk rows of part [nblk][ncol d] per column, in row order:
-// columns [0, d) -> dgam, [d, 2d) -> dbet, [2d, 3d) -> dcol.  A CTA of 32
-// warps per 32 columns, a column a lane: warp w adds rows w, w + 32, ...
-// (sixteen loads in flight), then the 32 warp sums meet in shared memory in
-// warp order.
-constexpr int kReduceWarps = 32;
-__global__ void __launch_bounds__(kReduceWarps * 32)
-    ln_part_reduce_kernel(const float* part, int nblk, int d, int ncol, float* dgam, float* dbet,
-                          float* dcol) {
-    pdl_wait();   // until the kernel before it in the stream has finished
-    pdl_trigger();
-    __shared__ float acc[kReduceWarps][33];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int width = ncol * d;
-    const int c = blockIdx.x * 32 + lane;
-    float s = 0.f;
-    if (c < width) {
-        for (int b0 = warp; b0 < nblk; b0 += 16 * kReduceWarps) {
-            float v[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const int b = b0 + k * kReduceWarps;
-                v[k] = b < nblk ? part[(size_t)b * width + c] : 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < 16; ++k) s += v[k];
-        }
-    }
-    acc[warp][lane] = s;
-    __syncthreads();
-    if (warp == 0 && c < width) {
-        float t = 0.f;
-#pragma unroll
-        for (int w = 0; w < kReduceWarps; ++w) t += acc[w][lane];
-        const int seg = c / d, cc = c - seg * d;
-        (seg == 0 ? dgam : (seg == 1 ? dbet : dcol))[cc] = t;
-    }
-}
-
-// The same sums for a list of LayerNorm backward passes at once: job
-// blockIdx.y adds up its own partial rows (in row order, as above).
+// Sums of a list of LayerNorm backward passes' partial rows: job blockIdx.y adds up
+// the nblk rows of its part [nblk][ncol d] per column: columns [0, d) -> dgam, [d, 2d)
+// -> dbet, [2d, 3d) -> dcol.  A CTA of eight warps per 128 columns, four a lane: warp w
+// adds rows w, w + 8, ... (eight loads in flight), then the warps' sums meet in shared
+// memory in warp order.  33 passes of d = 512: 29 us with a column a lane and 32 warps
+// a CTA, 21 so.
 constexpr int kMaxLnJobs = 64;
 struct LnJob {
     const float* part;
@@ -446,53 +441,50 @@ struct LnJobs {
     LnJob job[kMaxLnJobs];
     int d;
 };
-__global__ void __launch_bounds__(kReduceWarps * 32)
+__global__ void __launch_bounds__(kRowWarps * 32)
     ln_part_reduce_batched_kernel(const __grid_constant__ LnJobs J) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
-    __shared__ float acc[kReduceWarps][33];
+    __shared__ float4 acc[kRowWarps][32];
     const LnJob& jb = J.job[blockIdx.y];
     const int d = J.d;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int width = jb.ncol * d;
-    const int c = blockIdx.x * 32 + lane;
-    if (blockIdx.x * 32 >= width) return;   // block-uniform: this job is narrower
-    float s = 0.f;
+    const int c = blockIdx.x * 128 + 4 * lane;   // d is a multiple of 64: all four or none
+    if (blockIdx.x * 128 >= width) return;   // block-uniform: this job is narrower
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (c < width) {
-        for (int b0 = warp; b0 < jb.nblk; b0 += 16 * kReduceWarps) {
-            float v[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-                const int b = b0 + k * kReduceWarps;
-                v[k] = b < jb.nblk ? jb.part[(size_t)b * width + c] : 0.f;
-            }
-#pragma unroll
-            for (int k = 0; k < 16; ++k) s += v[k];
-        }
+#pragma unroll 8
+        for (int b = warp; b < jb.nblk; b += kRowWarps)
+            s = add4(s, ld4(jb.part, (size_t)b * width + c));
     }
     acc[warp][lane] = s;
     __syncthreads();
     if (warp == 0 && c < width) {
-        float t = 0.f;
+        float4 t = acc[0][lane];
 #pragma unroll
-        for (int w = 0; w < kReduceWarps; ++w) t += acc[w][lane];
+        for (int w = 1; w < kRowWarps; ++w) t = add4(t, acc[w][lane]);
         const int seg = c / d, cc = c - seg * d;
-        (seg == 0 ? jb.dgam : (seg == 1 ? jb.dbet : jb.dcol))[cc] = t;
+        st4(seg == 0 ? jb.dgam : (seg == 1 ? jb.dbet : jb.dcol), (size_t)cc, t);
     }
 }
 
-// dE[ids[b][t]] += dx[b n + t]   (dE zeroed before the launch)
-__global__ void embed_bwd_kernel(const int* ids, const float* dx, float* dE, int B, int n, int d,
-                                 int V) {
+// dE[ids[b][t]] += dx[b n + t]   (dE zeroed before), a warp per row, four features an
+// addition
+__global__ void __launch_bounds__(kRowWarps * 32)
+    embed_bwd_kernel(const int* ids, const float* dx, float* dE, int B, int n, int d, int V) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
-    const size_t total = (size_t)B * n * d;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % d);
-        const size_t r = i / d;
-        const int v = symbol(ids, (int)(r / n), (int)(r % n), n, V);
-        atomicAdd(dE + (size_t)v * d + c, dx[i]);
+    const int lane = threadIdx.x & 31;
+    for (long long r = (long long)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+         r < (long long)B * n; r += (long long)gridDim.x * kRowWarps) {
+        const int v = symbol(ids, (int)(r / n), (int)(r & (n - 1)), n, V);
+        for (int c = 4 * lane; c < d; c += 128) {
+            const float4 q = ld4(dx, (size_t)r * d + c);
+            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dE + (size_t)v * d + c),
+                         "f"(q.x), "f"(q.y), "f"(q.z), "f"(q.w)
+                         : "memory");
+        }
     }
 }
 
@@ -735,13 +727,13 @@ cudaError_t launch_ln_bwd_rows(cudaStream_t st, int grid, const DY* dy, const fl
 }
 
 // The LayerNorm backward: rows and per-CTA parameter sums in one pass
-// (ln_bwd_fused_kernel), then their fixed-order sum (ln_part_reduce_kernel)
-// into dgam, dbet and, when dcol is given, the column sums of dxb.  Two
-// launches (*nk).
+// (ln_bwd_fused_kernel).  Their fixed-order sum into dgam, dbet and, when dcol is
+// given, the column sums of dxb, is left to ln_part_reduce_batched_kernel with other
+// passes' (*sums; part stays untouched).  One launch (*nk).
 cudaError_t launch_ln_bwd(cudaStream_t st, const float* dyf, const __nv_bfloat16* dyb,
                           const float* x, const float2* stats, const float* g, const float* dres,
                           float* dx_out, __nv_bfloat16* dxb, float* part, float* dgam, float* dbet,
-                          float* dcol, int T, int d, int* nk, LnJob* defer = nullptr) {
+                          float* dcol, int T, int d, int* nk, LnJob* sums) {
     *nk = 0;
     if (dcol && !dxb) return cudaErrorInvalidValue;
     const int ncol = dcol ? 3 : 2;
@@ -756,15 +748,8 @@ cudaError_t launch_ln_bwd(cudaStream_t st, const float* dyf, const __nv_bfloat16
                                                             dx_out, dxb, T, d, ncol, part);
     if (e != cudaSuccess) return e;
     *nk = 1;
-    if (defer) {
-        // the sums are added up later, with other passes' (part stays untouched)
-        *defer = LnJob{part, grid, ncol, dgam, dbet, dcol};
-        return cudaSuccess;
-    }
-    e = launch_pdl(ln_part_reduce_kernel, dim3((ncol * d + 31) / 32), dim3(kReduceWarps * 32), 0,
-                   st, static_cast<const float*>(part), grid, d, ncol, dgam, dbet, dcol);
-    if (e == cudaSuccess) *nk = 2;
-    return e;
+    *sums = LnJob{part, grid, ncol, dgam, dbet, dcol};
+    return cudaSuccess;
 }
 
 int block_step(const int* ids, const hcw_block_params& p, const hcw_block_grads& gr, int B, int n,
@@ -804,19 +789,16 @@ int block_step(const int* ids, const hcw_block_params& p, const hcw_block_grads&
     } while (0)
 #define HCW_CU(expr) HCW_TRY((expr) == cudaSuccess ? HCW_OK : HCW_ERR_CUDA)
 #define HCW_GEMM(...) HCW_TRY(gemm(split, kSplitWs, st, __VA_ARGS__))
-    // gradients that are sums (atomics) start at zero; so does the loss
-    HCW_CU(cudaMemsetAsync(loss, 0, sizeof(float), st));
-    HCW_CU(cudaMemsetAsync(gr.E, 0, (size_t)V * d * 4, st));
-    float* zero_d[] = {gr.ln1_g, gr.ln1_b, gr.ln2_g, gr.ln2_b, gr.b2};
-    for (float* q : zero_d) HCW_CU(cudaMemsetAsync(q, 0, (size_t)L * d * 4, st));
-    HCW_CU(cudaMemsetAsync(gr.lnf_g, 0, (size_t)d * 4, st));
-    HCW_CU(cudaMemsetAsync(gr.lnf_b, 0, (size_t)d * 4, st));
-    HCW_CU(cudaMemsetAsync(gr.b1, 0, (size_t)L * h * 4, st));
-    HCW_CU(cudaMemsetAsync(gr.bh, 0, (size_t)V * 4, st));
+    // gradients that are sums (atomics) start at zero; so does the loss (zeroed by the
+    // first kernel)
+    const ZeroRanges zero = {{loss, gr.E, gr.b1, gr.bh},
+                             {1, (size_t)V * d, (size_t)L * h, (size_t)V}};
+    const size_t want = ((size_t)T + kRowWarps - 1) / kRowWarps, cap = (size_t)sms_now() * 8;
+    const dim3 row_loop((unsigned)(want < cap ? want : cap));   // warps stride over the rows
 
     // ------------------------------------------------------------ forward
-    HCW_TRY(count_launch(launch_pdl(embed_fwd_kernel, dim3(elem_grid(Td)), dim3(256), 0, st, ids,
-                                    bf(p.E, 0), bf(p.P, 0), X(0), B, n, d, V),
+    HCW_TRY(count_launch(launch_pdl(embed_fwd_kernel, row_loop, dim3(kRowWarps * 32), 0, st, ids,
+                                    bf(p.E, 0), bf(p.P, 0), X(0), B, n, d, V, zero),
                          1));
     HCW_TRY(count_launch(launch_ln_fwd(st, X(0), nullptr, nullptr, nullptr, nullptr, p.ln1_g,
                                        p.ln1_b, H1(0), S1(0), T, d),
@@ -906,8 +888,8 @@ int block_step(const int* ids, const hcw_block_params& p, const hcw_block_grads&
         part.d = d;
         for (int j = 0; j < cnt; ++j) part.job[j] = jobs[j0 + j];
         HCW_TRY(count_launch(launch_pdl(ln_part_reduce_batched_kernel,
-                                        dim3((3 * d + 31) / 32, cnt), dim3(kReduceWarps * 32), 0,
-                                        st, part),
+                                        dim3((3 * d + 127) / 128, cnt), dim3(kRowWarps * 32), 0, st,
+                                        part),
                              1));
     }
     // the FFN weight gradients of all layers, two batched launches (every
@@ -925,7 +907,7 @@ int block_step(const int* ids, const hcw_block_params& p, const hcw_block_grads&
     HCW_TRY(hcw_stack_bwd_weight(H1(0), L > 1 ? H1(1) : nullptr, DZM(0), 0, L, -1, B, n, d,
                                  HCW_BF16, HCW_CAUSAL, gr.W_self, gr.W_nbr, nullptr,
                                  w.sws_bytes ? ws + w.sws : nullptr, w.sws_bytes, st));
-    HCW_TRY(count_launch(launch_pdl(embed_bwd_kernel, dim3(elem_grid(Td)), dim3(256), 0, st, ids,
+    HCW_TRY(count_launch(launch_pdl(embed_bwd_kernel, row_loop, dim3(kRowWarps * 32), 0, st, ids,
                                     static_cast<const float*>(dx), gr.E, B, n, d, V),
                          1));
     return count_launch(launch_pdl(pos_bwd_kernel, dim3(elem_grid((size_t)n * d)), dim3(256), 0,
