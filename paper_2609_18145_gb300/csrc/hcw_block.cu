@@ -58,6 +58,18 @@ __device__ __forceinline__ int symbol(const int* ids, int b, int t, int n, int V
     return v;
 }
 
+// Drops a row of an fp32 GEMM output from L2 without writing it back: the warp has
+// read it for the last time (the values are in use: the caller has reduced over them),
+// and the next GEMM overwrites it.  The row and its size are multiples of 128 bytes.
+// At 16,384 rows of d = 512 the LayerNorm forward behind a GEMM took 18.5 us, 17.7 so,
+// its backward 30.4, 28.4 (33 MB less to DRAM each; bf16 rows gained nothing).
+template <typename V>
+__device__ __forceinline__ void discard_row(const V* row, int d) {
+    constexpr int kLine = 128 / sizeof(V);
+    for (int c = (threadIdx.x & 31) * kLine; c < d; c += 32 * kLine)
+        asm volatile("discard.global.L2 [%0], 128;" ::"l"(row + c) : "memory");
+}
+
 // One warp per row: x = x_in (+ add1 bf16) (+ add2 fp32) (+ badd[c]); x_out = x
 // when given; y = bf16((x - mean) rstd g + b); stats = (mean, rstd).  d <= 1024.
 __global__ void __launch_bounds__(kRowWarps * 32)
@@ -91,6 +103,7 @@ __global__ void __launch_bounds__(kRowWarps * 32)
     for (int i = 0; i < 32; ++i)
         if (i < nv) q += (v[i] - mean) * (v[i] - mean);
     const float rstd = rsqrtf(warp_sum(q) / d + kLnEps);
+    if (add2) discard_row(add2 + base, d);
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
         if (i < nv) {
@@ -194,6 +207,7 @@ __global__ void __launch_bounds__(kRowWarps * 32)
         }
     }
     const float rstd = rsqrtf(warp_sum(q) / d + kLnEps);
+    if (add2) discard_row(add2 + base, d);
 #pragma unroll
     for (int i = 0; i < NV4; ++i) {
         if (i < nv) {
@@ -392,6 +406,7 @@ __global__ void __launch_bounds__(kRowWarps * 32)
             }
         }
         const float m1 = warp_sum(s1) / d, m2 = warp_sum(s2) / d;
+        if (sizeof(DY) == 4) discard_row(dy + base, d);
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
             if (i < nv) {
