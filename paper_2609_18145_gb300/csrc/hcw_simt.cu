@@ -314,6 +314,8 @@ template <typename V>
 __global__ void __launch_bounds__(256)
     relu_grad_kernel(const V* __restrict__ dy, const V* __restrict__ z, V* __restrict__ dz,
                      size_t count) {
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
     constexpr int VEC = 16 / sizeof(V), U = 4;
     const size_t pieces = count / VEC, stride = (size_t)gridDim.x * blockDim.x;
     const size_t t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -464,6 +466,8 @@ __global__ void __launch_bounds__(512) splitk_reduce_kernel(
     const float* __restrict__ partial, int splits_max, int splits_self, int splits_nbr, int d,
     size_t part_stride, float* __restrict__ dWs, float* __restrict__ dWn, size_t out_stride,
     const float* __restrict__ bpart, float* __restrict__ dbias) {
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
     __shared__ float4 red[8][64];
     const int which = blockIdx.y;
     const int S = which == 1 ? splits_nbr : splits_self;
@@ -591,15 +595,14 @@ cudaError_t launch_f32_dw(F32DwArgs& a, int layers, int splits, cudaStream_t st,
 
 cudaError_t launch_relu_grad_f32(const float* dy, const float* z, float* dz, size_t count,
                                  cudaStream_t st) {
-    relu_grad_kernel<float><<<blocks_for(count / 4, 256), 256, 0, st>>>(dy, z, dz, count);
-    return cudaGetLastError();
+    return launch_pdl(relu_grad_kernel<float>, dim3(blocks_for(count / 4, 256)), dim3(256), 0, st,
+                      dy, z, dz, count);
 }
 
 cudaError_t launch_relu_grad_bf16(const __nv_bfloat16* dy, const __nv_bfloat16* z,
                                   __nv_bfloat16* dz, size_t count, cudaStream_t st) {
-    relu_grad_kernel<__nv_bfloat16>
-        <<<blocks_for(count / 8, 256), 256, 0, st>>>(dy, z, dz, count);
-    return cudaGetLastError();
+    return launch_pdl(relu_grad_kernel<__nv_bfloat16>, dim3(blocks_for(count / 8, 256)), dim3(256),
+                      0, st, dy, z, dz, count);
 }
 
 size_t colsum_workspace_bytes(long long rows, int d) {
@@ -640,10 +643,10 @@ cudaError_t launch_splitk_reduce(const float* partial, int splits_max, int split
     const size_t total4 = (size_t)d * d / 4;
     if (layers < 1) return cudaSuccess;
     const unsigned parts = (bpart && dbias) ? 3 : 2;
-    splitk_reduce_kernel<<<dim3((unsigned)((total4 + 63) / 64), parts, (unsigned)layers),
-                           dim3(64, 8), 0, st>>>(partial, splits_max, splits_self, splits_nbr, d,
-                                                 part_stride, dWs, dWn, out_stride, bpart, dbias);
-    return cudaGetLastError();
+    return launch_pdl(splitk_reduce_kernel,
+                      dim3((unsigned)((total4 + 63) / 64), parts, (unsigned)layers), dim3(64, 8), 0,
+                      st, partial, splits_max, splits_self, splits_nbr, d, part_stride, dWs, dWn,
+                      out_stride, bpart, dbias);
 }
 
 cudaError_t launch_shift_rows_bf16(const __nv_bfloat16* in, __nv_bfloat16* out, long long rows,

@@ -531,6 +531,12 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
     const uint32_t tmem_base = bars->tmem_base;
     volatile int* abort = &bars->abort;
     const uint64_t tmo = p.timeout_ns;
+    // a single-layer launch is a programmatic dependent: the prologue above, which
+    // touches no global memory, overlaps the end of the kernel before it
+    if (NL == 1) {
+        pdl_wait();
+        pdl_trigger();
+    }
     // the weight-gradient launch behind the fused one may take the SMs this
     // launch's CTAs leave at its end; it waits for its operands on the
     // completion counters (every CTA of this launch is resident by then)
@@ -2032,6 +2038,7 @@ static cudaError_t launch_one(const TcLaunch<NL>& L, int grid, cudaStream_t st) 
         if (e != cudaSuccess) return e;
         if (dev < 256) word.fetch_or(bit, std::memory_order_acq_rel);
     }
+    if (NL == 1) return launch_pdl(kern, dim3(grid), dim3(cta_threads(BN)), smem, st, L);
     if (!PAIR) {
         kern<<<grid, cta_threads(BN), smem, st>>>(L);
         return cudaGetLastError();
