@@ -1,6 +1,7 @@
 // hcw_api.cu -- the C ABI of include/hcw.h: argument validation, TMA tensor
 // maps, work decomposition and launches.  No device memory is allocated
 // here; every buffer is the caller's.
+#include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -242,6 +243,16 @@ bool map_f32_patches(CUtensorMap* m, const void* base, long long rows, int d) {
 
 int pick_bn(int d) { return d % 256 == 0 ? 256 : d % 128 == 0 ? 128 : 64; }
 
+// Widest column tile of the forward and input-gradient launches; the last tile of a d
+// that is not a multiple of it is ragged (its operand columns past d load as zeros, its
+// warps past d store nothing).  A unit's time is its operands' ingest, which hardly
+// falls with the tile (683, 655, 490 cycles a K step at 256 columns on pairs, 128 and
+// 64), so a ragged wide tile beats several narrow whole ones: at 64 columns for d = 320
+// a causal 13-layer forward of 58,624 tokens took 703 us, 415 so; an 18-layer one of
+// 49,152 tokens of d = 576 2,052 and 985 us; a layer of 64,256 tokens of d = 192 (forward
+// and backward) 103 and 75 us.
+int row_bn(int d) { return d <= 64 ? 64 : d <= 128 ? 128 : 256; }
+
 // ------------------------------------------------------------ validation
 struct Shape {
     int B, n, d, b, s;
@@ -420,6 +431,25 @@ int launched(cudaError_t e, int kernels) {
 }
 
 // ------------------------------------------------------------ layer internals
+// Column tile of a stacked forward / input-gradient launch.  With few tokens the
+// launch is the layer chain, not throughput: a unit's operands come at what one SM
+// takes in, so narrower tiles, spread over more SMs, shorten every step (each output
+// element sums the same products in the same order).  64 columns while every unit of
+// a layer has an SM of its own, 128 up to 1.75 waves, else 256 on pairs.  Microseconds a
+// layer of an 8-layer causal stack, forward / input gradient, at 64 | 128 | 256 columns:
+//   d = 256:  2048 tokens  6.3/6.8 | 6.9/7.3 | 8.6/8.9;   16384  12.2/13.9 | 8.6/9.7 | 9.6/9.9
+//   d = 512:   256 tokens  8.2/9.3 | 8.8/9.6 | 11.1/11.6;  2048  8.5/9.6 | 9.1/10.0 | 11.0/11.5
+//             4096 tokens  9.8/10.9 | 9.3/10.8 | 11.2/11.9;  8192  17.0/18.5 | 11.1/12.2 | 11.9/13.1
+//            16384 tokens  32.5/34.2 | 19.6/21.1 | 14.3/15.3
+//   d = 1024: 1024 tokens  12.8/15.1 | 13.6/15.0 | 15.5/16.5;  4096  27.3/29.8 | 16.8/18.3 | 17.0/18.3
+int stack_bn(const Shape& sh) {
+    const long long row_units = 2 * ((sh.tokens / 2 + 127) / 128);
+    const int sms = sm_count();
+    if (row_units * (sh.d / 64) <= sms) return 64;
+    if (sh.d > 64 && 4 * row_units * ((sh.d + 127) / 128) <= 7ll * sms) return 128;
+    return row_bn(sh.d);
+}
+
 // Row-unit geometry of a forward (or input-gradient) pass: which bit value's
 // rows take both parts.  Sec. 3.1 causal rule: in the forward, positions with
 // bit s set receive (K = 2d) and the others do not (K = d); in the input
@@ -430,7 +460,7 @@ void row_unit_params(TcParams& p, const Shape& sh, int BN, unsigned flags, bool 
     p.Mh = (int)(sh.tokens / 2);
     p.nK = d / 64;
     p.n_rb = (p.Mh + 127) / 128;
-    p.n_nt = d / BN;
+    p.n_nt = (d + BN - 1) / BN;
     if (flags & HCW_CAUSAL) {
         p.n_full = 1;
         p.full_bit0 = backward ? 0 : 1;
@@ -450,8 +480,8 @@ void row_unit_params(TcParams& p, const Shape& sh, int BN, unsigned flags, bool 
 // pair: the weight boxes hold half a column tile (each CTA of a pair loads
 // its half of B)
 bool fwd_maps(CUtensorMap* m, const Shape& sh, int s, const void* x, const void* Ws,
-              const void* Wn, const void* y, bool pair = false, int bn = 0) {
-    const int d = sh.d, BN = bn ? bn : pick_bn(d), k = 1 << s;
+              const void* Wn, const void* y, bool pair, int BN) {
+    const int d = sh.d, k = 1 << s;
     const int pw = epi_patch_cols(BN);
     const int box_o = pair ? BN / 2 : BN;
     if (!map_rows(&m[0], x, sh.tokens, d, k, 128) || !map_weight(&m[1], Ws, d, box_o) ||
@@ -467,10 +497,10 @@ bool fwd_maps(CUtensorMap* m, const Shape& sh, int s, const void* x, const void*
 int fwd_bf16(const Shape& sh, const void* x, const void* Ws, const void* Wn, const float* bias,
              unsigned flags, void* y, void* z, uint32_t* mask, cudaStream_t st,
              const void* xpair = nullptr) {
-    const int BN = pick_bn(sh.d);
+    const int BN = stack_bn(sh);
     TcLaunch<1> L;
     memset(&L, 0, sizeof(L));
-    if (!fwd_maps(L.maps[0], sh, sh.s, x, Ws, Wn, y)) return HCW_ERR_CUDA;
+    if (!fwd_maps(L.maps[0], sh, sh.s, x, Ws, Wn, y, false, BN)) return HCW_ERR_CUDA;
     // map 5: the row-aligned partner tensor, or the patches of z (never both: the
     // layer API has no shift layers)
     if (xpair && (z || !map_rows(&L.maps[0][5], xpair, sh.tokens, sh.d, 1 << sh.s, 128)))
@@ -503,25 +533,6 @@ size_t stack_counter_bytes(long long tokens, int L) {
 // row blocks.  Each SM of a pair loads its own rows and half of the weight
 // tile per stage.
 bool use_pairs(const Shape& sh, int BN) { return BN == 256 && sh.tokens / 2 > 128; }
-
-// Column tile of a stacked forward / input-gradient launch.  With few tokens the
-// launch is the layer chain, not throughput: a unit's operands come at what one SM
-// takes in, so narrower tiles, spread over more SMs, shorten every step (each output
-// element sums the same products in the same order).  64 columns while every unit of
-// a layer has an SM of its own, 128 up to 1.75 waves, else 256 on pairs.  Microseconds a
-// layer of an 8-layer causal stack, forward / input gradient, at 64 | 128 | 256 columns:
-//   d = 256:  2048 tokens  6.3/6.8 | 6.9/7.3 | 8.6/8.9;   16384  12.2/13.9 | 8.6/9.7 | 9.6/9.9
-//   d = 512:   256 tokens  8.2/9.3 | 8.8/9.6 | 11.1/11.6;  2048  8.5/9.6 | 9.1/10.0 | 11.0/11.5
-//             4096 tokens  9.8/10.9 | 9.3/10.8 | 11.2/11.9;  8192  17.0/18.5 | 11.1/12.2 | 11.9/13.1
-//            16384 tokens  32.5/34.2 | 19.6/21.1 | 14.3/15.3
-//   d = 1024: 1024 tokens  12.8/15.1 | 13.6/15.0 | 15.5/16.5;  4096  27.3/29.8 | 16.8/18.3 | 17.0/18.3
-int stack_bn(const Shape& sh) {
-    const long long row_units = 2 * ((sh.tokens / 2 + 127) / 128);
-    const int sms = sm_count();
-    if (row_units * (sh.d / 64) <= sms) return 64;
-    if (sh.d % 128 == 0 && 4 * row_units * (sh.d / 128) <= 7ll * sms) return 128;
-    return pick_bn(sh.d);
-}
 
 // Whether a bf16 stacked forward / input gradient runs on the resident
 // kernels (hcw_res.cu): the shape fits them (d in {128, 256, 512}, n <= 256,
@@ -660,7 +671,7 @@ int stack_fwd_resident(const Shape& sh, int l0, int n, const Sched& sc,
 int dx_bf16(const Shape& sh, const void* dz, const void* dy, const void* Ws, const void* Wn,
             unsigned flags, void* dx, cudaStream_t st, const uint32_t* mprev = nullptr,
             void* dz_out = nullptr, const void* dzpair = nullptr) {
-    const int d = sh.d, BN = pick_bn(d), k = 1 << sh.s;
+    const int d = sh.d, BN = stack_bn(sh), k = 1 << sh.s;
     const int pw = epi_patch_cols(BN);
     TcLaunch<1> L;
     memset(&L, 0, sizeof(L));
@@ -1744,7 +1755,7 @@ size_t step_counter_bytes(long long tokens, int L) {
 bool step_fused(const Shape& sh, int dtype, const Sched& sc, int L) {
     // 256- or 128-column tiles on pairs (d = 128 takes the latter), at least
     // two row blocks
-    const bool pairs = use_pairs(sh, pick_bn(sh.d)) || (pick_bn(sh.d) == 128 && sh.tokens / 2 > 128);
+    const bool pairs = row_bn(sh.d) >= 128 && sh.tokens / 2 > 128;
     return dtype == HCW_BF16 && (!sc.has_shift(L) || shift_stackable(sh)) && !use_resident(sh) &&
            pairs && L <= kMaxStackLayers && sh.tokens > 0;
 }
@@ -1765,12 +1776,26 @@ int step_fused_launch(const Shape& sh, const void* x, const uint8_t* Ws, const u
     // SM pairs without a unit of a layer (few tokens: the launch is the layer
     // chain, and narrower units shorten each of its steps)
     const int sms_all = sm_count();
-    int BN = pick_bn(sh.d);
+    int BN = row_bn(sh.d);
     {
         TcParams q;
         row_unit_params(q, sh, BN, flags, false);
         pair_units(q);
         if (BN == 256 && 2 * q.n_units <= sms_all / 2) BN = 128;
+        // with a ragged last tile also where the narrower tiles' waves take less time (a
+        // wave of 128 columns takes 0.73 of one of 256 by its ingest; 0.82 leaves out
+        // the near ties, which the wider tile won: 105 windows of 256, d = 320, 7 layers:
+        // 413 us at 256 columns, 478 at 128; 89 of 128, d = 384, 2 layers: 85 and 83)
+        if (BN == 256 && sh.d % 256 != 0) {
+            auto time = [&](int bn, double step) {
+                TcParams t;
+                row_unit_params(t, sh, bn, flags, false);
+                pair_units(t);
+                const double w = 2.0 * t.n_units / sms_all;
+                return (w < 4.0 ? ceil(w) : w) * step;
+            };
+            if (time(128, 0.82) < time(256, 1.0)) BN = 128;
+        }
     }
     const int d = sh.d, pw = epi_patch_cols(BN);
     const size_t ab = sh.act_bytes, a256 = align256(ab), wb = (size_t)d * d * 2;
@@ -1894,9 +1919,50 @@ int train_step_impl(const Shape& sh, const void* x, const void* W_self, const vo
     if (ws_bytes < bwd + fwd || !workspace) return HCW_ERR_WORKSPACE;
     if (!aligned16(workspace)) return HCW_ERR_ALIGNMENT;
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    if (!step_fused(sh, dtype, sc, L)) {
-        int rc = stack_fwd_impl(sh, x, W_self, W_nbr, bias, sc, L, dtype, flags, y, acts, masks,
-                                ws + bwd, fwd, stream);
+    int rc = HCW_OK;
+    const size_t ab = sh.act_bytes, wb = (size_t)d * d * 2;
+    const size_t acts_b = (size_t)(L - 1) * ab, m_b = (size_t)L * mask_bytes(sh);
+    auto check = [&]() -> int {
+        // the checks of the forward and the backward calls, on the same buffers
+        if (L > 1 && !acts) return HCW_ERR_INVALID_ARG;
+        if ((acts && !aligned16(acts)) || (masks && !aligned16(masks))) return HCW_ERR_ALIGNMENT;
+        rc = check_fwd_ptrs(sh, dtype, x, W_self, W_nbr, bias, y, nullptr);
+        if (rc) return rc;
+        if (overlaps(acts, acts_b, x, ab) || overlaps(acts, acts_b, y, ab) ||
+            overlaps(masks, m_b, x, ab) || overlaps(masks, m_b, y, ab) ||
+            overlaps(masks, m_b, acts, acts_b) || overlaps(acts, acts_b, W_self, L * wb) ||
+            overlaps(acts, acts_b, W_nbr, L * wb) || overlaps(ws, ws_bytes, x, ab) ||
+            overlaps(ws, ws_bytes, y, ab) || overlaps(ws, ws_bytes, acts, acts_b) ||
+            overlaps(ws, ws_bytes, masks, m_b) || overlaps(dx, ab, y, ab) ||
+            overlaps(dx, ab, acts, acts_b) || overlaps(dx, ab, x, ab) ||
+            overlaps(dx, ab, masks, m_b))
+            return HCW_ERR_ALIASING;
+        rc = check_stack_data(sh, dtype, flags, L, masks, dy, W_self, W_nbr, dx, ws, ws + zb, db);
+        if (rc) return rc;
+        if (want_dw) {
+            rc = check_stack_weight(sh, dtype, flags, L, x, acts, ws, dW_self, dW_nbr, dbias,
+                                    ws + zb + db, wbb);
+            if (rc) return rc;
+        }
+        if (overlaps(dx, ab, dW_self, (size_t)L * d * d * 4) ||
+            overlaps(dx, ab, dW_nbr, (size_t)L * d * d * 4) ||
+            overlaps(dx, ab, dbias, dbias ? (size_t)L * d * 4 : 0) ||
+            overlaps(dy, ab, y, ab) || overlaps(dy, ab, acts, acts_b) || overlaps(dy, ab, masks, m_b))
+            return HCW_ERR_ALIASING;
+        return HCW_OK;
+    };
+    bool fused = step_fused(sh, dtype, sc, L);
+    if (fused) {
+        rc = check();
+        // the two calls take overlaps that the one launch does not (its input gradient
+        // starts before the forward is done); they remain the way of a d that is not a
+        // multiple of 128
+        if (rc == HCW_ERR_ALIASING && d % 128 != 0) fused = false;
+        else if (rc) return rc;
+    }
+    if (!fused) {
+        rc = stack_fwd_impl(sh, x, W_self, W_nbr, bias, sc, L, dtype, flags, y, acts, masks,
+                            ws + bwd, fwd, stream);
         if (rc) return rc;
         if (want_dw)
             return stack_bwd_impl(sh, x, acts, masks, dy, W_self, W_nbr, sc, L, dtype, flags, dx,
@@ -1907,34 +1973,6 @@ int train_step_impl(const Shape& sh, const void* x, const void* W_self, const vo
                      static_cast<const uint8_t*>(W_nbr), sc, L, flags, dx, ws, ws + zb};
         return dtype == HCW_BF16 ? stack_data_bf16(sh, da, st) : stack_data_f32(sh, da, st);
     }
-    // the checks of the forward and the backward calls, on the same buffers
-    if (L > 1 && !acts) return HCW_ERR_INVALID_ARG;
-    if ((acts && !aligned16(acts)) || (masks && !aligned16(masks))) return HCW_ERR_ALIGNMENT;
-    int rc = check_fwd_ptrs(sh, dtype, x, W_self, W_nbr, bias, y, nullptr);
-    if (rc) return rc;
-    const size_t ab = sh.act_bytes, wb = (size_t)d * d * 2;
-    const size_t acts_b = (size_t)(L - 1) * ab, m_b = (size_t)L * mask_bytes(sh);
-    if (overlaps(acts, acts_b, x, ab) || overlaps(acts, acts_b, y, ab) ||
-        overlaps(masks, m_b, x, ab) || overlaps(masks, m_b, y, ab) ||
-        overlaps(masks, m_b, acts, acts_b) || overlaps(acts, acts_b, W_self, L * wb) ||
-        overlaps(acts, acts_b, W_nbr, L * wb) || overlaps(ws, ws_bytes, x, ab) ||
-        overlaps(ws, ws_bytes, y, ab) || overlaps(ws, ws_bytes, acts, acts_b) ||
-        overlaps(ws, ws_bytes, masks, m_b) || overlaps(dx, ab, y, ab) ||
-        overlaps(dx, ab, acts, acts_b) || overlaps(dx, ab, x, ab) ||
-        overlaps(dx, ab, masks, m_b))
-        return HCW_ERR_ALIASING;
-    rc = check_stack_data(sh, dtype, flags, L, masks, dy, W_self, W_nbr, dx, ws, ws + zb, db);
-    if (rc) return rc;
-    if (want_dw) {
-        rc = check_stack_weight(sh, dtype, flags, L, x, acts, ws, dW_self, dW_nbr, dbias,
-                                ws + zb + db, wbb);
-        if (rc) return rc;
-    }
-    if (overlaps(dx, ab, dW_self, (size_t)L * d * d * 4) ||
-        overlaps(dx, ab, dW_nbr, (size_t)L * d * d * 4) ||
-        overlaps(dx, ab, dbias, dbias ? (size_t)L * d * 4 : 0) ||
-        overlaps(dy, ab, y, ab) || overlaps(dy, ab, acts, acts_b) || overlaps(dy, ab, masks, m_b))
-        return HCW_ERR_ALIASING;
     const bool small = use_small(sh, L);
     if (small)
         rc = small_launch(sh, sc, L, flags, x, W_self, W_nbr, bias, y, acts,

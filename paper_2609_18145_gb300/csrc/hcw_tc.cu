@@ -1175,12 +1175,16 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                 const int qw = r.t * kBlockM + quarter * 32;   // first compressed row of the warp
                 const int lo_w = qw & (ly.k - 1), hi_w = qw >> ly.s;
                 const int q_row = qw + lane;
-                const int tok_row = q_row < p.Mh ? ((q_row >> ly.s) << (ly.s + 1)) +
-                                                       (r.beta << ly.s) + (q_row & (ly.k - 1))
-                                                 : -1;
+                // (d is a multiple of 64: of a ragged last column tile, a warp's columns are
+                // all inside or all past the end)
                 const int col0 = r.j * BN + cslice * WCOLS;
+                const bool cols_in = col0 < p.d;
+                const int tok_row = q_row < p.Mh && cols_in
+                                        ? ((q_row >> ly.s) << (ly.s + 1)) + (r.beta << ly.s) +
+                                              (q_row & (ly.k - 1))
+                                        : -1;
                 // a patch entirely past the end (ragged tail) loads and stores nothing
-                const bool inside = qw < p.Mh;
+                const bool inside = qw < p.Mh && cols_in;
                 const bool has_res = (p.flags & 2u) != 0 && inside;
                 const bool has_mprev = !fwd && ly.mprev != nullptr && ly.dz_out;
                 // fused launch: the last forward layer also writes the top layer's
@@ -1232,7 +1236,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                 float bias_reg[SUB];
 #pragma unroll
                 for (int h = 0; h < SUB; ++h)
-                    bias_reg[h] = fwd && ly.bias ? __ldg(ly.bias + col0 + h * 32 + lane) : 0.f;
+                    bias_reg[h] = fwd && ly.bias && cols_in ? __ldg(ly.bias + col0 + h * 32 + lane) : 0.f;
                 if (!wait_acc()) {
                     return false;
                 }
@@ -1354,7 +1358,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                         int* done = &bars->pub_done[kind][ordinal % kUnitQ];
                         if (atom_add_acq_rel_cta_shared(done, 1) == EW - 1) {
                             *done = 0;   // next used by ordinal + kUnitQ, after this unit
-                            const int cols = BN;
+                            const int cols = min(BN, p.d - r.j * BN);
                             int c0 = -1, n0 = 0, c1 = -1, n1 = 0;
                             for (int qd = 0; qd < 4; ++qd) {
                                 const int q = r.t * kBlockM + 32 * qd;

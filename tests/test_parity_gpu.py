@@ -522,6 +522,40 @@ def test_column_tile_choice_of_the_stack_keeps_the_bits(H, B, n, d):
     assert H.hcw_sync_status() == H.HCW_OK
 
 
+@pytest.mark.parametrize("B, n, d", [
+    (96, 256, 192),   # 256-column tiles, the only one ragged
+    (33, 256, 320),   # a whole and a ragged tile, a ragged last row block
+    (40, 256, 704),   # two whole tiles and one of 192 columns
+    (31, 256, 192),   # 128-column tiles, the second ragged
+])
+def test_ragged_column_tiles_keep_the_bits(H, B, n, d):
+    """Samples are independent, so the first one's rows of a large batch (wide column tiles,
+    the last one ragged where d is not a multiple of the tile) are bit for bit those of a
+    batch of one (64-column tiles): forward, masks, input gradient and the training step's
+    one-launch form of both."""
+    L, flags = 2, CAUSAL | RESIDUAL | RELU
+    g = torch.Generator(device="cuda").manual_seed(d)
+    x, dy = (torch.randn(B, n, d, generator=g, device="cuda").bfloat16() for _ in range(2))
+    Ws, Wn = ((torch.randn(L, d, d, generator=g, device="cuda") / (2 * d) ** 0.5).bfloat16()
+              for _ in range(2))
+    bias = torch.randn(L, d, generator=g, device="cuda")
+
+    def run(x, dy):
+        y, acts, masks = H.hcw_stack_fwd(x, Ws, Wn, bias, 3, -1, flags)
+        dx, dz = H.hcw_stack_bwd_data(masks, dy, Ws, Wn, 3, -1, flags)
+        z = H.hcw_layer_fwd(x, Ws[0], Wn[0], bias[0], 3, -1, flags, want_z=True)[1]
+        return [y, acts, masks, dx, dz, z]
+
+    big, one = run(x, dy), run(x[:1].contiguous(), dy[:1].contiguous())
+    step = H.hcw_stack_train_step(x, Ws, Wn, bias, dy, 3, -1, flags)
+    assert H.hcw_sync_status() == H.HCW_OK
+    for i, (a, b) in enumerate(zip(big, one)):
+        first = a[:, :1] if i in (1, 2, 4) else a[:1]
+        assert torch.equal(first, b), i
+    for i, j in ((0, 0), (1, 1), (2, 2), (3, 3)):
+        assert torch.equal(step[i], big[j]), i
+
+
 @pytest.mark.parametrize("B, n, d, L, flags, dims", [
     (1, 2, 64, 1, CAUSAL | RESIDUAL | RELU, None),            # the smallest
     (3, 64, 128, 6, RESIDUAL | RELU, None),                   # a ragged tile of 128 tokens
