@@ -544,7 +544,8 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
     }
 }
 
-// C[i] = sum over the splits s, in order, of part[s][i]; four at a time
+// C[i] = sum over the splits s, in order, of part[s][i]; four at a time with vec (count a
+// multiple of four: every split's partials start 16-byte aligned)
 __global__ void gemm_split_reduce_kernel(const float* part, int splits, size_t count, float* C,
                                          bool vec) {
     pdl_wait();   // until the kernel before it in the stream has finished
@@ -892,7 +893,7 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
         const unsigned g = (unsigned)(want < (size_t)sms * 8 ? (want ? want : 1) : (size_t)sms * 8);
         e = launch_pdl(gemm_split_reduce_kernel, dim3(g), dim3(256), 0, st,
                        static_cast<const float*>(split_ws), a.splits, count, C,
-                       aligned(C) && aligned(split_ws));
+                       aligned(C) && aligned(split_ws) && count % 4 == 0);
         if (e == cudaSuccess) *launches = 2;
     }
     return e;

@@ -61,6 +61,7 @@ CASES = [
     (64, 11, 64, False, True),        # 11 output columns (head of an 11-symbol vocabulary)
     (2048, 256, 512, False, True),    # the head's shape: tokens x V x d
     (512, 1024, 16384, True, False),  # a weight gradient: d x h x tokens, split
+    (65, 33, 4096, False, True),      # split, an output count not a multiple of four
     (37, 45, 29, False, False),       # plain kernel: rows TMA cannot read
     (11, 64, 32, True, False),        # plain kernel: MN-major A of 11 columns
 ]
