@@ -519,11 +519,13 @@ int hcw_block_step(const int* ids, const hcw_block_params* params, const hcw_blo
  * memory.  C is overwritten and must not overlap A, B or the workspace
  * (HCW_ERR_ALIASING).  M, N, K >= 1 (HCW_ERR_INVALID_ARG).  The workspace (may
  * be NULL; 16-byte aligned otherwise) holds fp32 partial sums when the K range
- * is split across CTAs: hcw_gemm_workspace_bytes gives the size that allows
- * the best split; a smaller one allows fewer splits, NULL none.  Partial sums
- * are added in split order.  Operands whose rows TMA cannot read (a K-major
- * row not a multiple of 16 bytes, an MN-major one not a multiple of 64
- * elements, a pointer not 16-byte aligned) take a plain tiled kernel.
+ * is split across CTAs, and padded copies of operands whose rows TMA cannot read
+ * (a K-major row not a multiple of 16 bytes, an MN-major one not a multiple of 64
+ * elements, a pointer not 16-byte aligned): hcw_gemm_workspace_bytes gives the
+ * size that allows the copies and the best split; a smaller one allows fewer
+ * splits, NULL none.  Partial sums are added in split order.  Without room for
+ * the copies (and where they would not pay) such operands take a plain tiled
+ * kernel.
  * Asynchronous on `stream`.
  */
 size_t hcw_gemm_workspace_bytes(int M, int N, int K);

@@ -31,8 +31,8 @@
 // Every wait is bounded: a CTA that gives up records HCW_ERR_TIMEOUT in the
 // error word, lets its copies and MMAs in flight finish, frees TMEM and
 // returns.  Shapes TMA cannot read (a K-major row stride not a multiple of 16
-// bytes, an MN-major one not a multiple of 64 elements) go to a plain tiled
-// kernel.
+// bytes, an MN-major one not a multiple of 64 elements) are packed into padded rows
+// first where the workspace has room and it pays, else go to a plain tiled kernel.
 #include "hcw.h"
 #include "hcw_internal.h"
 #include "hcw_ptx.cuh"
@@ -444,22 +444,29 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                     if (lane == 0) mbar_arrive_remote_tmem(tempty_leader);
                 }
                 const int col0 = ni * kGN + chalf * 128 + c * 32;
+                if (EPI == EPI_F32) {
+                    // rows TMA cannot write (not a multiple of 16 bytes): through a patch,
+                    // a row of 32 columns a store
+                    if (row0 >= a.M || col0 >= a.N) continue;   // warp-uniform
+                    uint8_t* buf = patch_buf(0);
+                    __syncwarp();
+#pragma unroll
+                    for (int m = 0; m < 8; ++m)
+                        *patch_chunk(buf, lane, m) =
+                            make_uint4(raw[4 * m], raw[4 * m + 1], raw[4 * m + 2], raw[4 * m + 3]);
+                    __syncwarp();
+                    float* dst = a.C + ((size_t)s * a.M + row0) * a.ldc + col0 + lane;
+                    const int rows = a.M - row0 < 32 ? a.M - row0 : 32;
+                    if (col0 + lane < a.N)
+#pragma unroll 8
+                        for (int r = 0; r < rows; ++r)
+                            dst[(size_t)r * a.ldc] = reinterpret_cast<const float*>(
+                                patch_chunk(buf, r, lane >> 2))[lane & 3];
+                    continue;
+                }
                 if (row >= a.M || col0 >= a.N) continue;
                 const bool full = a.vec && col0 + 32 <= a.N;
-                if (EPI == EPI_F32) {
-                    float* dst = a.C + ((size_t)s * a.M + row) * a.ldc + col0;
-                    if (full) {
-#pragma unroll
-                        for (int m = 0; m < 8; ++m)
-                            reinterpret_cast<float4*>(dst)[m] = make_float4(
-                                __uint_as_float(raw[4 * m]), __uint_as_float(raw[4 * m + 1]),
-                                __uint_as_float(raw[4 * m + 2]), __uint_as_float(raw[4 * m + 3]));
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            if (col0 + i < a.N) dst[i] = __uint_as_float(raw[i]);
-                    }
-                } else {
+                {
                     __nv_bfloat16* dst = a.out + (size_t)row * a.N + col0;
                     if (full) {
                         float v[32];
@@ -584,7 +591,8 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K,
     __shared__ float Bs[16][65];
     const int tm = blockIdx.y * 64, tn = blockIdx.x * 64;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int lda = e.lda ? e.lda : (ta ? M : K), ldc = e.ldc ? e.ldc : N;
+    const int lda = e.lda ? e.lda : (ta ? M : K), ldb = e.ldb ? e.ldb : (tb ? K : N);
+    const int ldc = e.ldc ? e.ldc : N;
     float acc[4][4] = {};
     for (int k0 = 0; k0 < K; k0 += 16) {
         for (int i = threadIdx.x; i < 16 * 64; i += 256) {
@@ -594,7 +602,7 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K,
             if (gm < M && gk < K)
                 av = __bfloat162float(ta ? A[(size_t)gk * lda + gm] : A[(size_t)gm * lda + gk]);
             if (gn < N && gk < K)
-                bv = __bfloat162float(tb ? B[(size_t)gn * K + gk] : B[(size_t)gk * N + gn]);
+                bv = __bfloat162float(tb ? B[(size_t)gn * ldb + gk] : B[(size_t)gk * ldb + gn]);
             As[kk][mm] = av;
             Bs[kk][mm] = bv;
         }
@@ -624,6 +632,33 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(int M, int N, int K,
                 if (e.colsum) atomicAdd(e.colsum + gn, __bfloat162float(e.out[o]));
             }
         }
+}
+
+// Copies of up to two row-major bf16 matrices (blockIdx.y) with their rows padded to ld
+// elements (a multiple of 8; the copy 16-byte aligned), zeros in the padding; a warp a
+// row, eight elements a lane.
+struct PackArgs {
+    const __nv_bfloat16* src[2];
+    __nv_bfloat16* dst[2];
+    int rows[2], cols[2], ld[2];
+};
+__global__ void __launch_bounds__(256) gemm_pack_kernel(const __grid_constant__ PackArgs p) {
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
+    const int q = blockIdx.y, lane = threadIdx.x & 31;
+    const int cols = p.cols[q], ld = p.ld[q];
+    for (int r = blockIdx.x * 8 + (threadIdx.x >> 5); r < p.rows[q]; r += gridDim.x * 8) {
+        const unsigned short* src =
+            reinterpret_cast<const unsigned short*>(p.src[q]) + (size_t)r * cols;
+        uint4* dst = reinterpret_cast<uint4*>(p.dst[q] + (size_t)r * ld);
+        for (int c = 8 * lane; c < ld; c += 256) {
+            uint32_t w[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) w[i] = c + i < cols ? src[c + i] : 0u;
+            dst[c / 8] = make_uint4(w[0] | w[1] << 16, w[2] | w[3] << 16, w[4] | w[5] << 16,
+                                    w[6] | w[7] << 16);
+        }
+    }
 }
 
 typedef CUresult (*GemmEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -785,6 +820,22 @@ bool epi_has_kernel(bool a_mn, bool b_mn, int epi) {
 
 namespace {
 
+// Padded row of an operand that TMA can read: 8 elements when K runs along the rows,
+// whole 64-column blocks otherwise; and the bytes of a padded copy.
+int pack_ld(int cols, bool k_major) { return k_major ? (cols + 7) & ~7 : (cols + 63) & ~63; }
+size_t pack_bytes(int rows, int cols, bool k_major) {
+    return ((size_t)rows * pack_ld(cols, k_major) * 2 + 255) & ~(size_t)255;
+}
+
+// Whether a product TMA cannot read is worth packing its operands: the plain kernel
+// takes 1.7 us per 16 of K and wave of tiles, the copies and the tensor-core kernel
+// about 10 us in all at these sizes (562 x 481 x 2674: 280 us plain, 21 packed; 848 x 76
+// x 4729: 445 and 17; 453 x 120 x 259: 28 and 16 a call, the host's part included).
+bool worth_packing(int M, int N, int K) {
+    const long long tiles = (long long)((M + 63) / 64) * ((N + 63) / 64);
+    return (double)K / 16 * 1.7 * ((double)tiles / 900 < 1 ? 1 : (double)tiles / 900) > 12.0;
+}
+
 // K splits for an M x N x K product on `sms` SMs (sms / 2 pairs): the count
 // that minimises the estimated time, waves of units x K steps per unit (about
 // 0.35 us each) plus writing and re-reading the fp32 partials (about 6 TB/s),
@@ -826,7 +877,8 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
     }
     if (bad) return cudaErrorInvalidValue;
     const bool a_mn = ta, b_mn = !tb;
-    const int lda = epi.lda ? epi.lda : (a_mn ? M : K), ldb = b_mn ? N : K;
+    const int lda = epi.lda ? epi.lda : (a_mn ? M : K);
+    const int ldb = epi.ldb ? epi.ldb : (b_mn ? N : K);
     const int ldc = epi.ldc ? epi.ldc : N;
     const auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
     // what TMA can read: 16-byte row strides, MN-major operands in whole
@@ -835,6 +887,43 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
     const bool tc = aligned(A) && aligned(B) && (a_mn ? lda % 64 == 0 : lda % 8 == 0) &&
                     (b_mn ? ldb % 64 == 0 : ldb % 8 == 0) && epi_has_kernel(a_mn, b_mn, epi.kind) &&
                     gemm_encode_fn() != nullptr;
+    if (!tc && epi.kind == EPI_F32 && gemm_encode_fn() && !epi.lda && !epi.ldb && split_ws &&
+        worth_packing(M, N, K)) {
+        // padded copies of the operands that TMA cannot read, in the workspace
+        const bool bad_a = !aligned(A) || (a_mn ? M % 64 : K % 8) != 0;
+        const bool bad_b = !aligned(B) || (b_mn ? N % 64 : K % 8) != 0;
+        PackArgs p = {};
+        size_t used = 0;
+        int n = 0, most = 0;
+        GemmEpi e2 = epi;
+        auto pack = [&](const void*& src, int rows, int cols, bool k_major, int& ld) {
+            ld = pack_ld(cols, k_major);
+            p.src[n] = static_cast<const __nv_bfloat16*>(src);
+            p.dst[n] = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<uint8_t*>(split_ws) + used);
+            p.rows[n] = rows;
+            p.cols[n] = cols;
+            p.ld[n] = ld;
+            src = p.dst[n];
+            used += pack_bytes(rows, cols, k_major);
+            most = rows > most ? rows : most;
+            ++n;
+        };
+        const void *A2 = A, *B2 = B;
+        if (bad_a) pack(A2, a_mn ? K : M, a_mn ? M : K, !a_mn, e2.lda);
+        if (bad_b) pack(B2, b_mn ? K : N, b_mn ? N : K, !b_mn, e2.ldb);
+        if (n > 0 && used <= split_ws_bytes) {
+            const int cap = gemm_sms() * 8, want = (most + 7) / 8;
+            cudaError_t e = launch_pdl(gemm_pack_kernel, dim3(want < cap ? want : cap, n),
+                                       dim3(256), 0, st, p);
+            if (e != cudaSuccess) return e;
+            int nl = 0;
+            e = gemm_bf16(M, N, K, A2, ta, B2, tb, C, e2,
+                          reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(split_ws) + used),
+                          split_ws_bytes - used, st, &nl);
+            *launches = 1 + nl;
+            return e;
+        }
+    }
     if (!tc) {
         dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
         const cudaError_t e = launch_pdl(gemm_simt_kernel, grid, dim3(256), 0, st, M, N, K,
@@ -847,7 +936,8 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
     // in shared memory only reach output rows and columns that are not stored)
     const int a_blk = (M + 63) / 64;
     const int a_box = a_mn ? (a_blk < kGM / 64 ? a_blk : kGM / 64) : (M < kGM ? M : kGM);
-    const int b_box = b_mn ? (N / 64 < kGN / 128 ? N / 64 : kGN / 128) : (N < kGN / 2 ? N : kGN / 2);
+    const int b_blk = (N + 63) / 64;
+    const int b_box = b_mn ? (b_blk < kGN / 128 ? b_blk : kGN / 128) : (N < kGN / 2 ? N : kGN / 2);
     GemmArgs a;
     memset(&a, 0, sizeof(a));
     if (!(a_mn ? map_mnmajor(&a.mA, A, K, M, lda, a_box) : map_kmajor(&a.mA, A, M, K, lda, a_box)) ||
@@ -977,7 +1067,13 @@ size_t hcw_gemm_workspace_bytes(int M, int N, int K) {
     if (M < 1 || N < 1 || K < 1) return 0;
     const size_t unlimited = (size_t)64 * M * N * sizeof(float);
     const int s = hcw::choose_splits(M, N, K, hcw::gemm_sms(), unlimited);
-    return s > 1 ? (size_t)s * M * N * sizeof(float) : 0;
+    const size_t split = s > 1 ? (size_t)s * M * N * sizeof(float) : 0;
+    // padded copies of operands whose rows TMA cannot read in some layout
+    if (M % 64 == 0 && N % 64 == 0 && K % 8 == 0) return split;
+    if (!hcw::worth_packing(M, N, K)) return split;
+    const auto larger = [](size_t a, size_t b) { return a > b ? a : b; };
+    return split + larger(hcw::pack_bytes(M, K, true), hcw::pack_bytes(K, M, false)) +
+           larger(hcw::pack_bytes(N, K, true), hcw::pack_bytes(K, N, false));
 }
 
 int hcw_gemm_bf16(int M, int N, int K, const void* A, int ta, const void* B, int tb, float* C,

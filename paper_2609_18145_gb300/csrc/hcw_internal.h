@@ -323,8 +323,8 @@ cudaError_t gemm_bf16_f32_batched(int M, int N, int K, const void* A, size_t a_b
                                   cudaStream_t st, int* launches);
 // Epilogues of the GEMM: fp32 C; out = bf16(relu(C + bias[col])); or
 // out = bf16(aux[row][col] > 0 ? C : 0), with colsum[col] (if given) += the
-// column sums of out.  out and aux are [M][N] bf16.  lda / ldc: elements from
-// one row of A (as stored) / C to the next; 0 = dense rows.
+// column sums of out.  out and aux are [M][N] bf16.  lda / ldb / ldc: elements from
+// one row of A / B (as stored) / C to the next; 0 = dense rows.
 enum GemmEpiKind { EPI_F32 = 0, EPI_BIAS_RELU = 1, EPI_RELU_GRAD = 2 };
 struct GemmEpi {
     int kind;
@@ -333,6 +333,7 @@ struct GemmEpi {
     __nv_bfloat16* out;
     float* colsum;
     int lda = 0;
+    int ldb = 0;
     int ldc = 0;
 };
 // gemm_bf16_f32 with an epilogue (C unused unless epi.kind is EPI_F32; only

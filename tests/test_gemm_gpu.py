@@ -64,6 +64,12 @@ CASES = [
     (65, 33, 4096, False, True),      # split, an output count not a multiple of four
     (37, 45, 29, False, False),       # plain kernel: rows TMA cannot read
     (11, 64, 32, True, False),        # plain kernel: MN-major A of 11 columns
+    # operands TMA cannot read, packed first, in each layout; ragged output rows
+    (900, 385, 228, True, False),
+    (562, 481, 674, False, True),
+    (70, 130, 1001, True, True),
+    (513, 77, 299, False, False),
+    (300, 257, 4099, False, True),    # the same with a long K: split
 ]
 
 
@@ -106,6 +112,15 @@ def test_misaligned_operands_take_the_plain_kernel(H):
     torch.cuda.synchronize()
     assert H.hcw_sync_status() == H.HCW_OK
     check(C.cpu(), A[:, 1:].contiguous(), B[:, 1:].contiguous(), False, True)
+
+
+def test_unreadable_operands_without_a_workspace_take_the_plain_kernel(H):
+    M, N, K = 130, 77, 299
+    A, B = operands(M, N, K, True, False, seed=6)
+    C = H.hcw_gemm_bf16(A.cuda(), B.cuda(), ta=True, split=False)
+    torch.cuda.synchronize()
+    assert H.hcw_sync_status() == H.HCW_OK
+    check(C.cpu(), A, B, True, False)
 
 
 BATCHED = [
