@@ -13,7 +13,8 @@
 // 64-element rows (128-byte swizzle), an MN-major one as blocks of 64 rows of
 // 64 columns, which is the layout tcgen05 reads as an MN-major operand.
 //
-// A cluster of two CTAs (one per SM) computes 256 x 256 output tiles with
+// A cluster of two CTAs (one per SM) computes 256 x 256 output tiles (256 x 128 in a
+// sparse last wave and past a narrow end of C) with
 // tcgen05.mma.cta_group::2: CTA r of the pair loads rows 128 r .. 128 r + 127
 // of the tile's A and columns 128 r .. 128 r + 127 of its B, so each SM takes
 // in 32 KB per 64-deep K step for 2 M multiply-adds.  In each CTA a producer
@@ -74,6 +75,7 @@ static_assert(kGSmem <= 232448, "shared memory budget");
 
 struct GemmArgs {
     CUtensorMap mA, mB;
+    CUtensorMap mBh;            // B in boxes half as wide, for the half units
     CUtensorMap mOut;           // output patches: fp32 (N, M, splits) box (32, 32, 1), or
                                 // bf16 (N, M) box (64, 32); 128-byte swizzle
     CUtensorMap mAux;           // EPI_RELU_GRAD: aux (N, M) bf16, box (64, 32)
@@ -87,18 +89,24 @@ struct GemmArgs {
     int ldc;                    // EPI_F32: elements from one row of C to the next
     int mt, nt;                 // tile counts (256-row tiles, 256-column tiles)
     int splits, kps;            // K splits and K steps per split
+    int full;                   // units below this one are whole tiles; each one from it on
+                                // is two of 256 x 128 (half_units)
     // batched (both operands MN-major, EPI_F32): `splits` counts independent
     // products instead of K splits; mA / mB carry the batch as a 4th dimension
     // and each unit takes the whole K range of product s into C[s]
     int batched;
     uint32_t stage_tx;          // bytes one CTA's two copies of a stage land
+    uint32_t stage_tx_half;     // the same in a half unit; 0 where every unit is whole
     int vec;                    // rows of the output start 16-byte aligned
     unsigned long long timeout_ns;
 };
 
-template <bool A_MN, bool B_MN, int EPI>
+// HALF: some units are 128 columns wide (without, every unit is a whole tile, and the
+// 2 % that choosing the width at run time costs long products is saved)
+template <bool A_MN, bool B_MN, int EPI, bool HALF>
 __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_constant__ GemmArgs a) {
     constexpr uint32_t IDESC = idesc_bf16_f32(2 * kGM, kGN, A_MN ? 1 : 0, B_MN ? 1 : 0);
+    constexpr uint32_t IDESC_HALF = idesc_bf16_f32(2 * kGM, kGN / 2, A_MN ? 1 : 0, B_MN ? 1 : 0);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -108,7 +116,8 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
     const uint32_t rank = cluster_ctarank();
     const int pair = (int)blockIdx.x >> 1, n_pairs = (int)gridDim.x >> 1;
     const int tiles = a.mt * a.nt;
-    const int n_units = tiles * a.splits;
+    // halves counted one by one
+    const int n_units = HALF ? 2 * tiles * a.splits - a.full : tiles * a.splits;
     const int nkb = (a.K + kGK - 1) / kGK;
     const uint64_t tmo = a.timeout_ns;
 
@@ -142,10 +151,25 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
     pdl_trigger();
     const uint32_t tmem_base = bars->tmem_base;
     volatile int* abort = &bars->abort;
-    // unit u -> (split, tile row, tile column), tile columns fastest: the pairs
-    // running together share their A rows (and B, the weights, is small)
-    auto unit_k = [&](int u, int& kb0, int& kb1) {
-        const int s = u / tiles;
+    // unit v -> (split, tile row, first column, width), tile columns fastest: the
+    // pairs running together share their A rows (and B, the weights, is small).  A unit
+    // is 128 columns wide where it is half of a tile, or the output ends in its first
+    // half; false where it holds no column at all.
+    struct Unit {
+        int s, mi, col0;
+        bool half;
+    };
+    auto unit = [&](int v, Unit& t) {
+        const int h = HALF ? v - a.full : -1;
+        const int u = h >= 0 ? a.full + (h >> 1) : v;
+        t.s = u / tiles;
+        const int rem = u - t.s * tiles;
+        t.mi = rem / a.nt;
+        t.col0 = (rem - t.mi * a.nt) * kGN + (h >= 0 ? (h & 1) * (kGN / 2) : 0);
+        t.half = HALF && (h >= 0 || t.col0 + kGN / 2 >= a.N);
+        return !HALF || t.col0 < a.N;
+    };
+    auto unit_k = [&](int s, int& kb0, int& kb1) {
         kb0 = a.batched ? 0 : s * a.kps;
         kb1 = a.batched ? nkb : (kb0 + a.kps < nkb ? kb0 + a.kps : nkb);
     };
@@ -157,9 +181,16 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
             uint32_t phase = 0, issued_mask = 0, issued_phase = 0;
             bool ok = true;
             for (int u = pair; u < n_units && ok; u += n_pairs) {
-                const int rem = u % tiles, mi = rem / a.nt, ni = rem - mi * a.nt;
+                Unit t;
+                if (!unit(u, t)) continue;
                 int kb0, kb1;
-                unit_k(u, kb0, kb1);
+                unit_k(t.s, kb0, kb1);
+                const CUtensorMap* mB = t.half ? &a.mBh : &a.mB;
+                const uint32_t tx = 2 * (t.half ? a.stage_tx_half : a.stage_tx);
+                // this CTA's 128 rows of A and its half of the unit's columns of B:
+                // 64-wide blocks of an MN-major operand, or rows of a K-major one
+                const int a_row = 2 * t.mi * kGM + (int)rank * kGM;
+                const int b_row = t.col0 + (int)rank * (t.half ? kGN / 4 : kGN / 2);
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (!mbar_wait(&bars->empty[stage], phase ^ 1, abort, tmo)) {
                         ok = false;
@@ -167,27 +198,22 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                     }
                     uint8_t* sA = smem + (size_t)stage * kGStage;
                     uint8_t* sB = sA + kGABytes;
-                    if (rank == 0) mbar_arrive_expect_tx(&bars->full[stage], 2 * a.stage_tx);
+                    if (rank == 0) mbar_arrive_expect_tx(&bars->full[stage], tx);
                     issued_mask |= 1u << stage;
                     issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
                     const uint32_t fb = mapa_shared(&bars->full[stage], 0);
-                    // this CTA's 128 rows of A and 128 columns of B: two 64-wide
-                    // blocks of an MN-major operand, or 128 rows of a K-major one
-                    const int a_row = 2 * mi * kGM + (int)rank * kGM;
-                    const int b_row = ni * kGN + (int)rank * (kGN / 2);
                     if (A_MN && B_MN && a.batched) {
-                        const int bi = u / tiles;   // the product
-                        tma_load_4d_pair(sA, &a.mA, fb, 0, kb * kGK, a_row / 64, bi);
-                        tma_load_4d_pair(sB, &a.mB, fb, 0, kb * kGK, b_row / 64, bi);
+                        tma_load_4d_pair(sA, &a.mA, fb, 0, kb * kGK, a_row / 64, t.s);
+                        tma_load_4d_pair(sB, mB, fb, 0, kb * kGK, b_row / 64, t.s);
                     } else {
                         if (A_MN)
                             tma_load_3d_pair(sA, &a.mA, fb, 0, kb * kGK, a_row / 64);
                         else
                             tma_load_2d_pair(sA, &a.mA, fb, kb * kGK, a_row);
                         if (B_MN)
-                            tma_load_3d_pair(sB, &a.mB, fb, 0, kb * kGK, b_row / 64);
+                            tma_load_3d_pair(sB, mB, fb, 0, kb * kGK, b_row / 64);
                         else
-                            tma_load_2d_pair(sB, &a.mB, fb, kb * kGK, b_row);
+                            tma_load_2d_pair(sB, mB, fb, kb * kGK, b_row);
                     }
                     if (++stage == kGStages) {
                         stage = 0;
@@ -208,8 +234,11 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true, any = false;
             for (int u = pair; u < n_units && ok; u += n_pairs) {
+                Unit t;
+                if (!unit(u, t)) continue;
                 int kb0, kb1;
-                unit_k(u, kb0, kb1);
+                unit_k(t.s, kb0, kb1);
+                const uint32_t idesc = t.half ? IDESC_HALF : IDESC;
                 if (!mbar_wait(&bars->tempty[acc], acc_phase ^ 1, abort, tmo)) {
                     ok = false;
                     break;
@@ -230,7 +259,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                                                  : smem_desc_sw128(sa + kk * 32, 16, 1024);
                         const uint64_t bd = B_MN ? smem_desc_sw128(sb + kk * 2048, 8192, 1024)
                                                  : smem_desc_sw128(sb + kk * 32, 16, 1024);
-                        mma_bf16_f32_pair(d_tmem, ad, bd, IDESC,
+                        mma_bf16_f32_pair(d_tmem, ad, bd, idesc,
                                           (kb != kb0 || kk != 0) ? 1u : 0u);
                     }
                     any = true;
@@ -254,7 +283,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
     } else {
         // ------------------------------------------------------------ epilogue (both CTAs)
         // warp e drains TMEM lane quarter warp % 4 (rows 32 q .. 32 q + 31 of
-        // this CTA's 128) and columns [128 (e / 4), 128 (e / 4) + 128)
+        // this CTA's 128) and half e / 4 of the unit's columns
         const int e = warp - 2;
         const int quarter = warp & 3, chalf = e >> 2;
         int acc = 0, nbuf = 0;
@@ -266,17 +295,20 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
             return reinterpret_cast<uint4*>(buf + r * 128 + ((m ^ (r & 7)) << 4));
         };
         for (int u = pair; u < n_units; u += n_pairs) {
-            const int s = u / tiles, rem = u % tiles, mi = rem / a.nt, ni = rem - mi * a.nt;
-            const int row0 = 2 * mi * kGM + (int)rank * kGM + quarter * 32;   // the warp's rows
+            Unit t;
+            if (!unit(u, t)) continue;
+            const int s = t.s;
+            const int cw = t.half ? kGN / 4 : kGN / 2;                        // the warp's columns
+            const int row0 = 2 * t.mi * kGM + (int)rank * kGM + quarter * 32;   // the warp's rows
             const int row = row0 + lane;
-            const int colw = ni * kGN + chalf * 128;                          // and columns
+            const int colw = t.col0 + chalf * cw;                             // and first column
             // EPI_RELU_GRAD: the aux patches of the tile's two 64-column halves go
             // into the warp's two buffers before the accumulator is ready (the
             // stores of the tile before have read them by then); the second half
             // is stored only if the first is, so half hh lands in buffer nbuf ^ hh
             int n_aux = 0;
             if (EPI == EPI_RELU_GRAD && a.tma_out) {
-                n_aux = (row0 < a.M && colw < a.N) + (row0 < a.M && colw + 64 < a.N);
+                n_aux = (row0 < a.M && colw < a.N) + (row0 < a.M && cw > 64 && colw + 64 < a.N);
                 if (lane == 0 && n_aux > 0) {
                     bulk_wait_read<0>();
                     mbar_arrive_expect_tx(&bars->aux[e], (uint32_t)(n_aux * kGPatch));
@@ -290,7 +322,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
             if (!__all_sync(0xffffffffu, okw)) break;
             tc_fence_after();
             const uint32_t tbase = tmem_base + ((uint32_t)(quarter * 32) << 16) +
-                                   (uint32_t)(acc * kGN + chalf * 128);
+                                   (uint32_t)(acc * kGN + chalf * cw);
             const uint32_t tempty_leader = mapa_shared(&bars->tempty[acc], 0);
             if (a.tma_out) {
                 // Patches of 32 rows x 128 bytes through shared memory (128-byte
@@ -300,7 +332,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                 bool okp = true;
                 if (EPI == EPI_F32) {
 #pragma unroll 1
-                    for (int c = 0; c < 4; ++c) {
+                    for (int c = 0; c < cw / 32; ++c) {
                         const bool st = row0 < a.M && colw + c * 32 < a.N;   // warp-uniform
                         uint32_t raw[32];
                         if (st) {
@@ -308,7 +340,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                             tmem_ld_32x32b_x32(tbase + (uint32_t)(c * 32), raw);
                             tmem_ld_wait_regs(raw);
                         }
-                        if (c == 3) {
+                        if (c == cw / 32 - 1) {
                             tc_fence_before();
                             __syncwarp();
                             if (lane == 0) mbar_arrive_remote_tmem(tempty_leader);
@@ -331,10 +363,10 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                     }
                 } else {
 #pragma unroll 1
-                    for (int hh = 0; hh < 2; ++hh) {
+                    for (int hh = 0; hh < cw / 64; ++hh) {
                         const int c0 = colw + hh * 64;
                         if (!(row0 < a.M && c0 < a.N)) {   // warp-uniform: nothing to store
-                            if (hh == 1) {
+                            if (hh == cw / 64 - 1) {
                                 tc_fence_before();
                                 __syncwarp();
                                 if (lane == 0) mbar_arrive_remote_tmem(tempty_leader);
@@ -350,7 +382,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                         tmem_ld_32x32b_x32(tbase + (uint32_t)(hh * 64 + 32), r1);
                         tmem_ld_wait_regs(r0);
                         tmem_ld_wait_regs(r1);
-                        if (hh == 1) {
+                        if (hh == cw / 64 - 1) {
                             tc_fence_before();
                             __syncwarp();
                             if (lane == 0) mbar_arrive_remote_tmem(tempty_leader);
@@ -431,19 +463,17 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                 continue;
             }
 #pragma unroll 1
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < cw / 32; ++c) {
                 uint32_t raw[32];
                 __syncwarp();
-                tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) +
-                                       (uint32_t)(acc * kGN + chalf * 128 + c * 32),
-                                   raw);
+                tmem_ld_32x32b_x32(tbase + (uint32_t)(c * 32), raw);
                 tmem_ld_wait_regs(raw);
-                if (c == 3) {
+                if (c == cw / 32 - 1) {
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive_remote_tmem(tempty_leader);
                 }
-                const int col0 = ni * kGN + chalf * 128 + c * 32;
+                const int col0 = colw + c * 32;
                 if (EPI == EPI_F32) {
                     // rows TMA cannot write (not a multiple of 16 bytes): through a patch,
                     // a row of 32 columns a store
@@ -761,9 +791,9 @@ int gemm_sms() {
     return n;
 }
 
-template <bool A_MN, bool B_MN, int EPI>
-cudaError_t launch_gemm_pair(const GemmArgs& a, int grid, cudaStream_t st) {
-    auto kern = gemm_pair_kernel<A_MN, B_MN, EPI>;
+template <bool A_MN, bool B_MN, int EPI, bool HALF>
+cudaError_t launch_gemm_half(const GemmArgs& a, int grid, cudaStream_t st) {
+    auto kern = gemm_pair_kernel<A_MN, B_MN, EPI, HALF>;
     static std::once_flag once[64];
     static cudaError_t set_err[64];
     int dev = 0;
@@ -791,6 +821,12 @@ cudaError_t launch_gemm_pair(const GemmArgs& a, int grid, cudaStream_t st) {
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+template <bool A_MN, bool B_MN, int EPI>
+cudaError_t launch_gemm_pair(const GemmArgs& a, int grid, cudaStream_t st) {
+    return a.stage_tx_half ? launch_gemm_half<A_MN, B_MN, EPI, true>(a, grid, st)
+                           : launch_gemm_half<A_MN, B_MN, EPI, false>(a, grid, st);
 }
 
 // The instantiated (layout, epilogue) combinations: every layout for fp32
@@ -835,6 +871,23 @@ bool worth_packing(int M, int N, int K) {
     const long long tiles = (long long)((M + 63) / 64) * ((N + 63) / 64);
     return (double)K / 16 * 1.7 * ((double)tiles / 900 < 1 ? 1 : (double)tiles / 900) > 12.0;
 }
+
+// The first of the units that are taken as two halves of 128 columns: the last, partial
+// wave, where its halves fit the pairs too (elsewhere `units`, none).
+// A half takes 24 KB instead of 32 a K step and half the epilogue, about 0.7 of a whole
+// tile's time, so it pays wherever the halves all run at once and costs nothing elsewhere.
+// In us a product, whole tiles and with halves: 16384 x 1024 x 512 (28 of 256 units in the
+// last wave) 22.5, 21.5; 2048 x 512 x 512 (16 units) 7.3, 6.2; 4096 x 256 x 128 5.6, 4.5;
+// 1024 x 1024 x 1024 9.8, 9.0; 8192 x 768 x 256 8.6, 7.9.  The block step at d = 128,
+// n = 64, V = 4,769: 822, 784.
+int half_units(int units, int pairs) {
+    if (pairs < 1) return units;
+    const int left = units % pairs;
+    return 2 * left <= pairs ? units - left : units;
+}
+
+// whether the last tile's columns all lie in its first half
+bool has_narrow_tile(int N) { return (N - 1) % kGN < kGN / 2; }
 
 // K splits for an M x N x K product on `sms` SMs (sms / 2 pairs): the count
 // that minimises the estimated time, waves of units x K steps per unit (about
@@ -956,6 +1009,16 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
         split_ws && epi.kind == EPI_F32 && ldc == N ? choose_splits(M, N, K, sms, split_ws_bytes) : 1;
     a.kps = (nkb + splits - 1) / splits;
     a.splits = (nkb + a.kps - 1) / a.kps;   // no empty split
+    const int whole = a.mt * a.nt * a.splits;
+    a.full = half_units(whole, sms / 2);
+    if (a.full < whole || has_narrow_tile(N)) {
+        const int h_box = b_mn ? 1 : (N < kGN / 4 ? N : kGN / 4);
+        if (!(b_mn ? map_mnmajor(&a.mBh, B, K, N, ldb, h_box)
+                   : map_kmajor(&a.mBh, B, N, K, ldb, h_box)))
+            return cudaErrorInvalidValue;
+        a.stage_tx_half = (uint32_t)(kGK * 2) * (uint32_t)((a_mn ? 64 * a_box : a_box) +
+                                                           (b_mn ? 64 : h_box));
+    }
     if (epi.kind == EPI_F32) {
         a.C = a.splits > 1 ? split_ws : C;
         a.ldc = ldc;
@@ -972,7 +1035,7 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
                     (epi.kind != EPI_RELU_GRAD || map_patch_bf16(&a.mAux, epi.aux, M, N));
     }
     a.timeout_ns = kGemmTimeoutNs;
-    const int units = a.mt * a.nt * a.splits;
+    const int units = 2 * whole - a.full;
     const int pairs = units < sms / 2 ? units : sms / 2;
     cudaError_t e = launch_gemm_any(a_mn, b_mn, epi.kind, a, 2 * (pairs > 0 ? pairs : 1), st);
     if (e != cudaSuccess) return e;
@@ -1045,7 +1108,14 @@ cudaError_t gemm_bf16_f32_batched(int M, int N, int K, const void* A, size_t a_b
     a.tma_out = map_out_f32(&a.mOut, C, M, N, N, batch);
     a.timeout_ns = kGemmTimeoutNs;
     const int sms = gemm_sms();
-    const int units = a.mt * a.nt * batch;
+    const int whole = a.mt * a.nt * batch;
+    a.full = half_units(whole, sms / 2);
+    if (a.full < whole || has_narrow_tile(N)) {
+        if (!map_mnmajor_batched(&a.mBh, B, K, N, 1, batch, b_batch_bytes))
+            return cudaErrorInvalidValue;
+        a.stage_tx_half = (uint32_t)(kGK * 2) * (uint32_t)(64 * a_box + 64);
+    }
+    const int units = 2 * whole - a.full;
     const int pairs = units < sms / 2 ? units : sms / 2;
     const cudaError_t e = launch_gemm_any(true, true, EPI_F32, a, 2 * pairs, st);
     if (e == cudaSuccess) *launches = 1;

@@ -70,6 +70,10 @@ CASES = [
     (70, 130, 1001, True, True),
     (513, 77, 299, False, False),
     (300, 257, 4099, False, True),    # the same with a long K: split
+    # whole tiles in full waves, the last wave's tiles as halves of 128 columns
+    (20 * 256, 4 * 256, 128, False, True),
+    (20 * 256 - 60, 4 * 256 - 200, 128, True, False),    # the last tile's second half empty
+    (11 * 256 + 8, 8 * 256 - 64, 72, False, False),
 ]
 
 
