@@ -1452,7 +1452,32 @@ int stack_weight_bf16(const Shape& sh, const StackWeight& a, cudaStream_t st) {
     return HCW_OK;
 }
 
-// fp32 input gradients, layer by layer (the correctness path).
+// The launch of all fp32 layers of a stack, forward or (bwd) input gradients.
+int f32_chain(const Shape& sh, const Sched& sc, int L, unsigned flags, int block_rows, bool bwd,
+              const void* in, const void* Ws, const void* Wn, const float* bias, void* acts,
+              void* out, uint32_t* mask_out, const void* masks, cudaStream_t st) {
+    F32ChainArgs c;
+    c.in = static_cast<const float*>(in);
+    c.Ws = static_cast<const float*>(Ws);
+    c.Wn = static_cast<const float*>(Wn);
+    c.bias = bias;
+    c.acts = static_cast<float*>(acts);
+    c.out = static_cast<float*>(out);
+    c.mask_out = mask_out;
+    c.masks = static_cast<const uint32_t*>(masks);
+    c.act_elems = sh.tokens * sh.d;
+    c.mask_words = (long long)(mask_bytes(sh) / 4);
+    c.rows = sh.tokens;
+    for (int l = 0; l < L; ++l) c.s[l] = sc.dim(sh, l);
+    c.n = sh.n;
+    c.d = sh.d;
+    c.L = L;
+    c.block_rows = block_rows;
+    c.flags = flags;
+    return launched(launch_f32_chain(c, bwd, st), 1);
+}
+
+// fp32 input gradients: one launch for narrow layers, else layer by layer.
 int stack_data_f32(const Shape& sh, const StackData& a, cudaStream_t st) {
     const int d = sh.d, L = a.L;
     const bool relu = (a.flags & HCW_ACT_RELU) != 0;
@@ -1464,6 +1489,9 @@ int stack_data_f32(const Shape& sh, const StackData& a, cudaStream_t st) {
         return reinterpret_cast<const uint32_t*>(static_cast<const uint8_t*>(a.masks) +
                                                  (size_t)l * mb);
     };
+    if (const int block_rows = f32_chain_rows(sh.tokens, sh.n, d, L, sm_count()))
+        return f32_chain(sh, a.sc, L, a.flags, block_rows, true, a.dy, a.Ws, a.Wn, nullptr, a.dz,
+                         a.dx, nullptr, relu ? a.masks : nullptr, st);
     int rc;
     if (relu) {
         rc = launched(launch_relu_grad_mask_f32(static_cast<const float*>(a.dy), mask(L - 1),
@@ -1688,6 +1716,17 @@ int stack_fwd_impl(const Shape& sh, const void* x, const void* W_self, const voi
         }
         return HCW_OK;
     }
+    const size_t wL = (size_t)L * wb, bias_b = bias ? (size_t)L * d * 4 : 0;
+    const int block_rows = f32_chain_rows(sh.tokens, n, d, L, sm_count());
+    // one launch where nothing it writes is read by another of its blocks (the checks
+    // above leave y or the masks over the weights or the bias to the launches' order)
+    if (block_rows && !overlaps(y, ab, W_self, wL) && !overlaps(y, ab, W_nbr, wL) &&
+        !overlaps(y, ab, x, ab) && !overlaps(y, ab, bias, bias_b) &&
+        !overlaps(acts, acts_b, bias, bias_b) &&
+        !(want_mask && (overlaps(masks, m_b, W_self, wL) || overlaps(masks, m_b, W_nbr, wL) ||
+                        overlaps(masks, m_b, bias, bias_b))))
+        return f32_chain(sh, sc, L, flags, block_rows, false, x, W_self, W_nbr, bias, acts, y,
+                         want_mask ? mask_ptr(0) : nullptr, nullptr, st);
     for (int l = 0; l < L; ++l) {
         Shape shl = sh;
         shl.s = sc.dim(sh, l);

@@ -388,6 +388,28 @@ struct F32DwArgs {
 };
 int f32_dw_splits(long long rows, int d, int layers, int sms);
 cudaError_t launch_f32_dw(F32DwArgs& a, int layers, int splits, cudaStream_t st, int* launches);
+// The fp32 layers of a stack in one launch: x through all layers (acts, y, mask words),
+// or with bwd dy down through all layers (in = dy, acts = every layer's dz, out = dx).
+struct F32ChainArgs {
+    const float* in;
+    const float* Ws;
+    const float* Wn;
+    const float* bias;           // or null
+    float* acts;
+    float* out;
+    uint32_t* mask_out;          // or null
+    const uint32_t* masks;       // bwd with the ReLU
+    long long act_elems, mask_words, rows;
+    int s[kMaxF32Layers];        // links, as for the other fp32 kernels
+    int n, d, L, block_rows;
+    // set by the launch: rows in 16-byte pieces, threads a row (a power of two, at least
+    // its pieces), buffers of the ring (a power of two)
+    int vec, lanes_log2, stages;
+    unsigned flags;
+};
+// The rows of a block where that launch is the faster way, else 0.
+int f32_chain_rows(long long rows, int n, int d, int L, int sms);
+cudaError_t launch_f32_chain(F32ChainArgs& a, bool bwd, cudaStream_t st);
 // dz = dy * (z > 0), elementwise over count elements (T = float or bf16)
 cudaError_t launch_relu_grad_f32(const float* dy, const float* z, float* dz, size_t count,
                                  cudaStream_t st);

@@ -12,6 +12,8 @@
 //          i receives iff i >= k (a shift always links earlier to later).
 #include "hcw_internal.h"
 
+#include <mutex>
+
 namespace hcw {
 
 namespace {
@@ -38,10 +40,9 @@ constexpr int T = 32;   // tile edge of the fp32 kernels
 // (checks and first experiments, d in the tens): they are bound by launches and by
 // the latency of a step, so every launch is a programmatic dependent of the one
 // before it, the input gradient writes the layer below's dz itself, and one launch
-// computes the weight and bias gradients of a whole stack (four layers forward and
-// backward at 64 rows of d = 32: 24 launches, 127 us, now 10, 48 us; seven layers
-// at 3,968 rows of d = 91, whose gradient blocks each walked all rows: 2,493 us,
-// now 402).
+// computes the weight and bias gradients of a whole stack (seven layers at 3,968 rows of
+// d = 91, whose gradient blocks each walked all rows: 2,493 us, now 402).  Narrow layers
+// run in one launch a direction (f32_chain_kernel).
 
 // z[r][o] = sum_k Ws[o][k] x[r][k] + m_r sum_k Wn[o][k] x[p(r)][k] + bias[o]
 // mout (optional): ReLU mask words [rows][ceil(d/32)], bit o%32 of word o/32 = (z > 0).
@@ -191,6 +192,237 @@ __global__ void __launch_bounds__(256)
         if (dx) dx[r * d + k] = v;
         // (the tile's 32 columns are one mask word)
         if (dz_prev) dz_prev[r * d + k] = (mprev[r * wpr + (k0 >> 5)] >> tx) & 1u ? v : 0.f;
+    }
+}
+
+// ---- fp32 stacks of narrow layers: all layers in one launch ----
+// A block keeps the rows of whole windows on chip and walks the layers over them (every
+// partner of a row is in its window), the next layers' weights, biases and masks on their
+// way into a ring of shared-memory buffers while one is computed.  Layer by layer these
+// stacks are bound by launches, about 4 us each: four layers forward and backward at 64
+// rows of d = 32 took 46 us a call of each, now 29 (the host's part), 19 of them on the
+// GPU.  A lane per output column, kChainRows rows per warp at a time, and the products in
+// the order of the tiled kernels: the same bits.  A layer is bound by shared-memory reads
+// (ten 16-byte ones for 32 products a lane), 0.7 us at 16 rows of d = 32.
+constexpr int kChainRows = 4;
+constexpr size_t kChainSmem = 232448;
+
+__device__ __forceinline__ void cp_async_f32(float* dst, const float* src, bool vec) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(dst);
+    if (vec)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(a), "l"(src) : "memory");
+}
+
+// Row stride in shared memory: whole 16-byte pieces, an odd number of them (a quarter of
+// a warp reading one piece of eight rows hits every bank once).
+__host__ __device__ inline int chain_ld(int d) { return 4 * (((d + 3) / 4) | 1); }
+
+// One buffer of the ring, in floats: both weights, and the bias or the rows' mask words.
+__host__ __device__ inline size_t chain_stage(int d, int rows) {
+    const size_t ld = chain_ld(d), d4 = (d + 3) & ~3, mw = (size_t)rows * ((d + 31) / 32);
+    return 2 * d4 * ld + (((mw > d4 ? mw : d4) + 3) & ~(size_t)3);
+}
+
+// Shared memory, in floats: the ring, three buffers of rows, a row of zeros.
+__host__ __device__ inline size_t chain_floats(int d, int rows, int stages) {
+    return stages * chain_stage(d, rows) + (3 * (size_t)rows + 1) * chain_ld(d);
+}
+
+// BWD false: x through layers 0 .. L-1 to acts, y and the mask words.  BWD true: dy down
+// through layers L-1 .. 0 to every layer's dz and dx.
+template <bool BWD>
+__global__ void __launch_bounds__(256) f32_chain_kernel(const __grid_constant__ F32ChainArgs A) {
+    extern __shared__ float4 chain_smem[];
+    float* smem = reinterpret_cast<float*>(chain_smem);
+    const int d = A.d, d4 = (d + 3) & ~3, ld = chain_ld(d), n = A.n;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wsz = d4 * ld, xsz = A.block_rows * ld;
+    const int stage = (int)chain_stage(d, A.block_rows);
+    float* const xbuf = smem + A.stages * stage;
+    float* const gbuf = xbuf + 2 * xsz;      // BWD: the unmasked gradient (residual)
+    const int zero = (int)(gbuf + xsz - smem);   // the row of zeros
+    const int pieces = (int)(chain_floats(d, A.block_rows, A.stages) / 4);
+    for (int i = threadIdx.x; i < pieces; i += blockDim.x)
+        chain_smem[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    pdl_wait();   // until the kernel before it in the stream has finished
+    pdl_trigger();
+
+    const long long r0 = (long long)blockIdx.x * A.block_rows;
+    const int rows = A.rows - r0 < A.block_rows ? (int)(A.rows - r0) : A.block_rows;
+    const bool vec = A.vec;
+    const int wpr = (d + 31) >> 5;
+    const bool relu = A.flags & 4u, res = A.flags & 2u;
+    // this thread's piece of a row, and the rows a pass of the block takes
+    const int prow = threadIdx.x >> A.lanes_log2, prows = 256 >> A.lanes_log2;
+    const int pcol = (threadIdx.x & ((1 << A.lanes_log2) - 1)) * (vec ? 4 : 1);
+    // the i-th layer of the walk into its buffer (nothing past the last: an empty group)
+    auto issue = [&](int i) {
+        if (i >= A.L) {
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            return;
+        }
+        const int l = BWD ? A.L - 1 - i : i;
+        float* const buf = smem + (i & (A.stages - 1)) * stage;
+        const float* const src[2] = {A.Ws + (size_t)l * d * d, A.Wn + (size_t)l * d * d};
+        for (int o = prow; o < d; o += prows)
+            if (pcol < d) {
+                cp_async_f32(buf + o * ld + pcol, src[0] + o * d + pcol, vec);
+                cp_async_f32(buf + wsz + o * ld + pcol, src[1] + o * d + pcol, vec);
+            }
+        const float* aux = nullptr;
+        int count = 0;
+        if (!BWD && A.bias) {
+            aux = A.bias + (size_t)l * d;
+            count = d;
+        } else if (BWD && relu && l > 0) {
+            aux = reinterpret_cast<const float*>(A.masks + (size_t)(l - 1) * A.mask_words + r0 * wpr);
+            count = rows * wpr;
+        }
+        for (int t = threadIdx.x; t < count; t += 256)
+            cp_async_f32(buf + 2 * wsz + t, aux + t, false);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    const int top = A.L - 1;
+    if (!BWD && pcol < d)   // the rows: part of the first layer's group
+        for (int r = prow; r < rows; r += prows)
+            cp_async_f32(xbuf + r * ld + pcol, A.in + (r0 + r) * d + pcol, vec);
+    for (int i = 0; i + 1 < A.stages; ++i) issue(i);
+    if (BWD && pcol < d) {
+        // the top layer's dz
+        const uint32_t* const mask = A.masks + (size_t)top * A.mask_words + r0 * wpr + (pcol >> 5);
+        auto row = [&](int r, auto v) {
+            const uint32_t w = (relu ? mask[r * wpr] : ~0u) >> (pcol & 31);
+            const size_t at = (r0 + r) * d + pcol;
+            *reinterpret_cast<decltype(v)*>(gbuf + r * ld + pcol) = v;
+            float* e = reinterpret_cast<float*>(&v);
+#pragma unroll
+            for (int j = 0; j < (int)(sizeof(v) / 4); ++j) e[j] = (w >> j) & 1u ? e[j] : 0.f;
+            *reinterpret_cast<decltype(v)*>(xbuf + r * ld + pcol) = v;
+            *reinterpret_cast<decltype(v)*>(A.acts + (size_t)top * A.act_elems + at) = v;
+        };
+        if (vec)
+            for (int r = prow; r < rows; r += prows)
+                row(r, *reinterpret_cast<const float4*>(A.in + (r0 + r) * d + pcol));
+        else
+            for (int r = prow; r < rows; r += prows) row(r, A.in[(r0 + r) * d + pcol]);
+    }
+
+    const int cwarps = wpr, groups = 8 / cwarps;   // column warps, row groups
+    const int cw = warp % cwarps, grp = warp / cwarps;
+    const int c = cw * 32 + lane;
+    const bool col_ok = c < d;
+    const int cc = col_ok ? c : 0;
+    for (int i = 0; i < A.L; ++i) {
+        const int l = BWD ? A.L - 1 - i : i;
+        if (A.stages == 4)
+            asm volatile("cp.async.wait_group 2;" ::: "memory");
+        else
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();   // this layer's weights and rows are there, the one before is done
+        issue(i + A.stages - 1);
+        const float* ws = smem + (i & (A.stages - 1)) * stage;
+        const float* wn = ws + wsz;
+        const float* aux = wn + wsz;
+        const float* cur = xbuf + (i & 1) * xsz;
+        const int curo = (int)(cur - smem);
+        float* next = xbuf + ((i + 1) & 1) * xsz;
+        const int s = A.s[l];
+        const bool last = i + 1 == A.L;
+        const float bias = !BWD && A.bias ? aux[cc] : 0.f;
+        if (grp < groups)
+            for (int rb = grp * kChainRows; rb < rows; rb += groups * kChainRows) {
+                int xr[kChainRows], pr[kChainRows];   // rows' offsets in shared memory
+                uint32_t mw[kChainRows];
+#pragma unroll
+                for (int q = 0; q < kChainRows; ++q) {
+                    const int rr = rb + q, j = rr & (n - 1);
+                    int from = -1;
+                    if (rr < rows) {
+                        if (BWD)
+                            from = reader_of(j, s, n, A.flags);
+                        else if (receives(j, s, A.flags))
+                            from = partner_of(j, s);
+                    }
+                    xr[q] = rr < rows ? curo + rr * ld : zero;
+                    pr[q] = from >= 0 ? curo + (rr - j + from) * ld : zero;
+                    mw[q] = BWD && relu && !last && rr < rows
+                                ? reinterpret_cast<const uint32_t*>(aux)[rr * wpr + cw]
+                                : ~0u;
+                }
+                float acc[kChainRows];
+#pragma unroll
+                for (int q = 0; q < kChainRows; ++q) acc[q] = 0.f;
+#pragma unroll 4
+                for (int k = 0; k < d4; k += 4) {
+                    float u[4], v[4];
+                    float4 xv[kChainRows], pv[kChainRows];
+                    if (BWD) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            u[j] = ws[(k + j) * ld + cc];
+                            v[j] = wn[(k + j) * ld + cc];
+                        }
+                    } else {
+                        const float4 a = *reinterpret_cast<const float4*>(ws + cc * ld + k);
+                        const float4 b = *reinterpret_cast<const float4*>(wn + cc * ld + k);
+                        u[0] = a.x, u[1] = a.y, u[2] = a.z, u[3] = a.w;
+                        v[0] = b.x, v[1] = b.y, v[2] = b.z, v[3] = b.w;
+                    }
+#pragma unroll
+                    for (int q = 0; q < kChainRows; ++q) {
+                        xv[q] = *reinterpret_cast<const float4*>(smem + xr[q] + k);
+                        pv[q] = *reinterpret_cast<const float4*>(smem + pr[q] + k);
+                    }
+                    auto step = [&](auto at, int j) {
+#pragma unroll
+                        for (int q = 0; q < kChainRows; ++q) acc[q] = fmaf(at(xv[q]), u[j], acc[q]);
+#pragma unroll
+                        for (int q = 0; q < kChainRows; ++q) acc[q] = fmaf(at(pv[q]), v[j], acc[q]);
+                    };
+                    step([](const float4& f) { return f.x; }, 0);
+                    step([](const float4& f) { return f.y; }, 1);
+                    step([](const float4& f) { return f.z; }, 2);
+                    step([](const float4& f) { return f.w; }, 3);
+                }
+#pragma unroll
+                for (int q = 0; q < kChainRows; ++q) {
+                    const int rr = rb + q;
+                    if (rr >= rows) break;   // warp-uniform
+                    const size_t at = (r0 + rr) * d + c;
+                    if (BWD) {
+                        float v = acc[q];
+                        if (!col_ok) continue;
+                        if (res) v += gbuf[rr * ld + c];
+                        gbuf[rr * ld + c] = v;
+                        if (last) {
+                            A.out[at] = v;
+                        } else {
+                            v = (mw[q] >> lane) & 1u ? v : 0.f;
+                            next[rr * ld + c] = v;
+                            A.acts[(size_t)(l - 1) * A.act_elems + at] = v;
+                        }
+                    } else {
+                        float v = col_ok ? acc[q] + bias : 0.f;
+                        if (A.mask_out) {
+                            const unsigned bits = __ballot_sync(0xffffffffu, v > 0.f);
+                            if (lane == 0)
+                                A.mask_out[(size_t)l * A.mask_words + (r0 + rr) * wpr + cw] = bits;
+                        }
+                        if (!col_ok) continue;
+                        if (relu) v = v > 0.f ? v : 0.f;
+                        if (res) v += cur[rr * ld + c];
+                        if (last) {
+                            A.out[at] = v;
+                        } else {
+                            next[rr * ld + c] = v;
+                            A.acts[(size_t)l * A.act_elems + at] = v;
+                        }
+                    }
+                }
+            }
     }
 }
 
@@ -591,6 +823,60 @@ cudaError_t launch_f32_dw(F32DwArgs& a, int layers, int splits, cudaStream_t st,
                    dim3(256), 0, st, a);
     if (e == cudaSuccess) *launches = 2;
     return e;
+}
+
+// The windows a block of the one launch takes, one wave of blocks, where a layer costs
+// it less than its own launch does.  Both sides in us a layer and direction, fitted to
+// four layers forward and backward (graphs; us layer by layer, in one launch): n = 16,
+// 64 rows: d = 16 35.6, 17.1; d = 32 36.2, 18.8; d = 64 52.7, 30.2; d = 91 67.3, 71;
+// d = 96 67, 59.  4,096 rows: d = 32 44.4, 35.0; d = 64 128, 85; d = 96 235, 177.
+// n = 64, 64 rows: d = 32 36.1, 34.3; d = 48 52, 73.  n = 256: one window is too much
+// for a block from d = 16 on (42, 83) unless there are many (64 windows: 113, 104).
+int f32_chain_rows(long long rows, int n, int d, int L, int sms) {
+    if (L < 2 || L > kMaxF32Layers || d > 128) return 0;
+    const long long windows = rows / n;
+    const long long per = (windows + sms - 1) / sms;   // windows a block, one wave
+    if (per * n > 4096) return 0;
+    const int R = (int)(per * n);
+    if (chain_floats(d, R, 2) * sizeof(float) > kChainSmem) return 0;
+    const int cols = (d + 31) / 32, groups = 8 / cols;
+    const int passes = (R + kChainRows * groups - 1) / (kChainRows * groups);
+    double chain = passes * (0.5 + 0.17 * ((d + 3) / 4) * (cols * groups / 8.0));
+    if (d % 4) chain *= 1.25;   // weights copied 4 bytes at a time
+    const double steps = (double)((rows + T - 1) / T) * cols * cols;   // of all tiles
+    const double one = 1.05 * (1.8 + 1.75 * cols), many = 1.0 + 0.0185 * steps;
+    return chain < (one > many ? one : many) ? R : 0;
+}
+
+template <bool BWD>
+static cudaError_t launch_chain(const F32ChainArgs& a, cudaStream_t st) {
+    static std::once_flag once[64];
+    static cudaError_t set_err[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    std::call_once(once[dev], [&] {
+        set_err[dev] = cudaFuncSetAttribute(f32_chain_kernel<BWD>,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)kChainSmem);
+    });
+    if (set_err[dev] != cudaSuccess) return set_err[dev];
+    const unsigned grid = (unsigned)((a.rows + a.block_rows - 1) / a.block_rows);
+    return launch_pdl(f32_chain_kernel<BWD>, dim3(grid), dim3(256),
+                      chain_floats(a.d, a.block_rows, a.stages) * sizeof(float), st, a);
+}
+
+cudaError_t launch_f32_chain(F32ChainArgs& a, bool bwd, cudaStream_t st) {
+    a.vec = a.d % 4 == 0 && (reinterpret_cast<uintptr_t>(a.Ws) & 15) == 0 &&
+            (reinterpret_cast<uintptr_t>(a.Wn) & 15) == 0 &&
+            (reinterpret_cast<uintptr_t>(a.in) & 15) == 0 &&
+            (reinterpret_cast<uintptr_t>(a.acts) & 15) == 0;
+    const int pieces = a.vec ? a.d / 4 : a.d;
+    a.lanes_log2 = 0;
+    while ((1 << a.lanes_log2) < pieces) ++a.lanes_log2;
+    a.stages = a.L > 2 && chain_floats(a.d, a.block_rows, 4) * sizeof(float) <= kChainSmem ? 4 : 2;
+    return bwd ? launch_chain<true>(a, st) : launch_chain<false>(a, st);
 }
 
 cudaError_t launch_relu_grad_f32(const float* dy, const float* z, float* dz, size_t count,

@@ -1100,3 +1100,50 @@ def test_bounded_wait_reports_timeout_and_context_survives(H):
     torch.cuda.synchronize()
     yr = O.layer_fwd(x64, W64, W64, None, 1, -1, CAUSAL, round_bf16=True)
     assert rel(host(y), yr) <= TOL_BF16
+
+
+# fp32 stacks whose layers run in one launch: B, n, d, flags, links
+CHAINS = [
+    (3, 16, 32, CAUSAL | RESIDUAL | RELU, (0, 3, 1, 2)),
+    (5, 2, 7, RELU, (0, 0)),                            # two buffers, unaligned rows
+    (1, 64, 32, 0, (5, -1, 2)),                         # a shift, several passes over the rows
+    (9, 8, 91, CAUSAL | RELU, (2, 1, -3, 0)),           # three column warps, the last ragged
+    (2, 16, 96, RESIDUAL | RELU, (3, 0, 2, 1, 3)),      # a ring of two buffers
+    (400, 16, 33, RESIDUAL, (1, 2, 3, 0, 1, 2)),        # three windows a block, the last fewer
+    (3, 8, 112, CAUSAL | RESIDUAL, (0, 1, 2)),          # the widest
+]
+
+
+@pytest.mark.parametrize("case", CHAINS, ids=lambda c: "B%d_n%d_d%d_f%d_L%d" % (c[:4] + (len(c[4]),)))
+def test_fp32_stack_in_one_launch_matches_its_layers(H, case):
+    """The launch of all layers adds the products in the order of the single-layer
+    kernels: every output has the bits that one call a layer gives."""
+    B, n, d, flags, dims = case
+    L = len(dims)
+    pr = synth.problem(B, n, d, L=L, seed=5 + d, w_std=(1 / (2 * d)) ** 0.5)
+    x, _ = dev(pr.x, torch.float32)
+    Ws, _ = dev(pr.W_self, torch.float32)
+    Wn, _ = dev(pr.W_nbr, torch.float32)
+    dy, _ = dev(pr.dy, torch.float32)
+    bias = torch.from_numpy(pr.bias).cuda()
+    before = H.hcw_launch_count()
+    y, acts, masks = H.hcw_stack_fwd_dims(x, Ws, Wn, bias, dims, flags)
+    assert H.hcw_launch_count() - before == 1
+    dx = H.hcw_stack_bwd(x, acts, masks, dy, Ws, Wn, flags=flags, dims=dims)[0]
+    def params(l):   # copies: an aligned start each
+        return [t[l:l + 1].clone() for t in (Ws, Wn, bias)]
+
+    cur, single = x, []
+    for l in range(L):
+        cur, _, m = H.hcw_stack_fwd_dims(cur, *params(l), dims[l:l + 1], flags)
+        single.append((acts[l - 1] if l else x, m))
+        assert torch.equal(cur, acts[l] if l + 1 < L else y)
+        if flags & RELU:
+            assert torch.equal(m[0], masks[l])
+    g = dy
+    for l in reversed(range(L)):
+        g = H.hcw_stack_bwd(single[l][0].clone(), None, single[l][1], g, *params(l)[:2],
+                            flags=flags, dims=dims[l:l + 1])[0]
+    assert torch.equal(dx, g)
+    torch.cuda.synchronize()
+    assert H.hcw_sync_status() == H.HCW_OK
