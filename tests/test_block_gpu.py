@@ -96,6 +96,13 @@ CASES = [
     (3, 16, 128, 256, 389, 2),    # logit rows past whole tiles and whole fours
     (3, 32, 128, 256, 256, 4),
     (1, 64, 192, 136, 37, 2),
+    # the cross-entropy's row kernels: a warp a row, a block a row, two passes
+    (2, 16, 64, 128, 130, 1),
+    (2, 16, 64, 128, 512, 1),
+    (2, 16, 64, 128, 515, 1),
+    (2, 16, 64, 128, 2046, 1),
+    (2, 16, 64, 128, 4097, 1),
+    (2, 16, 64, 128, 8193, 1),
 ]
 
 
