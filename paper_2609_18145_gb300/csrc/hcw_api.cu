@@ -1280,9 +1280,13 @@ int split_dw_launch(const Shape& sh, const StackWeight& a, int l0, int cnt, uint
     p.seq_n = sh.n;
     p.timeout_ns = g_timeout_ns;
     T.n_layers = cnt;
-    T.sched = sched;
-    if (cudaMemsetAsync(sched, 0, sizeof(int), st) != cudaSuccess) return HCW_ERR_CUDA;
     const int sms = sm_count(), total = w.units * cnt;
+    // a CTA a unit needs no counter, and no memset in front that would keep the launch
+    // from overlapping the end of the kernel before it
+    if (total > sms) {
+        T.sched = sched;
+        if (cudaMemsetAsync(sched, 0, sizeof(int), st) != cudaSuccess) return HCW_ERR_CUDA;
+    }
     int rc = launched(launch_tc_stack(MODE_DW, BN, T, total < sms ? total : sms, st), 1);
     if (rc) return rc;
     if (split)
@@ -1425,8 +1429,8 @@ int stack_weight_bf16(const Shape& sh, const StackWeight& a, cudaStream_t st) {
         p.seq_n = sh.n;
         p.timeout_ns = g_timeout_ns;
         T.n_layers = cnt;
-        T.sched = sched;
-        // the pair launch hands out its units statically (no unit counter); right
+        // the pair launch hands out its units statically, and so does one with a CTA for
+        // each (no unit counter); right
         // behind the fused launch it starts early, on the SMs that launch leaves
         const bool early = paired && a.fdx_counters != nullptr && L <= kMaxStackLayers;
         if (early) {
@@ -1434,10 +1438,12 @@ int stack_weight_bf16(const Shape& sh, const StackWeight& a, cudaStream_t st) {
             T.n_chunks = (int)((sh.tokens + 127) / 128);
             T.tokens = (int)sh.tokens;
             for (int i = 0; i < cnt; ++i) T.layer[i].dep_row = 2 * L - 2 - (l0 + i);
-        } else if (cudaMemsetAsync(sched, 0, sizeof(int), st) != cudaSuccess) {
-            return HCW_ERR_CUDA;
         }
         const int total = p.n_units * cnt;
+        if (!paired && total > sms) {
+            T.sched = sched;
+            if (cudaMemsetAsync(sched, 0, sizeof(int), st) != cudaSuccess) return HCW_ERR_CUDA;
+        }
         if (paired) {
             // clusters of two CTAs, one 256-row tile per cluster
             const int pairs = total / 2 < sms / 2 ? total / 2 : sms / 2;

@@ -172,6 +172,10 @@ __global__ void __launch_bounds__(kSmallThreads, D == 64 ? 2 : 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = bars->tmem_base;
+    // the prologue above touched no global memory: it overlaps the end of the kernel
+    // before it when launched as a programmatic dependent
+    pdl_wait();
+    pdl_trigger();
 
     if (warp == 0) {
         // ------------------------------------------------------------ weights
@@ -500,8 +504,7 @@ cudaError_t launch_small_t(const SmallLaunch& L, int sms, cudaStream_t st) {
     }
     const int blocks = (L.tokens + kTok - 1) / kTok;
     const int ctas = sms * (D == 64 ? 2 : 1);   // (two of the narrow kernel fit an SM)
-    kern<<<blocks < ctas ? blocks : ctas, kSmallThreads, smem, st>>>(L);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(blocks < ctas ? blocks : ctas), dim3(kSmallThreads), smem, st, L);
 }
 
 }  // namespace
