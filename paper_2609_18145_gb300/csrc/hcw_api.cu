@@ -241,7 +241,6 @@ bool map_f32_patches(CUtensorMap* m, const void* base, long long rows, int d) {
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int pick_bn(int d) { return d % 256 == 0 ? 256 : d % 128 == 0 ? 128 : 64; }
 
 // Widest column tile of the forward and input-gradient launches; the last tile of a d
 // that is not a multiple of it is ragged (its operand columns past d load as zeros, its
@@ -316,18 +315,50 @@ size_t mask_bytes(const Shape& sh) { return (size_t)sh.tokens * ((sh.d + 31) / 3
 
 // ------------------------------------------------------------ bf16 sizes
 struct WPlan {
+    int BN;   // column tile
     int n_ot, n_nt, qb, nkb_self, nkb_nbr, kb_per_unit, splits_self, splits_nbr, splits_max,
         units;
 };
+
+// Column tile of the weight gradients of `layers` layers in one launch; the last tile is
+// ragged where d is not a multiple of it (its operand columns past d load as zeros and
+// are not stored).  A unit's time is its operands' ingest, 128 + BN columns a token
+// block; a launch takes its waves of units, or, where the units split the token range to
+// fill one wave (split_dw_layers), their number.  Few tokens are bound by the units'
+// stores and latency and keep whole narrow tiles (16 layers of d = 576 over 512 tokens,
+// step: 341 us so, 349 ragged).  Steps before, with 64 columns, and so: 113,920 tokens, 6
+// layers of d = 448 2,398 and 1,454 us; 123,904 tokens, 7 of 704 5,225 and 3,438; 37,888
+// tokens, 3 of 320 351 and 251; 6,272 tokens, 18 of 704 836 and 713.
+int dw_bn(long long tokens, int d, int layers) {
+    if (d % 256 == 0) return 256;
+    if (tokens <= 2048) return d % 128 == 0 ? 128 : 64;
+    const int sms = sm_count(), rows = (d + 127) / 128;
+    int best = 64;
+    double best_t = 0;
+    for (int bn = 64; bn <= 256 && bn < 2 * d; bn *= 2) {
+        const int units = layers * rows * ((d + bn - 1) / bn);
+        double waves = (double)units / sms;
+        if (layers > 1 && units * 2 >= sms)
+            // self and partner part together in a unit, or apart in two
+            waves = 5 * units >= 3 * sms ? (units + sms - 1) / sms
+                                         : 0.5 * ((2 * units + sms - 1) / sms);
+        const double t = waves * (128 + bn);
+        if (bn == 64 || t <= best_t) {
+            best = bn;
+            best_t = t;
+        }
+    }
+    return best;
+}
 
 // The split of the token range of the weight gradient into units: one layer's,
 // or `layers` layers' sharing one launch.
 WPlan plan_dw(long long tokens, int d, unsigned flags, int layers = 1) {
     WPlan w;
-    const int BN = pick_bn(d);
+    w.BN = dw_bn(tokens, d, layers);
     const long long Mh = tokens / 2;
     w.n_ot = (d + 127) / 128;
-    w.n_nt = d / BN;
+    w.n_nt = (d + w.BN - 1) / w.BN;
     w.qb = (int)((Mh + 63) / 64);
     w.nkb_self = 2 * w.qb;
     w.nkb_nbr = (flags & HCW_CAUSAL) ? w.qb : 2 * w.qb;
@@ -360,10 +391,10 @@ WPlan plan_dw(long long tokens, int d, unsigned flags, int layers = 1) {
 // conditions of stack_weight_bf16 for one launch of <= kMaxStackLayers
 // layers), else 0.
 int dw_early_pairs(const Shape& sh, unsigned flags, int L) {
-    if (L > kMaxStackLayers || pick_bn(sh.d) < 128) return 0;
+    if (L > kMaxStackLayers || sh.d % 256 != 0) return 0;
     const WPlan w = plan_dw(sh.tokens, sh.d, flags);
     const int tiles = w.n_ot * w.n_nt, sms = sm_count();
-    if (L * tiles * 2 < sms || 5 * L * tiles < 3 * sms || w.n_ot % 2 != 0) return 0;
+    if (L * tiles * 2 < sms || 5 * L * tiles < 3 * sms) return 0;
     const int total = tiles * L;
     return total / 2 < sms / 2 ? total / 2 : sms / 2;
 }
@@ -703,9 +734,10 @@ int dx_bf16(const Shape& sh, const void* dz, const void* dy, const void* Ws, con
 // split has at least 256.  wws: weight workspace.
 int dw_bf16(const Shape& sh, const void* x, const void* dz, unsigned flags, float* dWs,
             float* dWn, float* dbias, uint8_t* wws, cudaStream_t st) {
-    const int d = sh.d, BN = pick_bn(d), k = 1 << sh.s;
+    const int d = sh.d, k = 1 << sh.s;
     const WsLayout lay = ws_layout(sh.tokens, d, HCW_BF16, flags);
     const WPlan w = plan_dw(sh.tokens, d, flags);
+    const int BN = w.BN;
     TcLaunch<1> L;
     memset(&L, 0, sizeof(L));
     CUtensorMap* maps = L.maps[0];
@@ -762,8 +794,9 @@ int dw_bf16(const Shape& sh, const void* x, const void* dz, unsigned flags, floa
 // (dW_self with a = dz; for a shift layer also dW_nbr, with a = the readers' dz).
 int dw_self_bf16(const Shape& sh, const void* x, const void* a, unsigned flags, float* dW,
                  uint8_t* wws, cudaStream_t st) {
-    const int d = sh.d, BN = pick_bn(d), k = 1 << sh.s;
+    const int d = sh.d, k = 1 << sh.s;
     const WPlan w = plan_dw(sh.tokens, d, flags);
+    const int BN = w.BN;
     TcLaunch<1> L;
     memset(&L, 0, sizeof(L));
     CUtensorMap* maps = L.maps[0];
@@ -947,7 +980,7 @@ size_t stack_data_ws(const Shape& sh, int dtype, unsigned flags, int L) {
 // tile) would leave most SMs idle: their launch then splits the token range
 // of every layer (split_dw_ws).
 bool split_dw_layers(const Shape& sh, unsigned flags, int cnt) {
-    const WPlan w = plan_dw(sh.tokens, sh.d, flags);
+    const WPlan w = plan_dw(sh.tokens, sh.d, flags, cnt);
     return cnt * w.n_ot * w.n_nt * 2 < sm_count();
 }
 
@@ -1230,9 +1263,10 @@ int stack_data_bf16(const Shape& sh, const StackData& a, cudaStream_t st) {
 // of stack_weight_bf16).
 int split_dw_launch(const Shape& sh, const StackWeight& a, int l0, int cnt, uint8_t* wws,
                     int* sched, cudaStream_t st) {
-    const int d = sh.d, BN = pick_bn(d);
+    const int d = sh.d;
     const size_t ab = sh.act_bytes, dd = (size_t)d * d;
     const WPlan w = plan_dw(sh.tokens, d, a.flags, cnt);
+    const int BN = w.BN;
     const bool split = w.splits_max > 1;
     const size_t part_floats = (size_t)2 * w.splits_max * dd;   // one layer's partials
     float* part = reinterpret_cast<float*>(wws);
@@ -1305,7 +1339,7 @@ int split_dw_launch(const Shape& sh, const StackWeight& a, int l0, int cnt, uint
 // schedule with shift layers that cannot take the batched launch runs layer
 // by layer.
 int stack_weight_bf16(const Shape& sh, const StackWeight& a, cudaStream_t st) {
-    const int d = sh.d, BN = pick_bn(d), L = a.L;
+    const int d = sh.d, L = a.L;
     const size_t ab = sh.act_bytes;
     const WsLayout wl = ws_layout(sh.tokens, d, HCW_BF16, a.flags);
     int* sched = reinterpret_cast<int*>(a.ws);
@@ -1313,7 +1347,7 @@ int stack_weight_bf16(const Shape& sh, const StackWeight& a, cudaStream_t st) {
     // from a (position, sample) view, 64 positions of one sample per stage,
     // hence n >= 128); otherwise every layer runs on its own.
     const WPlan wp = plan_dw(sh.tokens, d, a.flags);
-    const bool shift_batched = sh.n >= 128 && BN >= 128 && wp.n_ot % 2 == 0 && [&] {
+    const bool shift_batched = sh.n >= 128 && d % 256 == 0 && [&] {
         for (int l0 = 0; l0 < L; l0 += kMaxStackLayers) {
             const int cnt = L - l0 < kMaxStackLayers ? L - l0 : kMaxStackLayers;
             if (5 * cnt * wp.n_ot * wp.n_nt < 3 * sm_count()) return false;
@@ -1363,13 +1397,13 @@ int stack_weight_bf16(const Shape& sh, const StackWeight& a, cudaStream_t st) {
     auto act = [&](int l) -> const void* {
         return l == 0 ? a.x : static_cast<const uint8_t*>(a.acts) + (size_t)(l - 1) * ab;
     };
-    const WPlan w1 = plan_dw(sh.tokens, d, a.flags);
-    const int tiles = w1.n_ot * w1.n_nt;
     const int sms = sm_count();
     static thread_local TcLaunch<kMaxStackLayers> T;
     int rc;
     for (int l0 = 0; l0 < L; l0 += kMaxStackLayers) {
         const int cnt = L - l0 < kMaxStackLayers ? L - l0 : kMaxStackLayers;
+        const WPlan w1 = plan_dw(sh.tokens, d, a.flags, cnt);
+        const int tiles = w1.n_ot * w1.n_nt, BN = w1.BN;
         if (split_dw_layers(sh, a.flags, cnt)) {
             rc = split_dw_launch(sh, a, l0, cnt, wws, sched, st);
             if (rc) return rc;
@@ -1403,7 +1437,7 @@ int stack_weight_bf16(const Shape& sh, const StackWeight& a, cudaStream_t st) {
         // used when those units alone fill most of the GPU.  On pairs of SMs
         // (256-row tiles, cta_group::2) each SM takes in a third less per stage.
         const bool fused = 5 * cnt * tiles >= 3 * sms;
-        const bool paired = fused && BN >= 128 && w1.n_ot % 2 == 0;
+        const bool paired = fused && d % 256 == 0;
         if (paired)
             for (int i = 0; i < cnt; ++i) {
                 const int l = l0 + i;

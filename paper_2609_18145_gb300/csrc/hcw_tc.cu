@@ -1157,9 +1157,10 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                         uint32_t raw[32];
                         load_acc(which * BN + c * 32, raw);
                         if (which == 1 && c == WCOLS / 32 - 1) release_acc();
-                        if (row < p.d) {
+                        const int col = nt * BN + cslice * WCOLS + c * 32;
+                        if (row < p.d && col < p.d) {   // (ragged tiles)
                             float4* dst = reinterpret_cast<float4*>(
-                                base + (size_t)row * p.d + nt * BN + cslice * WCOLS + c * 32);
+                                base + (size_t)row * p.d + col);
 #pragma unroll
                             for (int m = 0; m < 8; ++m)
                                 dst[m] = make_float4(__uint_as_float(raw[4 * m]),
@@ -1545,9 +1546,10 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                         *patch_piece<128>(buf, lane, m) =
                             make_uint4(raw[4 * m], raw[4 * m + 1], raw[4 * m + 2], raw[4 * m + 3]);
                     publish();
-                    // d is a multiple of 64, so a warp's 32 rows are all inside or all
-                    // past the end (ragged o tile); the latter are not stored
-                    if (lane == 0 && w.ot * kBlockM + quarter * 32 < p.d) {
+                    // d is a multiple of 64, so a warp's 32 rows, and a patch's 32 columns,
+                    // are all inside or all past the end (ragged tiles); the latter are
+                    // not stored
+                    if (lane == 0 && w.ot * kBlockM + quarter * 32 < p.d && col0 + c * 32 < p.d) {
                         tma_store_2d(map, buf, col0 + c * 32, row0);
                         bulk_commit();
                     }
@@ -2092,11 +2094,8 @@ cudaError_t launch_tc_stack(int mode, int BN, const TcLaunch<kMaxStackLayers>& L
     if (mode == MODE_DWP) {
         bool shift = false;
         for (int i = 0; i < L.n_layers; ++i) shift = shift || L.layer[i].shift > 0;
-        if (BN == 256) return shift ? launch_pair<256, true>(L, grid, st)
-                                    : launch_pair<256, false>(L, grid, st);
-        if (BN == 128) return shift ? launch_pair<128, true>(L, grid, st)
-                                    : launch_pair<128, false>(L, grid, st);
-        return cudaErrorInvalidValue;
+        if (BN != 256) return cudaErrorInvalidValue;
+        return shift ? launch_pair<256, true>(L, grid, st) : launch_pair<256, false>(L, grid, st);
     }
 #define HCW_TC_STACK_CASE(M, N) \
     if (mode == M && BN == N) return launch_one<M, N, kMaxStackLayers>(L, grid, st);

@@ -1147,3 +1147,48 @@ def test_fp32_stack_in_one_launch_matches_its_layers(H, case):
     assert torch.equal(dx, g)
     torch.cuda.synchronize()
     assert H.hcw_sync_status() == H.HCW_OK
+
+
+# bf16 weight gradients whose last column tile is ragged: B, n, d, L, flags
+RAGGED_DW = [
+    (40, 64, 192, 2, CAUSAL),      # one tile of 256 columns, token splits
+    (20, 128, 320, 5, 0),          # two, the last a quarter full
+    (34, 64, 448, 16, CAUSAL),     # both parts in one unit
+    (33, 64, 576, 11, 0),
+    (33, 64, 320, 8, RELU),
+    (33, 64, 704, 5, 0),           # the parts apart
+    (33, 64, 384, 16, 0),
+    (33, 64, 704, 1, CAUSAL),
+    (4, 64, 320, 5, 0),            # few tokens: whole tiles
+]
+
+
+@pytest.mark.parametrize("case", RAGGED_DW, ids=lambda c: "B%d_n%d_d%d_L%d_f%d" % c)
+def test_ragged_weight_gradient_tiles(H, case):
+    """dW_self, dW_nbr and dbias of every layer against fp64 sums of the same bf16
+    values.  The products are exact in fp32; the sum of K = B n of them is off by at
+    most gamma_K (|dz|^T |x|), and the test allows four times that."""
+    B, n, d, L, flags = case
+    K, u32 = B * n, 2.0 ** -24
+    g = torch.Generator().manual_seed(d + L)
+    x = torch.randn(B, n, d, generator=g).to(torch.bfloat16).cuda()
+    acts = torch.randn(max(L - 1, 1), B, n, d, generator=g).to(torch.bfloat16).cuda()
+    dz = torch.randn(L, B, n, d, generator=g).to(torch.bfloat16).cuda()
+    gWs, gWn, gb = H.hcw_stack_bwd_weight(x, acts if L > 1 else None, dz, 1, -1, flags)
+    torch.cuda.synchronize()
+    assert H.hcw_sync_status() == H.HCW_OK
+    b = n.bit_length() - 1
+    i = torch.arange(n, device="cuda")
+    for l in range(L):
+        s = (1 + l) % b
+        xin = (x if l == 0 else acts[l - 1]).double()
+        dzl = dz[l].double()
+        recv = ((i >> s) & 1 if flags & CAUSAL else torch.ones_like(i)).double()[None, :, None]
+        xp = xin[:, i ^ (1 << s)] * recv
+        tol = 4 * (K + 2) * u32
+        for got, a in ((gWs[l], xin), (gWn[l], xp)):
+            f, r = dzl.reshape(K, d), a.reshape(K, d)
+            bound = tol * (f.abs().T @ r.abs()) + 1e-30
+            assert ((got.double() - f.T @ r).abs() <= bound).all()
+        ref = dzl.reshape(K, d)
+        assert ((gb[l].double() - ref.sum(0)).abs() <= tol * ref.abs().sum(0) + 1e-30).all()
