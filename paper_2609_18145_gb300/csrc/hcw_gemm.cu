@@ -13,12 +13,12 @@
 // 64-element rows (128-byte swizzle), an MN-major one as blocks of 64 rows of
 // 64 columns, which is the layout tcgen05 reads as an MN-major operand.
 //
-// A cluster of two CTAs (one per SM) computes 256 x 256 output tiles (256 x 128 in a
-// sparse last wave and past a narrow end of C) with
+// A cluster of two CTAs (one per SM) computes 256 x 256 output tiles (256 x 128
+// in a sparse last wave and past a narrow end of C) with
 // tcgen05.mma.cta_group::2: CTA r of the pair loads rows 128 r .. 128 r + 127
 // of the tile's A and columns 128 r .. 128 r + 127 of its B, so each SM takes
 // in 32 KB per 64-deep K step for 2 M multiply-adds.  In each CTA a producer
-// thread fills a ring of six stages, the leader's MMA thread issues the pair's
+// thread fills a ring of five stages, the leader's MMA thread issues the pair's
 // MMAs into a double-buffered TMEM accumulator (each CTA holds its 128 rows),
 // and eight warps drain the CTA's 128 x 256 fp32 results.  Tiles are handed
 // out round robin; a GEMM with few tiles and a long K (the weight gradients,

@@ -27,8 +27,8 @@
 // bias and ReLU, 500 without, bound by the warps' issue slots; the ReLU mask of dz 500;
 // A and A2 written 750, bound by shared-memory bandwidth; barriers 600).  Training
 // step of 16,384 tokens (n = 64, d = 128, 6 layers, without the causal rule): the forward
-// and input gradient 70.8 -> 37.9 us, the step 101 -> 64 us; a 20-layer causal forward of
-// 1,216 tokens 107 -> 58 us.
+// and input gradient 70.8 -> 37.9 us, the step 101 -> 64 us (55 as programmatic
+// dependents); a 20-layer causal forward of 1,216 tokens 107 -> 58 us.
 #include "hcw.h"
 #include "hcw_internal.h"
 #include "hcw_ptx.cuh"
