@@ -35,6 +35,8 @@ bool overlaps(const void* a, size_t na, const void* b, size_t nb) {
 
 size_t elem_size(int dtype) { return dtype == HCW_F32 ? 4 : 2; }
 
+size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
+
 int sm_count() {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 148;
@@ -320,6 +322,9 @@ struct WPlan {
         units;
 };
 
+// Scratch of the weight gradient without a workspace (hcw_layer_bwd_weight_noalloc).
+constexpr size_t kNoAllocScratchBytes = (size_t)32 << 20;   // 32 MiB
+
 // Column tile of the weight gradients of `layers` layers in one launch; the last tile is
 // ragged where d is not a multiple of it (its operand columns past d load as zeros and
 // are not stored).  A unit's time is its operands' ingest, 128 + BN columns a token
@@ -329,9 +334,10 @@ struct WPlan {
 // step: 341 us so, 349 ragged).  Steps before, with 64 columns, and so: 113,920 tokens, 6
 // layers of d = 448 2,398 and 1,454 us; 123,904 tokens, 7 of 704 5,225 and 3,438; 37,888
 // tokens, 3 of 320 351 and 251; 6,272 tokens, 18 of 704 836 and 713.
+int whole_bn(int d) { return d % 256 == 0 ? 256 : d % 128 == 0 ? 128 : 64; }
+
 int dw_bn(long long tokens, int d, int layers) {
-    if (d % 256 == 0) return 256;
-    if (tokens <= 2048) return d % 128 == 0 ? 128 : 64;
+    if (d % 256 == 0 || tokens <= 2048) return whole_bn(d);
     const int sms = sm_count(), rows = (d + 127) / 128;
     int best = 64;
     double best_t = 0;
@@ -351,11 +357,10 @@ int dw_bn(long long tokens, int d, int layers) {
     return best;
 }
 
-// The split of the token range of the weight gradient into units: one layer's,
-// or `layers` layers' sharing one launch.
-WPlan plan_dw(long long tokens, int d, unsigned flags, int layers = 1) {
+// The split of the token range of the weight gradient into units of column tile BN.
+WPlan split_dw(long long tokens, int d, unsigned flags, int layers, int BN) {
     WPlan w;
-    w.BN = dw_bn(tokens, d, layers);
+    w.BN = BN;
     const long long Mh = tokens / 2;
     w.n_ot = (d + 127) / 128;
     w.n_nt = (d + w.BN - 1) / w.BN;
@@ -386,6 +391,23 @@ WPlan plan_dw(long long tokens, int d, unsigned flags, int layers = 1) {
     return w;
 }
 
+// Partial sums of a layer's weight gradients.
+size_t dw_part_bytes(const WPlan& w, int d) {
+    return w.splits_max > 1 ? align256((size_t)2 * w.splits_max * d * d * 4) : 0;
+}
+
+// The split for one layer, or for `layers` layers sharing one launch.
+WPlan plan_dw(long long tokens, int d, unsigned flags, int layers = 1) {
+    const int BN = dw_bn(tokens, d, layers);
+    const WPlan w = split_dw(tokens, d, flags, layers, BN);
+    // Fewer, wider tiles are split more often, with more partial sums: sizes that fit
+    // the scratch of the call without a workspace with whole tiles keep fitting it.
+    if (layers == 1 && BN != whole_bn(d) &&
+        dw_part_bytes(w, d) + align256(colsum_workspace_bytes(tokens, d)) > kNoAllocScratchBytes)
+        return split_dw(tokens, d, flags, layers, whole_bn(d));
+    return w;
+}
+
 // SM pairs of the batched weight-gradient launch of a training step when it
 // runs on pairs behind the fused forward / input-gradient launch (the
 // conditions of stack_weight_bf16 for one launch of <= kMaxStackLayers
@@ -406,8 +428,6 @@ int dw_early_pairs(const Shape& sh, unsigned flags, int L) {
 struct WsLayout {
     size_t dz_off, dz_bytes, w_off, part_bytes, col_off, col_bytes, w_bytes, total;
 };
-
-size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // Partial sums of the fp32 weight gradients of `layers` layers (dw_f32).
 size_t f32_part_bytes(long long tokens, int d, int layers) {
@@ -431,8 +451,7 @@ WsLayout ws_layout(long long tokens, int d, int dtype, unsigned flags) {
     l.dz_bytes = (flags & HCW_ACT_RELU) ? align256((size_t)tokens * d * es) : 0;
     l.w_off = l.dz_off + l.dz_bytes;
     if (dtype == HCW_BF16 && tokens > 0) {
-        WPlan w = plan_dw(tokens, d, flags);
-        l.part_bytes = (w.splits_max > 1) ? align256((size_t)2 * w.splits_max * d * d * 4) : 0;
+        l.part_bytes = dw_part_bytes(plan_dw(tokens, d, flags), d);
     } else {
         l.part_bytes = 0;
     }
@@ -2551,7 +2570,6 @@ int hcw_selftest_wait(long long timeout_ns, void* stream) {
 // sums of dW and column-sum partials of dbias), so this variant keeps that
 // scratch in a fixed array linked into the library instead.  Every device
 // that loads the library reserves the array until the process exits.
-static constexpr size_t kNoAllocScratchBytes = (size_t)32 << 20;   // 32 MiB
 static __device__ __align__(256) unsigned char hcw_noalloc_scratch[kNoAllocScratchBytes];
 
 namespace {

@@ -157,6 +157,18 @@ def test_weight_gradient_rejects_dbias_over_its_inputs(hcw):
     assert ws(W + 16) == hcw.HCW_ERR_ALIASING                # inside the workspace
 
 
+@pytest.mark.parametrize("B,n,d", [(400, 4096, 704), (512, 8192, 320), (280, 4096, 832),
+                                   (600, 2048, 960), (400, 4096, 448), (3, 2048, 192)])
+def test_ragged_weight_gradients_fit_the_fixed_scratch(hcw, B, n, d):
+    """A d that 256 does not divide: the wider column tiles, with their more partial
+    sums, are not taken where a layer's scratch would outgrow the 32 MiB of the call
+    without a workspace (whole 64- or 128-column tiles fit it at these sizes)."""
+    for flags in (0, hcw.HCW_CAUSAL):
+        rc = hcw.lib().hcw_layer_bwd_weight_noalloc(None, None, 0, -1, B, n, d, hcw.HCW_BF16,
+                                                    flags, None, None, None, None)
+        assert rc == hcw.HCW_ERR_INVALID_ARG     # the pointers, not the size
+
+
 def test_workspace_sizes_f32(hcw):
     a = hcw.hcw_workspace_bytes(64, 256, 512, hcw.HCW_F32, 0)
     b = hcw.hcw_workspace_bytes(64, 256, 512, hcw.HCW_F32, hcw.HCW_ACT_RELU)
