@@ -201,9 +201,10 @@ __global__ void __launch_bounds__(256)
 // way into a ring of shared-memory buffers while one is computed.  Layer by layer these
 // stacks are bound by launches, about 4 us each: four layers forward and backward at 64
 // rows of d = 32 took 46 us a call of each, now 29 (the host's part), 19 of them on the
-// GPU.  A lane per output column, kChainRows rows per warp at a time, and the products in
-// the order of the tiled kernels: the same bits.  A layer is bound by shared-memory reads
-// (ten 16-byte ones for 32 products a lane), 0.7 us at 16 rows of d = 32.
+// GPU.  One or two output columns a lane, kChainRows rows per warp at a time, and the
+// products in the order of the tiled kernels: the same bits.  A layer is bound by
+// shared-memory reads (ten 16-byte ones for 32 products a lane, twelve for 64 with two
+// columns), 0.7 us at 16 rows of d = 32.
 constexpr int kChainRows = 4;
 constexpr size_t kChainSmem = 232448;
 
@@ -232,7 +233,8 @@ __host__ __device__ inline size_t chain_floats(int d, int rows, int stages) {
 
 // BWD false: x through layers 0 .. L-1 to acts, y and the mask words.  BWD true: dy down
 // through layers L-1 .. 0 to every layer's dz and dx.
-template <bool BWD>
+// NC: output columns a lane, 32 apart.
+template <bool BWD, int NC>
 __global__ void __launch_bounds__(256) f32_chain_kernel(const __grid_constant__ F32ChainArgs A) {
     extern __shared__ float4 chain_smem[];
     float* smem = reinterpret_cast<float*>(chain_smem);
@@ -310,11 +312,12 @@ __global__ void __launch_bounds__(256) f32_chain_kernel(const __grid_constant__ 
             for (int r = prow; r < rows; r += prows) row(r, A.in[(r0 + r) * d + pcol]);
     }
 
-    const int cwarps = wpr, groups = 8 / cwarps;   // column warps, row groups
-    const int cw = warp % cwarps, grp = warp / cwarps;
-    const int c = cw * 32 + lane;
-    const bool col_ok = c < d;
-    const int cc = col_ok ? c : 0;
+    const int cwarps = (wpr + NC - 1) / NC, groups = 8 / cwarps;   // column warps, row groups
+    const int cw = (warp % cwarps) * NC, grp = warp / cwarps;      // first mask word, group
+    const int c0 = cw * 32 + lane;
+    int cc[NC];
+#pragma unroll
+    for (int h = 0; h < NC; ++h) cc[h] = c0 + 32 * h < d ? c0 + 32 * h : 0;
     for (int i = 0; i < A.L; ++i) {
         const int l = BWD ? A.L - 1 - i : i;
         if (A.stages == 4)
@@ -331,11 +334,13 @@ __global__ void __launch_bounds__(256) f32_chain_kernel(const __grid_constant__ 
         float* next = xbuf + ((i + 1) & 1) * xsz;
         const int s = A.s[l];
         const bool last = i + 1 == A.L;
-        const float bias = !BWD && A.bias ? aux[cc] : 0.f;
+        float bias[NC];
+#pragma unroll
+        for (int h = 0; h < NC; ++h) bias[h] = !BWD && A.bias ? aux[cc[h]] : 0.f;
         if (grp < groups)
             for (int rb = grp * kChainRows; rb < rows; rb += groups * kChainRows) {
                 int xr[kChainRows], pr[kChainRows];   // rows' offsets in shared memory
-                uint32_t mw[kChainRows];
+                uint32_t mw[NC][kChainRows];
 #pragma unroll
                 for (int q = 0; q < kChainRows; ++q) {
                     const int rr = rb + q, j = rr & (n - 1);
@@ -348,28 +353,35 @@ __global__ void __launch_bounds__(256) f32_chain_kernel(const __grid_constant__ 
                     }
                     xr[q] = rr < rows ? curo + rr * ld : zero;
                     pr[q] = from >= 0 ? curo + (rr - j + from) * ld : zero;
-                    mw[q] = BWD && relu && !last && rr < rows
-                                ? reinterpret_cast<const uint32_t*>(aux)[rr * wpr + cw]
-                                : ~0u;
+#pragma unroll
+                    for (int h = 0; h < NC; ++h)
+                        mw[h][q] = BWD && relu && !last && rr < rows && cw + h < wpr
+                                       ? reinterpret_cast<const uint32_t*>(aux)[rr * wpr + cw + h]
+                                       : ~0u;
                 }
-                float acc[kChainRows];
+                float acc[NC][kChainRows];
 #pragma unroll
-                for (int q = 0; q < kChainRows; ++q) acc[q] = 0.f;
-#pragma unroll 4
+                for (int h = 0; h < NC; ++h)
+#pragma unroll
+                    for (int q = 0; q < kChainRows; ++q) acc[h][q] = 0.f;
+#pragma unroll(NC == 1 ? 4 : 2)
                 for (int k = 0; k < d4; k += 4) {
-                    float u[4], v[4];
+                    float u[NC][4], v[NC][4];
                     float4 xv[kChainRows], pv[kChainRows];
-                    if (BWD) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            u[j] = ws[(k + j) * ld + cc];
-                            v[j] = wn[(k + j) * ld + cc];
+                    for (int h = 0; h < NC; ++h) {
+                        if (BWD) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                u[h][j] = ws[(k + j) * ld + cc[h]];
+                                v[h][j] = wn[(k + j) * ld + cc[h]];
+                            }
+                        } else {
+                            const float4 a = *reinterpret_cast<const float4*>(ws + cc[h] * ld + k);
+                            const float4 b = *reinterpret_cast<const float4*>(wn + cc[h] * ld + k);
+                            u[h][0] = a.x, u[h][1] = a.y, u[h][2] = a.z, u[h][3] = a.w;
+                            v[h][0] = b.x, v[h][1] = b.y, v[h][2] = b.z, v[h][3] = b.w;
                         }
-                    } else {
-                        const float4 a = *reinterpret_cast<const float4*>(ws + cc * ld + k);
-                        const float4 b = *reinterpret_cast<const float4*>(wn + cc * ld + k);
-                        u[0] = a.x, u[1] = a.y, u[2] = a.z, u[3] = a.w;
-                        v[0] = b.x, v[1] = b.y, v[2] = b.z, v[3] = b.w;
                     }
 #pragma unroll
                     for (int q = 0; q < kChainRows; ++q) {
@@ -378,9 +390,15 @@ __global__ void __launch_bounds__(256) f32_chain_kernel(const __grid_constant__ 
                     }
                     auto step = [&](auto at, int j) {
 #pragma unroll
-                        for (int q = 0; q < kChainRows; ++q) acc[q] = fmaf(at(xv[q]), u[j], acc[q]);
+                        for (int h = 0; h < NC; ++h)
 #pragma unroll
-                        for (int q = 0; q < kChainRows; ++q) acc[q] = fmaf(at(pv[q]), v[j], acc[q]);
+                            for (int q = 0; q < kChainRows; ++q)
+                                acc[h][q] = fmaf(at(xv[q]), u[h][j], acc[h][q]);
+#pragma unroll
+                        for (int h = 0; h < NC; ++h)
+#pragma unroll
+                            for (int q = 0; q < kChainRows; ++q)
+                                acc[h][q] = fmaf(at(pv[q]), v[h][j], acc[h][q]);
                     };
                     step([](const float4& f) { return f.x; }, 0);
                     step([](const float4& f) { return f.y; }, 1);
@@ -391,34 +409,41 @@ __global__ void __launch_bounds__(256) f32_chain_kernel(const __grid_constant__ 
                 for (int q = 0; q < kChainRows; ++q) {
                     const int rr = rb + q;
                     if (rr >= rows) break;   // warp-uniform
-                    const size_t at = (r0 + rr) * d + c;
-                    if (BWD) {
-                        float v = acc[q];
-                        if (!col_ok) continue;
-                        if (res) v += gbuf[rr * ld + c];
-                        gbuf[rr * ld + c] = v;
-                        if (last) {
-                            A.out[at] = v;
+#pragma unroll
+                    for (int h = 0; h < NC; ++h) {
+                        if (cw + h >= wpr) break;   // warp-uniform
+                        const int c = c0 + 32 * h;
+                        const bool col_ok = c < d;
+                        const size_t at = (r0 + rr) * d + c;
+                        if (BWD) {
+                            float v = acc[h][q];
+                            if (!col_ok) continue;
+                            if (res) v += gbuf[rr * ld + c];
+                            gbuf[rr * ld + c] = v;
+                            if (last) {
+                                A.out[at] = v;
+                            } else {
+                                v = (mw[h][q] >> lane) & 1u ? v : 0.f;
+                                next[rr * ld + c] = v;
+                                A.acts[(size_t)(l - 1) * A.act_elems + at] = v;
+                            }
                         } else {
-                            v = (mw[q] >> lane) & 1u ? v : 0.f;
-                            next[rr * ld + c] = v;
-                            A.acts[(size_t)(l - 1) * A.act_elems + at] = v;
-                        }
-                    } else {
-                        float v = col_ok ? acc[q] + bias : 0.f;
-                        if (A.mask_out) {
-                            const unsigned bits = __ballot_sync(0xffffffffu, v > 0.f);
-                            if (lane == 0)
-                                A.mask_out[(size_t)l * A.mask_words + (r0 + rr) * wpr + cw] = bits;
-                        }
-                        if (!col_ok) continue;
-                        if (relu) v = v > 0.f ? v : 0.f;
-                        if (res) v += cur[rr * ld + c];
-                        if (last) {
-                            A.out[at] = v;
-                        } else {
-                            next[rr * ld + c] = v;
-                            A.acts[(size_t)l * A.act_elems + at] = v;
+                            float v = col_ok ? acc[h][q] + bias[h] : 0.f;
+                            if (A.mask_out) {
+                                const unsigned bits = __ballot_sync(0xffffffffu, v > 0.f);
+                                if (lane == 0)
+                                    A.mask_out[(size_t)l * A.mask_words + (r0 + rr) * wpr + cw + h] =
+                                        bits;
+                            }
+                            if (!col_ok) continue;
+                            if (relu) v = v > 0.f ? v : 0.f;
+                            if (res) v += cur[rr * ld + c];
+                            if (last) {
+                                A.out[at] = v;
+                            } else {
+                                next[rr * ld + c] = v;
+                                A.acts[(size_t)l * A.act_elems + at] = v;
+                            }
                         }
                     }
                 }
@@ -825,13 +850,23 @@ cudaError_t launch_f32_dw(F32DwArgs& a, int layers, int splits, cudaStream_t st,
     return e;
 }
 
+// Output columns a lane of the one launch: two, which halves the reads of x a product,
+// where one would take the rows in more than one pass (n = 16, 64 rows, graphs of four
+// layers forward and backward: d = 112 82 us, two columns 58; 4,096 rows of d = 64 86 and
+// 76; but one window of two rows and d = 64 23 and 27).
+static int chain_cols(int d, int rows) {
+    const int cols = (d + 31) / 32;
+    return cols > 1 && rows > kChainRows * (8 / cols) ? 2 : 1;
+}
+
 // The windows a block of the one launch takes, one wave of blocks, where a layer costs
 // it less than its own launch does.  Both sides in us a layer and direction, fitted to
 // four layers forward and backward (graphs; us layer by layer, in one launch): n = 16,
-// 64 rows: d = 16 35.6, 17.1; d = 32 36.2, 18.8; d = 64 52.7, 30.2; d = 91 67.3, 71;
-// d = 96 67, 59.  4,096 rows: d = 32 44.4, 35.0; d = 64 128, 85; d = 96 235, 177.
-// n = 64, 64 rows: d = 32 36.1, 34.3; d = 48 52, 73.  n = 256: one window is too much
-// for a block from d = 16 on (42, 83) unless there are many (64 windows: 113, 104).
+// 64 rows: d = 16 35.6, 16.6; d = 32 36.2, 18.6; d = 64 52.7, 30.5; d = 91 67, 65; d = 96
+// 67, 51; 1,024 rows of d = 91 77, 81.  4,096 rows: d = 32 44.4, 35.7; d = 64 128, 76;
+// d = 96 235, 160.  n = 64, 64 rows: d = 32 36.1, 34.3; d = 48 52, 56; 4,096 rows of
+// d = 64 122, 93.  n = 256: one window is too much for a block from d = 16 on (41, 80)
+// unless there are many (64 windows of d = 48: 348, 295).
 int f32_chain_rows(long long rows, int n, int d, int L, int sms) {
     if (L < 2 || L > kMaxF32Layers || d > 128) return 0;
     const long long windows = rows / n;
@@ -839,16 +874,17 @@ int f32_chain_rows(long long rows, int n, int d, int L, int sms) {
     if (per * n > 4096) return 0;
     const int R = (int)(per * n);
     if (chain_floats(d, R, 2) * sizeof(float) > kChainSmem) return 0;
-    const int cols = (d + 31) / 32, groups = 8 / cols;
+    const int cols = (d + 31) / 32, nc = chain_cols(d, R), groups = 8 / ((cols + nc - 1) / nc);
     const int passes = (R + kChainRows * groups - 1) / (kChainRows * groups);
-    double chain = passes * (0.5 + 0.17 * ((d + 3) / 4) * (cols * groups / 8.0));
-    if (d % 4) chain *= 1.25;   // weights copied 4 bytes at a time
+    const double step = nc == 1 ? 0.17 * (cols * groups / 8.0) : 0.2;   // of four k
+    double chain = passes * (0.5 + step * ((d + 3) / 4));
+    if (d % 4) chain *= 1.5;   // weights copied 4 bytes at a time
     const double steps = (double)((rows + T - 1) / T) * cols * cols;   // of all tiles
     const double one = 1.05 * (1.8 + 1.75 * cols), many = 1.0 + 0.0185 * steps;
     return chain < (one > many ? one : many) ? R : 0;
 }
 
-template <bool BWD>
+template <bool BWD, int NC>
 static cudaError_t launch_chain(const F32ChainArgs& a, cudaStream_t st) {
     static std::once_flag once[64];
     static cudaError_t set_err[64];
@@ -857,13 +893,13 @@ static cudaError_t launch_chain(const F32ChainArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::call_once(once[dev], [&] {
-        set_err[dev] = cudaFuncSetAttribute(f32_chain_kernel<BWD>,
+        set_err[dev] = cudaFuncSetAttribute(f32_chain_kernel<BWD, NC>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)kChainSmem);
     });
     if (set_err[dev] != cudaSuccess) return set_err[dev];
     const unsigned grid = (unsigned)((a.rows + a.block_rows - 1) / a.block_rows);
-    return launch_pdl(f32_chain_kernel<BWD>, dim3(grid), dim3(256),
+    return launch_pdl(f32_chain_kernel<BWD, NC>, dim3(grid), dim3(256),
                       chain_floats(a.d, a.block_rows, a.stages) * sizeof(float), st, a);
 }
 
@@ -876,7 +912,9 @@ cudaError_t launch_f32_chain(F32ChainArgs& a, bool bwd, cudaStream_t st) {
     a.lanes_log2 = 0;
     while ((1 << a.lanes_log2) < pieces) ++a.lanes_log2;
     a.stages = a.L > 2 && chain_floats(a.d, a.block_rows, 4) * sizeof(float) <= kChainSmem ? 4 : 2;
-    return bwd ? launch_chain<true>(a, st) : launch_chain<false>(a, st);
+    if (chain_cols(a.d, a.block_rows) == 1)
+        return bwd ? launch_chain<true, 1>(a, st) : launch_chain<false, 1>(a, st);
+    return bwd ? launch_chain<true, 2>(a, st) : launch_chain<false, 2>(a, st);
 }
 
 cudaError_t launch_relu_grad_f32(const float* dy, const float* z, float* dz, size_t count,

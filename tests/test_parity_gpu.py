@@ -1111,6 +1111,8 @@ CHAINS = [
     (2, 16, 96, RESIDUAL | RELU, (3, 0, 2, 1, 3)),      # a ring of two buffers
     (400, 16, 33, RESIDUAL, (1, 2, 3, 0, 1, 2)),        # three windows a block, the last fewer
     (3, 8, 112, CAUSAL | RESIDUAL, (0, 1, 2)),          # the widest
+    (200, 16, 70, CAUSAL | RESIDUAL | RELU, (0, 2, -5, 3)),   # two columns a lane, ragged
+    (4, 16, 112, RELU, (3, 1, 0)),
 ]
 
 
