@@ -288,7 +288,9 @@ __device__ __forceinline__ void pdl_trigger() {
 
 // Launch `kern` with programmatic stream serialization: it may start while the
 // kernel before it in the stream finishes, and must call pdl_wait()
-// before it touches memory that kernel reads or writes.
+// before it touches memory that kernel reads or writes.  It must call it in any case,
+// before it ends: the wait of the kernel behind it covers this kernel alone, and what
+// this one depends on only through it.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t st, Args... args) {

@@ -1990,6 +1990,10 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
         __syncwarp();
     }
 
+    // The counters cover the dz this launch reads, not the fused launch's last work (dx,
+    // the masks).  A kernel behind this one waits for this one alone, so this one must
+    // not complete before the fused launch has.
+    pdl_wait();
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();   // neither CTA frees the pair's TMEM while the other uses it

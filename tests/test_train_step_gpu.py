@@ -100,6 +100,31 @@ def test_train_step_rejects_overlapping_dy(H):
     assert e.value.status == H.HCW_ERR_ALIASING
 
 
+@pytest.mark.parametrize("B, n", [(2, 256), (4, 128), (4, 256)])
+def test_calls_behind_a_step_see_its_finished_outputs(H, B, n):
+    """With few tokens the weight gradient, which starts behind the fused launch and waits
+    for dz alone, may run out of work before the last layer's input gradient does.  Single
+    layers, programmatic dependents of it, then read dx: enqueued right behind the step they
+    give the bits of a run that waits in between."""
+    d, L, flags = 512, 16, CAUSAL | RESIDUAL | RELU
+    _, x, Ws, Wn, dy, bias = problem(B, n, d, L, seed=14)
+
+    def run(wait):
+        step = H.hcw_stack_train_step(x, Ws, Wn, bias, dy, 0, -1, flags)
+        if wait:
+            torch.cuda.synchronize()
+        dx = step[3]
+        y, z = H.hcw_layer_fwd(dx, Ws[0], Wn[0], bias[0], 0, -1, flags, want_z=True)
+        return [dx, y, z] + list(H.hcw_layer_bwd(x, z, dx, Ws[0], Wn[0], 0, -1, flags))
+
+    ref = run(True)
+    for _ in range(10):
+        got = run(False)
+        for i, (a, b) in enumerate(zip(got, ref)):
+            assert torch.equal(a, b), i
+    assert H.hcw_sync_status() == H.HCW_OK
+
+
 DIMS_CASES = [
     # B, n, d, flags, dims (-k: a shift of Eq. (1) by k)
     (4, 256, 512, CAUSAL | RESIDUAL | RELU, [-1, 7, -1, -1, 5, -1, 4, -1, -1, 2, -1, 1, -1, 0]),
