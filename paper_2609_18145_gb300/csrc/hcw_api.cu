@@ -634,6 +634,14 @@ int small_launch(const Shape& sh, const Sched& sc, int L, unsigned flags, const 
     return launched(launch_small(S, d, sm_count(), st), 1);
 }
 
+// A g buffer whose lines may be discarded (TcLayer::g_discard): rows are multiples of 128
+// bytes, so all start on a line if the first does, as they do not in a workspace that is
+// only 16-byte aligned.
+const __nv_bfloat16* discardable(const void* g) {
+    return (reinterpret_cast<uintptr_t>(g) & 127) == 0 ? static_cast<const __nv_bfloat16*>(g)
+                                                       : nullptr;
+}
+
 // Row-unit geometry of a pair launch: units count row-block pairs.
 void pair_units(TcParams& p) { p.n_units = ((p.n_rb + 1) / 2) * p.n_nt * 2; }
 
@@ -1241,8 +1249,7 @@ int stack_data_bf16(const Shape& sh, const StackData& a, cudaStream_t st) {
                           dzo ? mask(l - 1) : nullptr, dzo != nullptr};
             T.layer[i].shift = sl < 0 ? -sl : 0;
             // the g buffers written by this launch (not dy, not a previous launch's)
-            if (keep_g && i > 0)
-                T.layer[i].g_discard = static_cast<const __nv_bfloat16*>(res);
+            if (keep_g && i > 0) T.layer[i].g_discard = discardable(res);
         }
         row_unit_params(T.p, sh, BN, a.flags, true);
         if (pair) pair_units(T.p);
@@ -1957,7 +1964,7 @@ int step_fused_launch(const Shape& sh, const void* x, const uint8_t* Ws, const u
                           dzo ? mask(l - 1) : nullptr, dzo != nullptr};
         T.layer[L + i].shift = sl < 0 ? -sl : 0;
         // the g buffers written by this launch (not dy)
-        if (keep_g && i > 0) T.layer[L + i].g_discard = static_cast<const __nv_bfloat16*>(res);
+        if (keep_g && i > 0) T.layer[L + i].g_discard = discardable(res);
     }
     row_unit_params(T.p, sh, BN, flags, false);
     pair_units(T.p);

@@ -73,7 +73,8 @@ struct TcLayer {
     // DX of a stacked launch: the residual term (map 3) when it is one of the
     // launch's own g buffers, [tokens][d] bf16; each epilogue warp discards its
     // patch's L2 lines once it has read them (nothing reads them again, and
-    // the buffer is written anew two layers later), or null
+    // the buffer is written anew two layers later), or null (also where the buffer
+    // does not start on a line)
     const __nv_bfloat16* g_discard;
     // A shift layer of Eq. (1) by `shift` positions (0: a hypercube layer).
     // MODE_DWP: its rows are grouped as a hypercube view with k = 64 (64

@@ -136,6 +136,36 @@ def test_an_id_outside_the_vocabulary_is_reported(H):
     assert H.hcw_sync_status() == H.HCW_OK      # the report is read once
 
 
+@pytest.mark.parametrize("offset", [16, 64])
+@pytest.mark.parametrize("case", [(4, 64, 128, 256, 37, 3), (2, 64, 192, 384, 130, 2)],
+                         ids=lambda c: "B%d_n%d_d%d_h%d_V%d_L%d" % c)
+def test_a_workspace_off_a_line_changes_nothing(H, case, offset):
+    """The workspace need only be 16-byte aligned: where rows do not start on a 128-byte
+    line, no line that they share with others may be dropped.  The gradients without atomic
+    additions keep their bits; the others (and the loss) are sums of at most B n terms in an
+    order that varies: 2 u B n of their largest entry at most."""
+    B, n, d, h, V, L = case
+    ids, params, _ = device_problem(synth.block_problem(B, n, d, h, V, L, seed=10))
+    need = H.hcw_block_workspace_bytes(B, n, d, h, V, L)
+    buf = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+    assert buf.data_ptr() % 128 == 0
+
+    def run(at):
+        loss, grads = H.hcw_block_step(ids, params, workspace=buf[at:at + need])
+        return dict({f: g.clone() for f, g in grads.items()}, loss=loss.clone())
+
+    ref = run(0)
+    for _ in range(3):
+        got = run(offset)
+        for f, a in got.items():
+            if f in ("E", "b1", "bh", "loss"):
+                tol = 2 * 2.0 ** -24 * B * n * float(ref[f].abs().max())
+                assert float((a - ref[f]).abs().max()) <= tol, f
+            else:
+                assert torch.equal(a, ref[f]), f
+    assert H.hcw_sync_status() == H.HCW_OK
+
+
 def test_full_size_batch_is_the_weighted_sum_of_its_parts(H):
     """Window 256, d = 512, h = 1024, V = 256, 16 layers, B = 64 (the metric's
     shape): sequences are independent, so the batch's loss and gradients are

@@ -125,6 +125,31 @@ def test_calls_behind_a_step_see_its_finished_outputs(H, B, n):
     assert H.hcw_sync_status() == H.HCW_OK
 
 
+@pytest.mark.parametrize("offset", [16, 64])
+@pytest.mark.parametrize("B, n, d, L", [(4, 256, 512, 6), (33, 256, 320, 4), (2, 256, 256, 5)])
+def test_a_workspace_off_a_line_keeps_the_bits(H, B, n, d, L, offset):
+    """The workspace need only be 16-byte aligned: where the g buffers' rows do not start on
+    a 128-byte line, no line that they share with others may be dropped (the step, and the
+    input gradient on its own)."""
+    flags = RESIDUAL | RELU
+    _, x, Ws, Wn, dy, bias = problem(B, n, d, L, seed=15)
+    need = H.hcw_stack_train_step_workspace_bytes(B, n, d, H.HCW_BF16, flags, L)
+    buf = torch.empty(need + 256, dtype=torch.uint8, device="cuda")
+    assert buf.data_ptr() % 128 == 0
+
+    def run(at):
+        ws = buf[at:at + need]
+        step = H.hcw_stack_train_step(x, Ws, Wn, bias, dy, 0, -1, flags, workspace=ws)
+        return list(step) + list(H.hcw_stack_bwd_data(step[2], dy, Ws, Wn, 0, -1, flags,
+                                                      workspace=ws))
+
+    ref = run(0)
+    for _ in range(3):
+        for i, (a, b) in enumerate(zip(run(offset), ref)):
+            assert torch.equal(a, b), i
+    assert H.hcw_sync_status() == H.HCW_OK
+
+
 DIMS_CASES = [
     # B, n, d, flags, dims (-k: a shift of Eq. (1) by k)
     (4, 256, 512, CAUSAL | RESIDUAL | RELU, [-1, 7, -1, -1, 5, -1, 4, -1, -1, 2, -1, 1, -1, 0]),
