@@ -1769,9 +1769,14 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                 if (issued_mask & (1u << s))
                     mbar_wait_drain(&bars->full[s], (issued_phase >> s) & 1u, tmo);
         }
+    } else if (warp == 1 && rank != 0) {
+        // The counters cover the dz this launch reads, not the fused launch's last work
+        // (dx, the masks).  A kernel behind this one waits for this one alone, so this one
+        // must not complete before the fused launch has: the warp without work waits for it.
+        pdl_wait();
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (leader)
-        if (lane == 0 && rank == 0) {
+        if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true, any = false;
@@ -1990,10 +1995,6 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
         __syncwarp();
     }
 
-    // The counters cover the dz this launch reads, not the fused launch's last work (dx,
-    // the masks).  A kernel behind this one waits for this one alone, so this one must
-    // not complete before the fused launch has.
-    pdl_wait();
     tc_fence_before();
     __syncthreads();
     cluster_sync_all();   // neither CTA frees the pair's TMEM while the other uses it
