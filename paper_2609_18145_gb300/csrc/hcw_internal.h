@@ -291,7 +291,9 @@ __device__ __forceinline__ void pdl_trigger() {
 // kernel before it in the stream finishes, and must call pdl_wait()
 // before it touches memory that kernel reads or writes.  It must call it in any case,
 // before it ends: the wait of the kernel behind it covers this kernel alone, and what
-// this one depends on only through it.
+// this one depends on only through it.  Its pointers carry no __restrict__, and what the
+// kernel before may write it reads with plain loads: that is still being written while this
+// one lives, which the read-only path (const __restrict__, __ldg) does not allow.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t st, Args... args) {

@@ -47,10 +47,9 @@ constexpr int T = 32;   // tile edge of the fp32 kernels
 // z[r][o] = sum_k Ws[o][k] x[r][k] + m_r sum_k Wn[o][k] x[p(r)][k] + bias[o]
 // mout (optional): ReLU mask words [rows][ceil(d/32)], bit o%32 of word o/32 = (z > 0).
 __global__ void __launch_bounds__(256)
-    f32_fwd_kernel(const float* __restrict__ x, const float* __restrict__ Ws,
-                   const float* __restrict__ Wn, const float* __restrict__ bias, int s, int n,
-                   int d, long long rows, unsigned flags, float* __restrict__ y,
-                   float* __restrict__ z, uint32_t* __restrict__ mout) {
+    f32_fwd_kernel(const float* x, const float* Ws, const float* Wn, const float* bias, int s,
+                   int n, int d, long long rows, unsigned flags, float* y, float* z,
+                   uint32_t* mout) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
     __shared__ float xs[T][T + 1], xp[T][T + 1], ws[T][T + 1], wn[T][T + 1];
@@ -125,10 +124,9 @@ __global__ void __launch_bounds__(256)
 // written to dx (if given) and, where the mask bits mprev of the layer below are set
 // (else 0), to dz_prev (if given).
 __global__ void __launch_bounds__(256)
-    f32_dx_kernel(const float* __restrict__ dz, const float* __restrict__ dy,
-                  const float* __restrict__ Ws, const float* __restrict__ Wn, int s, int n, int d,
-                  long long rows, unsigned flags, float* __restrict__ dx,
-                  const uint32_t* __restrict__ mprev, float* __restrict__ dz_prev) {
+    f32_dx_kernel(const float* dz, const float* dy, const float* Ws, const float* Wn, int s, int n,
+                  int d, long long rows, unsigned flags, float* dx, const uint32_t* mprev,
+                  float* dz_prev) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
     __shared__ float gs[T][T + 1], gp[T][T + 1], ws[T][T + 1], wn[T][T + 1];
@@ -464,8 +462,8 @@ __global__ void __launch_bounds__(256) f32_dw_kernel(const __grid_constant__ F32
     const int l = blockIdx.z / A.splits, sp = blockIdx.z - l * A.splits;
     const int n = A.n, d = A.d, s = A.s[l];
     const unsigned flags = A.flags;
-    const float* __restrict__ x = l == 0 ? A.x : A.acts + (l - 1) * A.act_elems;
-    const float* __restrict__ dz = A.dz + l * A.act_elems;
+    const float* x = l == 0 ? A.x : A.acts + (l - 1) * A.act_elems;
+    const float* dz = A.dz + l * A.act_elems;
     const long long rb = (long long)sp * A.rows_per_split;
     const long long re = rb + A.rows_per_split < A.rows ? rb + A.rows_per_split : A.rows;
     const int o0 = blockIdx.y * T, k0 = blockIdx.x * T;
@@ -569,8 +567,7 @@ __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 v) {
 // element a thread and access, 13 us so.
 template <typename V>
 __global__ void __launch_bounds__(256)
-    relu_grad_kernel(const V* __restrict__ dy, const V* __restrict__ z, V* __restrict__ dz,
-                     size_t count) {
+    relu_grad_kernel(const V* dy, const V* z, V* dz, size_t count) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
     constexpr int VEC = 16 / sizeof(V), U = 4;
@@ -600,9 +597,8 @@ __global__ void __launch_bounds__(256)
 
 // dz[t][o] = mask bit (t, o) ? dy[t][o] : 0, masks as written by the forward
 // (any d: rows of ceil(d / 32) mask words).
-__global__ void relu_grad_mask_f32_kernel(const float* __restrict__ dy,
-                                          const uint32_t* __restrict__ mask,
-                                          float* __restrict__ dz, long long rows, int d) {
+__global__ void relu_grad_mask_f32_kernel(const float* dy, const uint32_t* mask, float* dz,
+                                          long long rows, int d) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
     const int wpr = (d + 31) >> 5;
@@ -720,9 +716,9 @@ __global__ void __launch_bounds__(1024) colsum_final_kernel(const float* __restr
 // splits y, y + 8, ... in order, then the 8 lane sums meet in shared memory
 // in lane order (deterministic).  grid.y = the part, grid.z = the layer.
 __global__ void __launch_bounds__(512) splitk_reduce_kernel(
-    const float* __restrict__ partial, int splits_max, int splits_self, int splits_nbr, int d,
-    size_t part_stride, float* __restrict__ dWs, float* __restrict__ dWn, size_t out_stride,
-    const float* __restrict__ bpart, float* __restrict__ dbias) {
+    const float* partial, int splits_max, int splits_self, int splits_nbr, int d,
+    size_t part_stride, float* dWs, float* dWn, size_t out_stride, const float* bpart,
+    float* dbias) {
     pdl_wait();   // until the kernel before it in the stream has finished
     pdl_trigger();
     __shared__ float4 red[8][64];

@@ -1237,7 +1237,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
 #pragma unroll
                 for (int h = 0; h < SUB; ++h)
                     mp[h] = (has_mprev && tok_row >= 0)
-                                ? __ldg(ly.mprev + (size_t)tok_row * wpr + (col0 >> 5) + h)
+                                ? ly.mprev[(size_t)tok_row * wpr + (col0 >> 5) + h]
                                 : 0u;
                 // this warp's bias slice in registers, column h * 32 + lane in
                 // bias_reg[h], handed to the lanes by shuffles (no shared memory:
@@ -1245,7 +1245,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                 float bias_reg[SUB];
 #pragma unroll
                 for (int h = 0; h < SUB; ++h)
-                    bias_reg[h] = fwd && ly.bias && cols_in ? __ldg(ly.bias + col0 + h * 32 + lane) : 0.f;
+                    bias_reg[h] = fwd && ly.bias && cols_in ? ly.bias[col0 + h * 32 + lane] : 0.f;
                 if (!wait_acc()) {
                     return false;
                 }
@@ -1441,7 +1441,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                                 const uint4* src = reinterpret_cast<const uint4*>(
                                     L.top_dy + (size_t)tok_row * p.d + col0 + h * 32);
 #pragma unroll
-                                for (int m = 0; m < 4; ++m) q4[m] = __ldg(src + m);
+                                for (int m = 0; m < 4; ++m) q4[m] = src[m];
                             }
                             const PairMasks keep((p.flags & 4u) ? mbits[h] : ~0u);
 #pragma unroll
