@@ -468,6 +468,32 @@ def test_shift_schedule_fp32(H, flags):
         assert rel(host(got), ref) <= TOL_F32, what
 
 
+@pytest.mark.parametrize("B, d", [
+    (2, 1),        # fewer rows than one step
+    (1024, 576),   # 16,384 rows in one split
+    (1025, 33),    # many splits, a ragged last one
+])
+def test_fp32_bias_gradient_keeps_its_digits_over_many_rows(H, B, d):
+    """dbias against the fp64 column sum of the same dz.  The rounding errors of a thread's
+    long sum are kept, so what is left are the few additions around it: about sqrt(5) u
+    (u = 2^-24) of sqrt(rows), the size of a sum of that many unit normals (a lone column's
+    own sum may cancel), 4 u allowed; one chain over 2,048 rows is 12 u off, a tree of
+    64-row sums 3 u.  Infinities stay infinities."""
+    n = 16
+    g = torch.Generator(device="cuda").manual_seed(d)
+    x, dz = (torch.randn(B, n, d, generator=g, device="cuda") for _ in range(2))
+    _, _, db = H.hcw_layer_bwd_weight(x, dz, 1, -1, CAUSAL)
+    ref = dz.double().sum((0, 1))
+    assert float((db.double() - ref).norm()) <= 4 * 2.0 ** -24 * (B * n * d) ** 0.5
+    dz[B // 2, 3, 0] = float("inf")
+    _, _, db = H.hcw_layer_bwd_weight(x, dz, 1, -1, CAUSAL)
+    assert float(db[0]) == float("inf") and bool(torch.isfinite(db[1:]).all())
+    dz[0, 0, 0] = -float("inf")
+    _, _, db = H.hcw_layer_bwd_weight(x, dz, 1, -1, CAUSAL)
+    assert bool(torch.isnan(db[0]))
+    assert H.hcw_sync_status() == H.HCW_OK
+
+
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_schedule_array_of_the_rotation_equals_the_rotated_stack(H, dtype):
     """dims = (layer0 + l) mod log2 n reproduces hcw_stack_fwd / hcw_stack_bwd
