@@ -534,9 +534,10 @@ __global__ void __launch_bounds__(kRowWarps * 32)
 // Sums of a list of LayerNorm backward passes' partial rows: job blockIdx.y adds up
 // the nblk rows of its part [nblk][ncol d] per column: columns [0, d) -> dgam, [d, 2d)
 // -> dbet, [2d, 3d) -> dcol.  A CTA of eight warps per 128 columns, four a lane: warp w
-// adds rows w, w + 8, ... (eight loads in flight), then the warps' sums meet in shared
-// memory in warp order.  33 passes of d = 512: 29 us with a column a lane and 32 warps
-// a CTA, 21 so.
+// takes rows w, w + 8, ..., eight at a time, whose sum in pairs joins its chain (at most
+// 16 such sums, where one row after the other made chains of 128), then the warps' sums
+// meet in shared memory in pairs.  33 passes of d = 512: 29 us with a column a lane and
+// 32 warps a CTA, 21 so.
 constexpr int kMaxLnJobs = 64;
 struct LnJob {
     const float* part;
@@ -549,6 +550,9 @@ struct LnJobs {
     LnJob job[kMaxLnJobs];
     int d;
 };
+__device__ __forceinline__ float4 sum_pairs(const float4 (&v)[8]) {
+    return add4(add4(add4(v[0], v[1]), add4(v[2], v[3])), add4(add4(v[4], v[5]), add4(v[6], v[7])));
+}
 __global__ void __launch_bounds__(kRowWarps * 32)
     ln_part_reduce_batched_kernel(const __grid_constant__ LnJobs J) {
     pdl_wait();   // until the kernel before it in the stream has finished
@@ -562,16 +566,25 @@ __global__ void __launch_bounds__(kRowWarps * 32)
     if (blockIdx.x * 128 >= width) return;   // block-uniform: this job is narrower
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (c < width) {
-#pragma unroll 8
-        for (int b = warp; b < jb.nblk; b += kRowWarps)
-            s = add4(s, ld4(jb.part, (size_t)b * width + c));
+        for (int b0 = warp; b0 < jb.nblk; b0 += 8 * kRowWarps) {
+            float4 v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const int b = b0 + k * kRowWarps;
+                v[k] = b < jb.nblk ? ld4(jb.part, (size_t)b * width + c)
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            s = add4(s, sum_pairs(v));
+        }
     }
     acc[warp][lane] = s;
     __syncthreads();
     if (warp == 0 && c < width) {
-        float4 t = acc[0][lane];
+        float4 v[8];
+        static_assert(kRowWarps == 8, "the warps' sums meet in pairs");
 #pragma unroll
-        for (int w = 1; w < kRowWarps; ++w) t = add4(t, acc[w][lane]);
+        for (int w = 0; w < kRowWarps; ++w) v[w] = acc[w][lane];
+        const float4 t = sum_pairs(v);
         const int seg = c / d, cc = c - seg * d;
         st4(seg == 0 ? jb.dgam : (seg == 1 ? jb.dbet : jb.dcol), (size_t)cc, t);
     }
