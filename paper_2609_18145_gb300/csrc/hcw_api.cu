@@ -1855,12 +1855,20 @@ size_t step_counter_bytes(long long tokens, int L) {
 
 // Whether a training step runs its forward and input gradient as one launch:
 // bf16, any schedule whose shift layers the stacked launches take
-// (shift_stackable), the streaming kernels on SM pairs (d a multiple of 128),
-// and up to kMaxStackLayers layers.
+// (shift_stackable), the streaming kernels on SM pairs (d above 64), and up to
+// kMaxStackLayers layers.
+// Not where d is an odd multiple of 64, the stacked launches take 64-column tiles (few
+// tokens, stack_bn) and the layers are many: their steps are then shorter than those of
+// the pairs' 128 columns, by less the wider the layer, against one launch more.  us for
+// forward and input gradient, one launch | two: d = 192, 512 tokens, 4 layers 52 | 53, 8
+// layers 96 | 90, 16 layers 184 | 168; d = 320, 5 layers 76 | 76, 16 layers 222 | 206; d =
+// 576, 6 layers 116 | 119, 8 layers 151 | 150, 12 layers 223 | 214; d = 704, 8 layers 169 |
+// 170, 12 layers 250 | 242.
 bool step_fused(const Shape& sh, int dtype, const Sched& sc, int L) {
     // 256- or 128-column tiles on pairs (d = 128 takes the latter), at least
     // two row blocks
     const bool pairs = row_bn(sh.d) >= 128 && sh.tokens / 2 > 128;
+    if (sh.d % 128 != 0 && L > 4 + sh.d / 160 && stack_bn(sh) == 64) return false;
     return dtype == HCW_BF16 && (!sc.has_shift(L) || shift_stackable(sh)) && !use_resident(sh) &&
            pairs && L <= kMaxStackLayers && sh.tokens > 0;
 }
@@ -1887,19 +1895,24 @@ int step_fused_launch(const Shape& sh, const void* x, const uint8_t* Ws, const u
         row_unit_params(q, sh, BN, flags, false);
         pair_units(q);
         if (BN == 256 && 2 * q.n_units <= sms_all / 2) BN = 128;
-        // with a ragged last tile also where the narrower tiles' waves take less time (a
-        // wave of 128 columns takes 0.73 of one of 256 by its ingest; 0.82 leaves out
-        // the near ties, which the wider tile won: 105 windows of 256, d = 320, 7 layers:
-        // 413 us at 256 columns, 478 at 128; 89 of 128, d = 384, 2 layers: 85 and 83)
+        // With a ragged last tile also where the narrower tiles take less time.  A layer's
+        // step takes 0.87 of the wider tiles' (shorter units), up to 1.2 waves of pairs
+        // (1.45 causal: half of its units have half the depth) while units of neighbouring
+        // layers fill the gaps, and grows with the waves above.  us for forward and input
+        // gradient of 8 layers at 128 | 256 columns (waves), not causal: d = 192, 12,288
+        // tokens 115 (1.3) | 125 (0.6), 16,384 134 (1.7) | 129 (0.8); d = 384, 8,192 tokens
+        // 149 (1.3) | 168 (0.8), 12,288 202 (1.9) | 175 (1.3); d = 832, 3,072 tokens 211 (1.1)
+        // | 233 (0.6), 4,096 253 (1.5) | 236 (0.8); causal 215 | 230.
         if (BN == 256 && sh.d % 256 != 0) {
+            const double full = (flags & HCW_CAUSAL) ? 1.45 : 1.2;
             auto time = [&](int bn, double step) {
                 TcParams t;
                 row_unit_params(t, sh, bn, flags, false);
                 pair_units(t);
-                const double w = 2.0 * t.n_units / sms_all;
-                return (w < 4.0 ? ceil(w) : w) * step;
+                const double w = 2.0 * t.n_units / sms_all / full;
+                return step * (w > 1 ? w : 1);
             };
-            if (time(128, 0.82) < time(256, 1.0)) BN = 128;
+            if (time(128, 0.87) < time(256, 1.0)) BN = 128;
         }
     }
     const int d = sh.d, pw = epi_patch_cols(BN);

@@ -48,6 +48,10 @@ CASES = [
     (32, 64, 128, 6, 1, CAUSAL | RESIDUAL | RELU),
     (2, 64, 128, 3, 0, RESIDUAL | RELU),               # 128 tokens: the two calls
     (4, 64, 192, 3, 0, CAUSAL | RESIDUAL | RELU),      # 64-column tiles: the two calls
+    (8, 64, 192, 5, 0, CAUSAL | RESIDUAL | RELU),      # odd multiple of 64, few layers: one launch
+    (8, 64, 192, 6, 0, CAUSAL | RESIDUAL | RELU),      # more: the two calls
+    (40, 256, 384, 2, 0, RESIDUAL | RELU),             # ragged: 256 columns by the waves
+    (24, 256, 384, 2, 0, RESIDUAL | RELU),             # ... and 128
     # enough layers for the batched weight gradient on SM pairs, which then
     # starts behind the fused launch and waits on its completion counters
     (4, 256, 512, 12, 5, CAUSAL | RESIDUAL | RELU),
