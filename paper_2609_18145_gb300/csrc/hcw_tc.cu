@@ -94,11 +94,11 @@ struct __align__(8) Barriers {
     int dep_unit;   // the producer has seen the inputs of this CTA's units up to this ordinal
     int unit_q[kUnitQ];   // dynamic scheduling: unit claimed for ordinal o, in slot o % kUnitQ
     int q_pub;            // highest ordinal published in unit_q
-    int q_read;           // slot reads so far (the MMA thread and every epilogue warp)
     // stacked row launches: epilogue warps whose stores of the unit in slot o %
     // kUnitQ have completed, per published output (0: the counters' output,
     // 1: the input gradient's g); the last one publishes the CTA's rows
     int pub_done[2][kUnitQ];
+    int q_read[kUnitQ];   // reads of each slot so far (the MMA thread and every epilogue warp)
 };
 
 // epilogue patch buffers (MODE_DWF stores from registers)
@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
         bars->abort = 0;
         bars->dep_unit = -1;
         bars->q_pub = -1;
-        bars->q_read = 0;
+        for (int i = 0; i < kUnitQ; ++i) bars->q_read[i] = 0;
         for (int i = 0; i < 2 * kUnitQ; ++i) (&bars->pub_done[0][0])[i] = 0;
         fence_mbar_init();
     }
@@ -562,9 +562,10 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
             return u < n_units ? u : -1;
         }
         if (!wait_shared_geq<PAIR>(&bars->q_pub, ord, abort, tmo)) return -2;
-        const int u = *reinterpret_cast<volatile int*>(&bars->unit_q[ord % kUnitQ]);
+        const uint32_t slot = (uint32_t)ord % kUnitQ;
+        const int u = *reinterpret_cast<volatile int*>(&bars->unit_q[slot]);
         __threadfence_block();
-        atomicAdd(&bars->q_read, 1);
+        atomicAdd(&bars->q_read[slot], 1);
         return u;
     };
 
@@ -594,17 +595,21 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                     else
                         u = atomicAdd(L.sched, 1);
                     if (u >= n_units) u = -1;
-                    // the slot's previous unit has been read by every consumer
+                    // The slot's previous unit has been read by every consumer.  (Counted
+                    // slot by slot: in a count over all slots the reads of consumers that
+                    // are ahead stood for those of one that was behind, whose unit was then
+                    // overwritten: with one K step a unit, causal d = 64, the ring lets the
+                    // producer get that far ahead.)
+                    const uint32_t slot = (uint32_t)ordinal % kUnitQ;
+                    const int need = (int)((uint32_t)ordinal / kUnitQ) * (EW + 1);
                     if (ordinal >= kUnitQ &&
-                        !wait_shared_geq(&bars->q_read, (ordinal - kUnitQ + 1) * (EW + 1), abort,
-                                         tmo)) {
+                        !wait_shared_geq(&bars->q_read[slot], need, abort, tmo)) {
                         ok = false;
                         break;
                     }
                     if (PAIR) {
                         // ... and in the other CTA of the pair
-                        const uint32_t peer_read = mapa_shared(&bars->q_read, 1);
-                        const int need = (ordinal - kUnitQ + 1) * (EW + 1);
+                        const uint32_t peer_read = mapa_shared(&bars->q_read[slot], 1);
                         bool okp = true;
                         if (ordinal >= kUnitQ && ld_acquire_cluster_remote(peer_read) < need) {
                             const uint64_t t0 = globaltimer_ns();
@@ -621,10 +626,10 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                             ok = false;
                             break;
                         }
-                        st_remote(mapa_shared(&bars->unit_q[ordinal % kUnitQ], 1), u);
+                        st_remote(mapa_shared(&bars->unit_q[slot], 1), u);
                         st_release_cluster_remote(mapa_shared(&bars->q_pub, 1), ordinal);
                     }
-                    bars->unit_q[ordinal % kUnitQ] = u;
+                    bars->unit_q[slot] = u;
                     st_release_cta_shared(&bars->q_pub, ordinal);
                 } else {
                     u = (int)blockIdx.x + ordinal * (int)gridDim.x;
@@ -1364,7 +1369,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                     if (lane == 0) {
                         if (inside) bulk_wait<0>();
                         fence_proxy_async_global();
-                        int* done = &bars->pub_done[kind][ordinal % kUnitQ];
+                        int* done = &bars->pub_done[kind][(uint32_t)ordinal % kUnitQ];
                         if (atom_add_acq_rel_cta_shared(done, 1) == EW - 1) {
                             *done = 0;   // next used by ordinal + kUnitQ, after this unit
                             const int cols = min(BN, p.d - r.j * BN);

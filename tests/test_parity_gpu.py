@@ -582,6 +582,33 @@ def test_ragged_column_tiles_keep_the_bits(H, B, n, d):
         assert torch.equal(step[i], big[j]), i
 
 
+@pytest.mark.parametrize("n, L", [(16, 12), (64, 6)])
+def test_streaming_units_of_one_step_are_each_read(H, n, L):
+    """Causal layers of d = 64 have units of a single K step: a CTA's producer hands out units
+    many slots ahead of its slowest reader.  Every unit is still run by every warp: many
+    rounds of many units a CTA give the bits of the kernel that keeps the tokens on chip."""
+    B, d, flags = 98304 // n, 64, CAUSAL | RESIDUAL | RELU
+    g = torch.Generator(device="cuda").manual_seed(n)
+    x, dy = (torch.randn(B, n, d, generator=g, device="cuda").bfloat16() for _ in range(2))
+    Ws, Wn = ((torch.randn(L, d, d, generator=g, device="cuda") / (2 * d) ** 0.5).bfloat16()
+              for _ in range(2))
+    bias = torch.randn(L, d, generator=g, device="cuda")
+
+    def run():
+        y, acts, masks = H.hcw_stack_fwd(x, Ws, Wn, bias, 0, -1, flags)
+        return (y, acts, masks) + H.hcw_stack_bwd_data(masks, dy, Ws, Wn, 0, -1, flags)
+
+    ref = run()
+    H.hcw_set_stack_kernels(H.HCW_STACK_STREAMING)
+    try:
+        for _ in range(30):
+            for i, (a, b) in enumerate(zip(run(), ref)):
+                assert torch.equal(a, b), i
+    finally:
+        H.hcw_set_stack_kernels(H.HCW_STACK_AUTO)
+    assert H.hcw_sync_status() == H.HCW_OK
+
+
 @pytest.mark.parametrize("B, n, d, L, flags, dims", [
     (1, 2, 64, 1, CAUSAL | RESIDUAL | RELU, None),            # the smallest
     (3, 64, 128, 6, RESIDUAL | RELU, None),                   # a ragged tile of 128 tokens
