@@ -481,23 +481,50 @@ int launched(cudaError_t e, int kernels) {
 }
 
 // ------------------------------------------------------------ layer internals
-// Column tile of a stacked forward / input-gradient launch.  With few tokens the
-// launch is the layer chain, not throughput: a unit's operands come at what one SM
+// Waves of a layer's row units over the SMs (pairs of SMs at 256 columns count the same),
+// by column tile.
+double unit_waves(const Shape& sh, int BN) {
+    const long long row_units = 2 * ((sh.tokens / 2 + 127) / 128);
+    return (double)(row_units * ((sh.d + BN - 1) / BN)) / sm_count();
+}
+
+// Column tile of a forward (or, dx, input-gradient) launch of L layers.  With few tokens
+// the launch is the layer chain, not throughput: a unit's operands come at what one SM
 // takes in, so narrower tiles, spread over more SMs, shorten every step (each output
 // element sums the same products in the same order).  64 columns while every unit of
-// a layer has an SM of its own, 128 up to 1.75 waves, else 256 on pairs.  Microseconds a
+// a layer has an SM of its own, and in many layers somewhat beyond, since the units of
+// neighbouring layers fill the gaps of a wave (further causal, where half of them have
+// half the depth); a short stack's input gradient gains nothing there from d = 640 on
+// (three layers of d = 896 over 512 tokens 54 us, 50 at 128 columns).  Then 128 columns up
+// to a line that falls with the depth of the products, else 256 on pairs; where the last
+// of the wide tiles is half empty the line lies as much higher.  Microseconds a
 // layer of an 8-layer causal stack, forward / input gradient, at 64 | 128 | 256 columns:
 //   d = 256:  2048 tokens  6.3/6.8 | 6.9/7.3 | 8.6/8.9;   16384  12.2/13.9 | 8.6/9.7 | 9.6/9.9
 //   d = 512:   256 tokens  8.2/9.3 | 8.8/9.6 | 11.1/11.6;  2048  8.5/9.6 | 9.1/10.0 | 11.0/11.5
 //             4096 tokens  9.8/10.9 | 9.3/10.8 | 11.2/11.9;  8192  17.0/18.5 | 11.1/12.2 | 11.9/13.1
 //            16384 tokens  32.5/34.2 | 19.6/21.1 | 14.3/15.3
 //   d = 1024: 1024 tokens  12.8/15.1 | 13.6/15.0 | 15.5/16.5;  4096  27.3/29.8 | 16.8/18.3 | 17.0/18.3
-int stack_bn(const Shape& sh) {
-    const long long row_units = 2 * ((sh.tokens / 2 + 127) / 128);
-    const int sms = sm_count();
-    if (row_units * (sh.d / 64) <= sms) return 64;
-    if (sh.d > 64 && 4 * row_units * ((sh.d + 127) / 128) <= 7ll * sms) return 128;
-    return row_bn(sh.d);
+// and 128 | 256 columns relative to the better one, by waves of the 128 ones, three and
+// twelve layers, not causal: d = 256, 1.7 waves 1.02 | 1, 1 | 1.07; d = 512, 1.3 waves
+// 1 | 1, 1 | 1.11, 1.7 waves 1.13 | 1, 1.02 | 1; d = 1024, 1.3 waves 1.05 | 1, 1 | 1.03, 1.7
+// waves 1.28 | 1, 1.18 | 1; causal: d = 512, 1.7 waves 1.01 | 1, 1 | 1.09; d = 1024 1.08 | 1,
+// 1 | 1.01; d = 384, 1.9 (three tiles against two) 1 | 1.08, 1 | 1.06.
+int stack_bn(const Shape& sh, unsigned flags, int L, bool dx) {
+    const int d = sh.d;
+    const bool causal = (flags & HCW_CAUSAL) != 0, many = L >= 8;
+    const double beyond = causal ? 1.5 : 1.27;
+    if (unit_waves(sh, 64) <= (many ? beyond : 1.0) && (!dx || many || d < 640)) return 64;
+    if (d <= 64) return 64;
+    double line;
+    if (causal)
+        line = d <= 640 ? 1.75 : 1.5;
+    else if (d <= 256)
+        line = 1.75;
+    else
+        line = !many && d <= 384 ? 1.45 : many || d <= 640 ? 1.27 : 1.0;
+    line *= 2.0 * ((d + 255) / 256) / ((d + 127) / 128);
+    if (unit_waves(sh, 128) <= (line < 1.95 ? line : 1.95)) return 128;
+    return row_bn(d);
 }
 
 // Row-unit geometry of a forward (or input-gradient) pass: which bit value's
@@ -547,7 +574,7 @@ bool fwd_maps(CUtensorMap* m, const Shape& sh, int s, const void* x, const void*
 int fwd_bf16(const Shape& sh, const void* x, const void* Ws, const void* Wn, const float* bias,
              unsigned flags, void* y, void* z, uint32_t* mask, cudaStream_t st,
              const void* xpair = nullptr) {
-    const int BN = stack_bn(sh);
+    const int BN = stack_bn(sh, flags, 1, false);
     TcLaunch<1> L;
     memset(&L, 0, sizeof(L));
     if (!fwd_maps(L.maps[0], sh, sh.s, x, Ws, Wn, y, false, BN)) return HCW_ERR_CUDA;
@@ -663,7 +690,7 @@ template <class In, class Out, class Mask>
 int stack_fwd_group(const Shape& sh, int l0, int n, const Sched& sc,
                     const uint8_t* Ws, const uint8_t* Wn, const float* bias, unsigned flags,
                     In in_ptr, Out out_ptr, Mask mask_ptr, int* counters, cudaStream_t st) {
-    const int d = sh.d, BN = stack_bn(sh);
+    const int d = sh.d, BN = stack_bn(sh, flags, n, false);
     const size_t wb = (size_t)d * d * 2;
     const bool pair = use_pairs(sh, BN);
     static thread_local TcLaunch<kMaxStackLayers> L;
@@ -729,7 +756,7 @@ int stack_fwd_resident(const Shape& sh, int l0, int n, const Sched& sc,
 int dx_bf16(const Shape& sh, const void* dz, const void* dy, const void* Ws, const void* Wn,
             unsigned flags, void* dx, cudaStream_t st, const uint32_t* mprev = nullptr,
             void* dz_out = nullptr, const void* dzpair = nullptr) {
-    const int d = sh.d, BN = stack_bn(sh), k = 1 << sh.s;
+    const int d = sh.d, BN = stack_bn(sh, flags, 1, true), k = 1 << sh.s;
     const int pw = epi_patch_cols(BN);
     TcLaunch<1> L;
     memset(&L, 0, sizeof(L));
@@ -1194,7 +1221,7 @@ int stack_data_bf16(const Shape& sh, const StackData& a, cudaStream_t st) {
     if (a.sc.has_shift(a.L) && (!shift_stackable(sh) || use_resident(sh)))
         return stack_data_layers_bf16(sh, a, st);
     if (use_resident(sh)) return stack_data_resident(sh, a, st);
-    const int d = sh.d, BN = stack_bn(sh), L = a.L;
+    const int d = sh.d, L = a.L, BN = stack_bn(sh, a.flags, L, true);
     const bool relu = (a.flags & HCW_ACT_RELU) != 0;
     const bool resid = (a.flags & HCW_RESIDUAL) != 0;
     const bool keep_g = relu && resid;
@@ -1857,8 +1884,8 @@ size_t step_counter_bytes(long long tokens, int L) {
 // bf16, any schedule whose shift layers the stacked launches take
 // (shift_stackable), the streaming kernels on SM pairs (d above 64), and up to
 // kMaxStackLayers layers.
-// Not where d is an odd multiple of 64, the stacked launches take 64-column tiles (few
-// tokens, stack_bn) and the layers are many: their steps are then shorter than those of
+// Not where d is an odd multiple of 64, the stacked launches have an SM for every unit of
+// 64 columns (few tokens) and the layers are many: their steps are then shorter than those of
 // the pairs' 128 columns, by less the wider the layer, against one launch more.  us for
 // forward and input gradient, one launch | two: d = 192, 512 tokens, 4 layers 52 | 53, 8
 // layers 96 | 90, 16 layers 184 | 168; d = 320, 5 layers 76 | 76, 16 layers 222 | 206; d =
@@ -1868,7 +1895,7 @@ bool step_fused(const Shape& sh, int dtype, const Sched& sc, int L) {
     // 256- or 128-column tiles on pairs (d = 128 takes the latter), at least
     // two row blocks
     const bool pairs = row_bn(sh.d) >= 128 && sh.tokens / 2 > 128;
-    if (sh.d % 128 != 0 && L > 4 + sh.d / 160 && stack_bn(sh) == 64) return false;
+    if (sh.d % 128 != 0 && L > 4 + sh.d / 160 && unit_waves(sh, 64) <= 1.0) return false;
     return dtype == HCW_BF16 && (!sc.has_shift(L) || shift_stackable(sh)) && !use_resident(sh) &&
            pairs && L <= kMaxStackLayers && sh.tokens > 0;
 }
