@@ -517,34 +517,49 @@ def test_schedule_array_of_the_rotation_equals_the_rotated_stack(H, dtype):
         assert torch.equal(u, v)
 
 
-@pytest.mark.parametrize("B, n, d", [
-    (1, 256, 512),    # 64-column tiles: the fewest tokens
-    (19, 256, 256),   # 64-column tiles, 152 units: the most they take on 152 SMs
-    (5, 128, 256),    # 64-column tiles, a ragged last row block
-    (33, 256, 256),   # 128-column tiles, a ragged last row block
-    (16, 256, 1024),  # 128-column tiles, 256 units: the most they take
+@pytest.mark.parametrize("B, n, d, L", [
+    (19, 256, 256, 3),   # 64-column tiles, 152 units: the most that three layers take on 152 SMs
+    (5, 128, 256, 3),    # 64-column tiles, a ragged last row block
+    (28, 256, 256, 8),   # 64-column tiles beyond one wave: many layers
+    (33, 256, 256, 3),   # 128-column tiles, a ragged last row block
+    (16, 256, 512, 3),   # 128-column tiles
+    (8, 256, 1024, 3),   # 128-column tiles (the input gradient's from one sample on)
+    (96, 256, 256, 3),   # 256-column tiles on pairs
+    (64, 256, 512, 3),   # 256-column tiles on pairs
+    (16, 256, 1024, 3),  # 256-column tiles on pairs
 ])
-def test_column_tile_choice_of_the_stack_keeps_the_bits(H, B, n, d):
-    """The stacked launches choose their column tile by the tokens; whatever the tile,
-    forward and input gradient are bit for bit the chain of single-layer calls (whose
-    tile depends on d alone)."""
-    L, flags = 3, CAUSAL | RESIDUAL
+def test_column_tile_choice_of_the_stack_keeps_the_bits(H, B, n, d, L):
+    """The stacked launches choose their column tile by the tokens.  Samples are independent,
+    so the first and the last one's rows of a batch are bit for bit those of batches of one,
+    which take 64-column tiles (the input gradient of a wide d 128-column ones): forward and
+    input gradient of the stack, and of its layers one by one, whose launches choose for
+    themselves."""
+    flags = CAUSAL | RESIDUAL
     g = torch.Generator(device="cuda").manual_seed(B)
     x, dy = (torch.randn(B, n, d, generator=g, device="cuda").bfloat16() for _ in range(2))
     Ws, Wn = ((torch.randn(L, d, d, generator=g, device="cuda") / (2 * d) ** 0.5).bfloat16()
               for _ in range(2))
     bias = torch.randn(L, d, generator=g, device="cuda")
-    y, acts, _ = H.hcw_stack_fwd(x, Ws, Wn, bias, 0, -1, flags)
-    h = x
-    for l in range(L):
-        h = H.hcw_layer_fwd(h, Ws[l], Wn[l], bias[l], l, -1, flags)
-        assert torch.equal(h, acts[l] if l < L - 1 else y)
-    dx, dz = H.hcw_stack_bwd_data(None, dy, Ws, Wn, 0, -1, flags)
-    q = dy
-    for l in reversed(range(L)):
-        assert torch.equal(dz[l], q)
-        q = H.hcw_layer_bwd_data(q, q, Ws[l], Wn[l], l, -1, flags)
-    assert torch.equal(dx, q)
+
+    def run(x, dy):
+        y, acts, _ = H.hcw_stack_fwd(x, Ws, Wn, bias, 0, -1, flags)
+        dx, dz = H.hcw_stack_bwd_data(None, dy, Ws, Wn, 0, -1, flags)
+        h = x
+        for l in range(L):
+            h = H.hcw_layer_fwd(h, Ws[l], Wn[l], bias[l], l, -1, flags)
+            assert torch.equal(h, acts[l] if l < L - 1 else y)
+        q = dy
+        for l in reversed(range(L)):
+            assert torch.equal(dz[l], q)
+            q = H.hcw_layer_bwd_data(q, q, Ws[l], Wn[l], l, -1, flags)
+        assert torch.equal(dx, q)
+        return y, dx, acts, dz
+
+    big = run(x, dy)
+    for b in (0, B - 1):
+        one = run(x[b:b + 1].contiguous(), dy[b:b + 1].contiguous())
+        for i, (a, r) in enumerate(zip(big, one)):
+            assert torch.equal(a[b:b + 1] if i < 2 else a[:, b:b + 1], r), i
     assert H.hcw_sync_status() == H.HCW_OK
 
 
