@@ -360,9 +360,10 @@ int hcw_layer_bwd_weight_noalloc(const void* x, const void* dz, int layer, int d
  * (hcw_stack_fwd, hcw_stack_bwd_data, hcw_stack_bwd).  Process-wide.
  *   HCW_STACK_AUTO       the faster family as measured on GB300 for the
  *                        shape: streaming, and for narrow layers over short
- *                        windows (d 64 or 128, n <= 128, L <= 64) a kernel that
- *                        keeps 128 tokens on chip through all layers, with the
- *                        streaming kernels' results bit for bit.  The default.
+ *                        windows (d 64 or 128, n <= 128, L <= 64; at d = 128 up
+ *                        to as many tokens as it is the faster one for) a kernel
+ *                        that keeps 128 tokens on chip through all layers, with
+ *                        the streaming kernels' results bit for bit.  The default.
  *   HCW_STACK_RESIDENT   resident wherever the shape fits.
  *   HCW_STACK_STREAMING  streaming only.
  * Resident: a cluster of two CTAs keeps 256 consecutive tokens (whole

@@ -625,11 +625,28 @@ bool use_resident(const Shape& sh) {
     return mode == HCW_STACK_RESIDENT;
 }
 
-// Whether a bf16 stack runs on the kernel that keeps 128 tokens on chip through all
-// layers (hcw_small.cu): narrow layers, short windows, no kernel family asked for.
-bool use_small(const Shape& sh, int L) {
-    return g_stack_kernels.load(std::memory_order_relaxed) == HCW_STACK_AUTO &&
-           small_supported(sh.d, sh.n, sh.tokens, L);
+// Whether a bf16 stack's forward (fwd) and / or input gradient (bwd) runs on the kernel
+// that keeps 128 tokens on chip through all layers (hcw_small.cu): narrow layers, short
+// windows, no kernel family asked for.  At d = 128 a CTA fills an SM and takes its blocks of
+// tokens one after the other, paying the layer chain each time, where the stacked launches
+// overlap layers: beyond one wave of blocks the waves have to be well filled and the layers
+// many.  us on chip | streaming, causal, n = 64: forward, 20,480 tokens (1.05 waves) 3
+// layers 28 | 25, 12 layers 73 | 72; 49,152 (2.5) 3 layers 39 | 33, 12 layers 111 | 105; 98,304
+// (5.05) 1 layer 39 | 22, 12 layers 213 | 187.  Forward and input gradient: 40,960 (2.1) 1
+// layer 35 | 29, 3 layers 68 | 59, 6 layers 112 | 109; 131,072 (6.7) 2 layers 120 | 115, 3 layers
+// 156 | 166.  Input gradient: 49,152 1 layer 22 | 21, 98,304 39 | 35, more layers as fast or faster.
+bool use_small(const Shape& sh, const Sched& sc, int L, bool fwd, bool bwd) {
+    if (g_stack_kernels.load(std::memory_order_relaxed) != HCW_STACK_AUTO ||
+        !small_supported(sh.d, sh.n, sh.tokens, L))
+        return false;
+    if (sh.d == 64) return true;   // (two CTAs an SM)
+    if (sc.has_shift(L) && !shift_stackable(sh)) return true;   // else layer by layer
+    const double waves = (double)((sh.tokens + 127) / 128) / sm_count();
+    const bool filled = ceil(waves) < 1.1 * waves;
+    if (waves <= 1) return true;
+    if (fwd && bwd) return waves <= 2 || L >= 5 || (L >= 3 && filled);
+    if (bwd) return waves <= 2 || L > 1;
+    return waves <= 2 ? L == 1 || (L >= 6 && waves > 1.2) : L >= 10 && filled;
 }
 
 // The forward (y given) and / or the input gradient (dx given) of a stack there.
@@ -1215,7 +1232,7 @@ int stack_data_layers_bf16(const Shape& sh, const StackData& a, cudaStream_t st)
 }
 
 int stack_data_bf16(const Shape& sh, const StackData& a, cudaStream_t st) {
-    if (use_small(sh, a.L))
+    if (use_small(sh, a.sc, a.L, false, true))
         return small_launch(sh, a.sc, a.L, a.flags, nullptr, a.Ws, a.Wn, nullptr, nullptr, nullptr,
                             const_cast<void*>(a.masks), a.dy, a.dx, a.dz, st);
     if (a.sc.has_shift(a.L) && (!shift_stackable(sh) || use_resident(sh)))
@@ -1760,7 +1777,7 @@ int stack_fwd_impl(const Shape& sh, const void* x, const void* W_self, const voi
         return want_mask ? reinterpret_cast<uint32_t*>(static_cast<uint8_t*>(masks) + (size_t)l * mb)
                          : nullptr;
     };
-    if (dtype == HCW_BF16 && use_small(sh, L))
+    if (dtype == HCW_BF16 && use_small(sh, sc, L, true, false))
         return small_launch(sh, sc, L, flags, x, W_self, W_nbr, bias, y, acts,
                             want_mask ? masks : nullptr, nullptr, nullptr, nullptr, st);
     if (dtype == HCW_BF16 && sc.has_shift(L) && (!shift_stackable(sh) || use_resident(sh))) {
@@ -2118,7 +2135,7 @@ int train_step_impl(const Shape& sh, const void* x, const void* W_self, const vo
                      static_cast<const uint8_t*>(W_nbr), sc, L, flags, dx, ws, ws + zb};
         return dtype == HCW_BF16 ? stack_data_bf16(sh, da, st) : stack_data_f32(sh, da, st);
     }
-    const bool small = use_small(sh, L);
+    const bool small = use_small(sh, sc, L, true, true);
     if (small)
         rc = small_launch(sh, sc, L, flags, x, W_self, W_nbr, bias, y, acts,
                           (flags & HCW_ACT_RELU) ? masks : nullptr, dy, dx, ws, st);

@@ -632,7 +632,10 @@ def test_streaming_units_of_one_step_are_each_read(H, n, L):
     (4, 32, 128, 4, 0, None),                                 # plain Eq. (1)
     (9, 64, 128, 7, CAUSAL | RESIDUAL | RELU, [-1, 5, -7, 0, -63, 3, -1]),
     (7, 128, 64, 4, RESIDUAL | RELU, [-64, 6, -127, 0]),
-    (320, 64, 128, 3, CAUSAL | RESIDUAL | RELU, None),        # more tiles than SMs
+    (320, 64, 128, 3, CAUSAL | RESIDUAL | RELU, None),        # more tiles than SMs: not forward alone
+    (400, 64, 128, 6, CAUSAL | RESIDUAL | RELU, None),        # ... and with as many layers that too
+    (640, 64, 128, 2, RESIDUAL | RELU, None),                 # the input gradient alone
+    (330, 64, 128, 3, RESIDUAL | RELU, [-1, 5, -7]),          # shifts that nothing else takes at once
     (700, 64, 64, 17, RESIDUAL | RELU, None),                 # the same at d = 64
 ])
 def test_on_chip_stack_equals_the_streaming_one(H, B, n, d, L, flags, dims):
