@@ -325,37 +325,7 @@ struct WPlan {
 // Scratch of the weight gradient without a workspace (hcw_layer_bwd_weight_noalloc).
 constexpr size_t kNoAllocScratchBytes = (size_t)32 << 20;   // 32 MiB
 
-// Column tile of the weight gradients of `layers` layers in one launch; the last tile is
-// ragged where d is not a multiple of it (its operand columns past d load as zeros and
-// are not stored).  A unit's time is its operands' ingest, 128 + BN columns a token
-// block; a launch takes its waves of units, or, where the units split the token range to
-// fill one wave (split_dw_layers), their number.  Few tokens are bound by the units'
-// stores and latency and keep whole narrow tiles (16 layers of d = 576 over 512 tokens,
-// step: 341 us so, 349 ragged).  Steps before, with 64 columns, and so: 113,920 tokens, 6
-// layers of d = 448 2,398 and 1,454 us; 123,904 tokens, 7 of 704 5,225 and 3,438; 37,888
-// tokens, 3 of 320 351 and 251; 6,272 tokens, 18 of 704 836 and 713.
 int whole_bn(int d) { return d % 256 == 0 ? 256 : d % 128 == 0 ? 128 : 64; }
-
-int dw_bn(long long tokens, int d, int layers) {
-    if (d % 256 == 0 || tokens <= 2048) return whole_bn(d);
-    const int sms = sm_count(), rows = (d + 127) / 128;
-    int best = 64;
-    double best_t = 0;
-    for (int bn = 64; bn <= 256 && bn < 2 * d; bn *= 2) {
-        const int units = layers * rows * ((d + bn - 1) / bn);
-        double waves = (double)units / sms;
-        if (layers > 1 && units * 2 >= sms)
-            // self and partner part together in a unit, or apart in two
-            waves = 5 * units >= 3 * sms ? (units + sms - 1) / sms
-                                         : 0.5 * ((2 * units + sms - 1) / sms);
-        const double t = waves * (128 + bn);
-        if (bn == 64 || t <= best_t) {
-            best = bn;
-            best_t = t;
-        }
-    }
-    return best;
-}
 
 // The split of the token range of the weight gradient into units of column tile BN.
 WPlan split_dw(long long tokens, int d, unsigned flags, int layers, int BN) {
@@ -396,16 +366,54 @@ size_t dw_part_bytes(const WPlan& w, int d) {
     return w.splits_max > 1 ? align256((size_t)2 * w.splits_max * d * d * 4) : 0;
 }
 
-// The split for one layer, or for `layers` layers sharing one launch.
+// Estimated us of the launch that takes the split w (its mode as in stack_weight_bf16).  A
+// unit of one part costs its operands' ingest, 128 + BN columns a block of 64 tokens, and
+// no less than at 136 columns; slower where the operands exceed what L2 holds.  A split in
+// several parts adds its partial sums and the launch that reduces them, a unit of both
+// parts (every block read once, twice the products) the stores of its two tiles.  Fitted
+// to 2,880 launches (d = 192 .. 960, 3,072 .. 49,152 tokens, 1 .. 16 layers, three tiles):
+// 9 % rms.
+double dw_cost(const WPlan& w, long long tokens, int d, int layers) {
+    const int sms = sm_count(), tiles = layers * w.n_ot * w.n_nt, cols = 128 + w.BN;
+    const bool resident = 4.0 * layers * tokens * d < 100e6;
+    const double block = (resident ? 1.11e-3 : 1.3e-3) * (cols > 264 ? cols : 264);
+    if (layers == 1 || 2 * tiles < sms) {   // the token range split where the units leave SMs idle
+        const int units = layers * w.units;
+        const int blocks = w.kb_per_unit < w.nkb_self ? w.kb_per_unit : w.nkb_self;
+        const double sums = 9.6 + 0.045e-6 * 2 * w.splits_max * d * d * 4 * layers;
+        return 6 + (units + sms - 1) / sms * blocks * block + (w.splits_max > 1 ? sums : 0);
+    }
+    if (5 * tiles < 3 * sms)   // self and partner part apart, one SM taking two of the latter
+        return 6 + 1.12 * block * (w.nkb_self > 2 * w.nkb_nbr ? w.nkb_self : 2 * w.nkb_nbr);
+    return 6 + (tiles + sms - 1) / sms * (w.nkb_self * (0.145 + 1.075e-3 * cols) + 0.06 * w.BN);
+}
+
+// The split for one layer, or for `layers` layers sharing one launch, and its column tile:
+// the one of the least dw_cost; the last tile is ragged where d is not a multiple of it
+// (its operand columns past d load as zeros and are not stored).  Few tokens are bound by
+// the units' stores and latency and keep whole narrow tiles.  us at 64 | 128 | 256 columns,
+// not causal: d = 704, 3,072 tokens, 2 layers 26 | 20 | 34 (split, partial sums); d = 320,
+// 49,152 tokens, 8 layers 321 | 271 | 374 (96 units on 152 SMs), causal 321 | 258 | 208;
+// d = 448, 49,152 tokens, 4 layers 321 | 261 | 196; d = 896, 6,144 tokens, 2 layers 89 | 53 | 41.
 WPlan plan_dw(long long tokens, int d, unsigned flags, int layers = 1) {
-    const int BN = dw_bn(tokens, d, layers);
-    const WPlan w = split_dw(tokens, d, flags, layers, BN);
-    // Fewer, wider tiles are split more often, with more partial sums: sizes that fit
-    // the scratch of the call without a workspace with whole tiles keep fitting it.
-    if (layers == 1 && BN != whole_bn(d) &&
-        dw_part_bytes(w, d) + align256(colsum_workspace_bytes(tokens, d)) > kNoAllocScratchBytes)
-        return split_dw(tokens, d, flags, layers, whole_bn(d));
-    return w;
+    const int whole = whole_bn(d);
+    WPlan best = split_dw(tokens, d, flags, layers, whole);
+    if (d % 256 == 0 || tokens <= 2048) return best;
+    double least = 0;
+    for (int bn = 64; bn <= 256 && bn < 2 * d; bn *= 2) {
+        const WPlan w = split_dw(tokens, d, flags, layers, bn);
+        // Fewer, wider tiles are split more often, with more partial sums: sizes that fit
+        // the scratch of the call without a workspace with whole tiles keep fitting it.
+        if (layers == 1 && bn != whole &&
+            dw_part_bytes(w, d) + align256(colsum_workspace_bytes(tokens, d)) > kNoAllocScratchBytes)
+            continue;
+        const double c = dw_cost(w, tokens, d, layers);
+        if (least == 0 || c <= least) {
+            least = c;
+            best = w;
+        }
+    }
+    return best;
 }
 
 // SM pairs of the batched weight-gradient launch of a training step when it

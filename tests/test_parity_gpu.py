@@ -1224,8 +1224,11 @@ def test_fp32_stack_in_one_launch_matches_its_layers(H, case):
 
 # bf16 weight gradients whose last column tile is ragged: B, n, d, L, flags
 RAGGED_DW = [
-    (40, 64, 192, 2, CAUSAL),      # one tile of 256 columns, token splits
-    (20, 128, 320, 5, 0),          # two, the last a quarter full
+    (40, 64, 192, 2, CAUSAL),      # two tiles of 128 columns, token splits
+    (40, 64, 192, 3, 0),           # one of 256 columns, token splits
+    (20, 128, 320, 5, 0),          # tiles of 128, the last half full
+    (34, 64, 320, 12, 0),          # of 256, the last a quarter full
+    (66, 64, 576, 4, CAUSAL),
     (34, 64, 448, 16, CAUSAL),     # both parts in one unit
     (33, 64, 576, 11, 0),
     (33, 64, 320, 8, RELU),
