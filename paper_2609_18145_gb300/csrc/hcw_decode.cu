@@ -505,6 +505,14 @@ __device__ __forceinline__ void copy_to_peer(uint32_t dst, uint32_t src, uint32_
         : "memory");
 }
 
+// takes bytes off a barrier's pending transactions, as if a copy of that size had landed
+__device__ __forceinline__ void mbar_complete_tx(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+                 "r"(bytes)
+                 : "memory");
+}
+constexpr uint64_t kDrainNs = 1000000000ull;   // 1 s
+
 // 16 features of a row
 struct Feat16 {
     uint32_t r[8];
@@ -594,7 +602,11 @@ __global__ void __launch_bounds__(mma_threads(OC), 1)
     __nv_bfloat16** outp = reinterpret_cast<__nv_bfloat16**>(bars + kMmaBars);
     int* prow = reinterpret_cast<int*>(outp + kMaxDecodeLayers);
     volatile int* abort = prow + kMaxDecodeLayers;
-    float* bias_s = const_cast<float*>(reinterpret_cast<volatile float*>(abort + 4));   // [L][OC]
+    // after an abort somewhere in the cluster: that there was one, and for every CTA of the
+    // cluster how many of its slices it did not send to this one
+    volatile int* down = abort + 1;
+    volatile int* unsent = abort + 4;   // [16]
+    float* bias_s = const_cast<float*>(reinterpret_cast<volatile float*>(unsent + 16));   // [L][OC]
     const bool partner_warp = SPLIT && threadIdx.x >= kMmaWarps * 32;
     const int warp = (threadIdx.x >> 5) - (partner_warp ? kMmaWarps : 0);
     const int lane = threadIdx.x & 31;
@@ -607,8 +619,10 @@ __global__ void __launch_bounds__(mma_threads(OC), 1)
         outp[threadIdx.x] = a.out[threadIdx.x];
         prow[threadIdx.x] = a.prow[threadIdx.x];
     }
+    if (threadIdx.x < 16) unsent[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         *abort = 0;
+        *down = 0;
         for (int i = 0; i < kMmaBars; ++i) mbar_init(&bars[i], 1);
         fence_mbar_init();
     }
@@ -667,6 +681,7 @@ __global__ void __launch_bounds__(mma_threads(OC), 1)
     // every lane waits (each gets the acquire); the outcome is made warp-uniform so
     // that the aligned MMAs never run divergent
     bool ok = true;
+    int armed = 0, seen = 0;   // last layer whose input this thread has armed, and waited for
     auto wait = [&](uint64_t* bar, uint32_t parity, bool cluster) {
         const bool r = ok && (cluster ? mbar_wait_cluster(bar, parity, abort, a.timeout_ns)
                                       : mbar_wait(bar, parity, abort, a.timeout_ns));
@@ -747,14 +762,17 @@ __global__ void __launch_bounds__(mma_threads(OC), 1)
         const uint8_t* const xa = xs + k0 / OC * SS + g * RB + k0 % OC * 2;
         const bool relu = (a.flags & 4u) != 0, residual = (a.flags & 2u) != 0;
         uint32_t use = 0;
+        int sent = 0;   // slices that this lane has sent
         __syncthreads();   // x_t and the biases in place
 
         for (int l = 0; l < L; ++l) {
             const uint32_t xb = l & 1;
             const bool recv = prow[l] >= 0;
             // the next layer's input arrives as a slice from every CTA of the cluster
-            if (threadIdx.x == 0 && l + 1 < L)
+            if (threadIdx.x == 0 && ok && l + 1 < L) {
                 mbar_arrive_expect_tx(&xs_bar[xb ^ 1], a.csize * SB);
+                armed = l + 1;
+            }
             const float2 bv = *reinterpret_cast<const float2*>(bias + l * OC);
             if (SPLIT) {
 #pragma unroll
@@ -797,6 +815,7 @@ __global__ void __launch_bounds__(mma_threads(OC), 1)
             }
             const uint8_t* xl = xa + xb * xbuf;
             if (l > 0) wait(&xs_bar[xb], ((l - 1) >> 1) & 1, true);
+            if (ok) seen = l;
 #pragma unroll
             for (int i = 0; i < GP; ++i)
                 if (i < ng) {
@@ -862,32 +881,48 @@ __global__ void __launch_bounds__(mma_threads(OC), 1)
                 // free: the copies of two layers ago were part of inputs since used.)
                 fence_proxy_async_smem();
                 named_bar_sync(1, kMmaWarps * 32);
-                if (ok && sends)
+                if (ok && sends) {
                     copy_to_peer(smem_u32(xs) + (xb ^ 1) * xbuf + q * SS + peer,
                                  smem_u32(slice) + (xb ^ 1) * SB, SB,
                                  smem_u32(xs_bar) + 8 * (xb ^ 1) + peer);
+                    ++sent;
+                }
                 __syncwarp();
             }
         }
+        if (!ok) {   // a warp that gave up: every CTA is told, and what it was not sent
+            if (sends) st_remote(mapa_shared(const_cast<int*>(unsent) + q, to), L - 1 - sent);
+            if (lane < a.csize) st_remote(mapa_shared(const_cast<int*>(down), lane), 1);
+        }
     }
-    // Normally every copy has been waited for as part of an input.  After an abort the
-    // ones in flight, from and to this CTA, get ample time to land before it leaves.
-    auto settle = [&]() {
-        if (*abort)
-            for (const uint64_t t0 = globaltimer_ns(); globaltimer_ns() - t0 < 100000;) {
-            }
-    };
-    settle();
     __syncwarp();
-    cluster_sync_all();   // no CTA leaves while a peer may still write its shared memory
-    settle();
+    cluster_sync_all();   // no CTA sends any more
+    // Normally every copy has been waited for as part of an input.  After an abort the ones
+    // on their way into this CTA are: the bytes of the slices that were not sent are taken
+    // off an input's barrier, and it completes when the others have landed.  (At most two
+    // inputs are under way, on different barriers: a CTA sends the one after next only with
+    // this CTA's slice of the next.)  Then all CTAs leave, with nothing read from them either.
+    if (*down) {
+        if (threadIdx.x == 0)
+            for (int l = seen + 1; l < L; ++l) {
+                int n = 0;
+                for (int i = 0; i < a.csize; ++i) n += L - 1 - unsent[i] >= l;
+                if (n == 0) break;
+                uint64_t* bar = &xs_bar[l & 1];
+                if (l > armed) mbar_arrive_expect_tx(bar, a.csize * SB);
+                if (n < a.csize) mbar_complete_tx(bar, (a.csize - n) * SB);
+                if (!mbar_wait_drain(bar, ((l - 1) >> 1) & 1, kDrainNs)) break;
+            }
+        __syncthreads();
+        cluster_sync_all();
+    }
 }
 
 size_t decode_mma_smem(int d, int oc, int L) {
     return (size_t)2 * (d / oc) * mma_slice_step(oc) + 2 * mma_slice_bytes(oc) +
            (size_t)kMmaWarps * kRows * mma_sum_row(oc) * 4 +
            (mma_split(oc) ? (size_t)2 * kPWarps * kRows * oc * 4 : 0) + kMmaBars * 8 +
-           kMaxDecodeLayers * 12 + 16 + (size_t)L * oc * 4;
+           kMaxDecodeLayers * 12 + 16 + 64 + (size_t)L * oc * 4;
 }
 
 }  // namespace
