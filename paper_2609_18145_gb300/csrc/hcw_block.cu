@@ -18,6 +18,7 @@
 // and its gradient are fp32; the GEMM operands are bf16 (h, M(h), g, relu(u),
 // hf, dlogits, bf16(dx), the FFN pre-activation gradient); the other GEMM
 // outputs are fp32.
+#include <float.h>
 #include <mutex>
 #include <vector>
 
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(kRowWarps * 32)
         const float zt = tail ? z[vt] + bh[vt] : -INFINITY;
         // running maximum m (finite, so that a logit of -inf adds 0) and sum s of exp(z - m)
         // of the lane's symbols, in one pass
-        float m = fmaxf(zt, -3.4e38f), s = expf(zt - m);
+        float m = fmaxf(zt, -FLT_MAX), s = expf(zt - m);
 #pragma unroll 4
         for (int v = 4 * lane; v < v4; v += 128) {
             const float4 q = add4(ld4(z, v), ld4(bh, v));
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(kRowWarps * 32)
         const float zt = tail ? z[vt] + bh[vt] : -INFINITY;
         const float ztgt = z[tgt] + bh[tgt];
         float4 q[NV];
-        float m = fmaxf(zt, -3.4e38f);   // finite, so that a logit of -inf adds 0
+        float m = fmaxf(zt, -FLT_MAX);   // finite, so that a logit of -inf adds 0
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
             const int v = 4 * (ti + i * kThreads);

@@ -136,6 +136,30 @@ def test_an_id_outside_the_vocabulary_is_reported(H):
     assert H.hcw_sync_status() == H.HCW_OK      # the report is read once
 
 
+@pytest.mark.parametrize("V", [11, 130, 1000, 8193])
+def test_logits_at_the_lowest_value(H, V):
+    """A head bias that masks symbols with the lowest fp32 value: rows of which every symbol
+    is masked so (their logits all round to that value) stay finite, and up to 8,192 symbols
+    get the uniform distribution's gradient; with one symbol left open it takes all."""
+    B, n, d, h, L = 2, 16, 64, 128, 1
+    ids, params, _ = device_problem(synth.block_problem(B, n, d, h, V, L, seed=12))
+    low = torch.finfo(torch.float32).min
+    params["bh"] = torch.full_like(params["bh"], low)
+    loss, grads = H.hcw_block_step(ids, params)
+    assert torch.isfinite(loss).all() and all(bool(torch.isfinite(g).all()) for g in grads.values())
+    want = -torch.bincount(ids[:, 1:].flatten().long(), minlength=V).double() / (B * n)
+    if V <= 8192:
+        # each position's entry is a bf16: half an ulp, 2^-9, of itself
+        bound = 2.0 ** -9 * (want.abs() + 1.0 / V) * 1.01
+        assert bool(((grads["bh"].double() - (want + 1.0 / V)).abs() <= bound).all())
+    params["bh"][3] = 0.0
+    loss, grads = H.hcw_block_step(ids, params)
+    want[3] += 1.0
+    assert bool(((grads["bh"].double() - want).abs() <= 2.0 ** -8).all())
+    assert all(bool(torch.isfinite(g).all()) for g in grads.values())
+    assert H.hcw_sync_status() == H.HCW_OK
+
+
 @pytest.mark.parametrize("offset", [16, 64])
 @pytest.mark.parametrize("case", [(4, 64, 128, 256, 37, 3), (2, 64, 192, 384, 130, 2)],
                          ids=lambda c: "B%d_n%d_d%d_h%d_V%d_L%d" % c)
