@@ -465,8 +465,8 @@ WsLayout ws_layout(long long tokens, int d, int dtype, unsigned flags) {
     }
     l.col_off = l.part_bytes;   // relative to w_off
     l.col_bytes = align256(colsum_workspace_bytes(tokens, d));
-    // fp32: the split's partial sums, or the column sums' size where that is larger
-    // (what callers without an allocator were promised to fit stays so)
+    // fp32: the split's partial sums; no less than the bf16 column sums' size, which no
+    // fp32 kernel uses but which the limit of the call without a workspace is stated in
     if (dtype != HCW_BF16) {
         const size_t part = f32_part_bytes(tokens, d, 1);
         if (part > l.col_bytes) l.col_bytes = part;

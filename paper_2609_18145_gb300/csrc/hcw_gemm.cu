@@ -97,7 +97,7 @@ struct GemmArgs {
     int batched;
     uint32_t stage_tx;          // bytes one CTA's two copies of a stage land
     uint32_t stage_tx_half;     // the same in a half unit; 0 where every unit is whole
-    int vec;                    // rows of the output start 16-byte aligned
+    int vec;                    // bf16 output: its rows start 16-byte aligned
     unsigned long long timeout_ns;
 };
 
@@ -496,68 +496,66 @@ __global__ void __launch_bounds__(kGThreads, 1) gemm_pair_kernel(const __grid_co
                 }
                 if (row >= a.M || col0 >= a.N) continue;
                 const bool full = a.vec && col0 + 32 <= a.N;
-                {
-                    __nv_bfloat16* dst = a.out + (size_t)row * a.N + col0;
-                    if (full) {
-                        float v[32];
-                        if (EPI == EPI_BIAS_RELU) {
-                            const float4* b4 = reinterpret_cast<const float4*>(a.bias + col0);
+                __nv_bfloat16* dst = a.out + (size_t)row * a.N + col0;
+                if (full) {
+                    float v[32];
+                    if (EPI == EPI_BIAS_RELU) {
+                        const float4* b4 = reinterpret_cast<const float4*>(a.bias + col0);
 #pragma unroll
-                            for (int m = 0; m < 8; ++m) {
-                                const float4 b = __ldg(b4 + m);
-                                v[4 * m] = __uint_as_float(raw[4 * m]) + b.x;
-                                v[4 * m + 1] = __uint_as_float(raw[4 * m + 1]) + b.y;
-                                v[4 * m + 2] = __uint_as_float(raw[4 * m + 2]) + b.z;
-                                v[4 * m + 3] = __uint_as_float(raw[4 * m + 3]) + b.w;
-                            }
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) v[i] = v[i] > 0.f ? v[i] : 0.f;
-                        } else {
-                            const uint4* m4 =
-                                reinterpret_cast<const uint4*>(a.aux + (size_t)row * a.N + col0);
-#pragma unroll
-                            for (int m = 0; m < 4; ++m) {
-                                const uint4 q = __ldg(m4 + m);
-                                const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-                                for (int j = 0; j < 4; ++j) {
-                                    const float2 am = unpack_bf16x2(w[j]);
-                                    const int i = 8 * m + 2 * j;
-                                    v[i] = am.x > 0.f ? __uint_as_float(raw[i]) : 0.f;
-                                    v[i + 1] = am.y > 0.f ? __uint_as_float(raw[i + 1]) : 0.f;
-                                }
-                            }
+                        for (int m = 0; m < 8; ++m) {
+                            const float4 b = __ldg(b4 + m);
+                            v[4 * m] = __uint_as_float(raw[4 * m]) + b.x;
+                            v[4 * m + 1] = __uint_as_float(raw[4 * m + 1]) + b.y;
+                            v[4 * m + 2] = __uint_as_float(raw[4 * m + 2]) + b.z;
+                            v[4 * m + 3] = __uint_as_float(raw[4 * m + 3]) + b.w;
                         }
 #pragma unroll
-                        for (int m = 0; m < 4; ++m)
-                            reinterpret_cast<uint4*>(dst)[m] = make_uint4(
-                                pack_bf16x2(v[8 * m], v[8 * m + 1]),
-                                pack_bf16x2(v[8 * m + 2], v[8 * m + 3]),
-                                pack_bf16x2(v[8 * m + 4], v[8 * m + 5]),
-                                pack_bf16x2(v[8 * m + 6], v[8 * m + 7]));
-                        if (EPI == EPI_RELU_GRAD && a.colsum) {
-#pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                atomicAdd(a.colsum + col0 + i,
-                                          __bfloat162float(__float2bfloat16_rn(v[i])));
-                        }
+                        for (int i = 0; i < 32; ++i) v[i] = v[i] > 0.f ? v[i] : 0.f;
                     } else {
+                        const uint4* m4 =
+                            reinterpret_cast<const uint4*>(a.aux + (size_t)row * a.N + col0);
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            if (col0 + i >= a.N) continue;
-                            float x = __uint_as_float(raw[i]);
-                            if (EPI == EPI_BIAS_RELU) {
-                                x += a.bias[col0 + i];
-                                x = x > 0.f ? x : 0.f;
-                            } else {
-                                const float am =
-                                    __bfloat162float(a.aux[(size_t)row * a.N + col0 + i]);
-                                x = am > 0.f ? x : 0.f;
+                        for (int m = 0; m < 4; ++m) {
+                            const uint4 q = __ldg(m4 + m);
+                            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const float2 am = unpack_bf16x2(w[j]);
+                                const int i = 8 * m + 2 * j;
+                                v[i] = am.x > 0.f ? __uint_as_float(raw[i]) : 0.f;
+                                v[i + 1] = am.y > 0.f ? __uint_as_float(raw[i + 1]) : 0.f;
                             }
-                            dst[i] = __float2bfloat16_rn(x);
-                            if (EPI == EPI_RELU_GRAD && a.colsum)
-                                atomicAdd(a.colsum + col0 + i, __bfloat162float(dst[i]));
                         }
+                    }
+#pragma unroll
+                    for (int m = 0; m < 4; ++m)
+                        reinterpret_cast<uint4*>(dst)[m] = make_uint4(
+                            pack_bf16x2(v[8 * m], v[8 * m + 1]),
+                            pack_bf16x2(v[8 * m + 2], v[8 * m + 3]),
+                            pack_bf16x2(v[8 * m + 4], v[8 * m + 5]),
+                            pack_bf16x2(v[8 * m + 6], v[8 * m + 7]));
+                    if (EPI == EPI_RELU_GRAD && a.colsum) {
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            atomicAdd(a.colsum + col0 + i,
+                                      __bfloat162float(__float2bfloat16_rn(v[i])));
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        if (col0 + i >= a.N) continue;
+                        float x = __uint_as_float(raw[i]);
+                        if (EPI == EPI_BIAS_RELU) {
+                            x += a.bias[col0 + i];
+                            x = x > 0.f ? x : 0.f;
+                        } else {
+                            const float am =
+                                __bfloat162float(a.aux[(size_t)row * a.N + col0 + i]);
+                            x = am > 0.f ? x : 0.f;
+                        }
+                        dst[i] = __float2bfloat16_rn(x);
+                        if (EPI == EPI_RELU_GRAD && a.colsum)
+                            atomicAdd(a.colsum + col0 + i, __bfloat162float(dst[i]));
                     }
                 }
             }
@@ -1022,7 +1020,6 @@ cudaError_t gemm_bf16(int M, int N, int K, const void* A, bool ta, const void* B
     if (epi.kind == EPI_F32) {
         a.C = a.splits > 1 ? split_ws : C;
         a.ldc = ldc;
-        a.vec = (ldc % 4 == 0) && aligned(a.C);
         a.tma_out = map_out_f32(&a.mOut, a.C, M, N, ldc, a.splits);
     } else {
         a.out = epi.out;
@@ -1104,7 +1101,6 @@ cudaError_t gemm_bf16_f32_batched(int M, int N, int K, const void* A, size_t a_b
     a.kps = (K + kGK - 1) / kGK;
     a.C = C;
     a.ldc = N;
-    a.vec = N % 4 == 0;
     a.tma_out = map_out_f32(&a.mOut, C, M, N, N, batch);
     a.timeout_ns = kGemmTimeoutNs;
     const int sms = gemm_sms();

@@ -632,10 +632,10 @@ __global__ void relu_grad_mask_f32_kernel(const float* dy, const uint32_t* mask,
 
 // The same for bf16 rows (d a multiple of 64): one thread per 16 bytes of a
 // row, so a group never straddles a mask word.
-template <typename V>
-__global__ void relu_grad_mask_kernel(const V* __restrict__ dy, const uint32_t* __restrict__ mask,
-                                      V* __restrict__ dz, long long rows, int d) {
-    constexpr int VEC = 16 / sizeof(V);
+__global__ void relu_grad_mask_kernel(const __nv_bfloat16* __restrict__ dy,
+                                      const uint32_t* __restrict__ mask,
+                                      __nv_bfloat16* __restrict__ dz, long long rows, int d) {
+    constexpr int VEC = 8;
     const int wpr = d >> 5;
     const int gpr = d / VEC;   // groups per row
     const size_t count = (size_t)rows * gpr;
@@ -646,15 +646,10 @@ __global__ void relu_grad_mask_kernel(const V* __restrict__ dy, const uint32_t* 
         const uint32_t bits = (mask[r * wpr + (o >> 5)] >> (o & 31)) & ((1u << VEC) - 1u);
         uint4 v = reinterpret_cast<const uint4*>(dy)[t];
         uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        if (VEC == 8) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                w[i] &= ((bits >> (2 * i)) & 1u ? 0x0000FFFFu : 0u) |
-                        ((bits >> (2 * i + 1)) & 1u ? 0xFFFF0000u : 0u);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) w[i] = (bits >> i) & 1u ? w[i] : 0u;
-        }
+        for (int i = 0; i < 4; ++i)
+            w[i] &= ((bits >> (2 * i)) & 1u ? 0x0000FFFFu : 0u) |
+                    ((bits >> (2 * i + 1)) & 1u ? 0xFFFF0000u : 0u);
         reinterpret_cast<uint4*>(dz)[t] = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
@@ -663,14 +658,12 @@ __global__ void relu_grad_mask_kernel(const V* __restrict__ dy, const uint32_t* 
 // fill the GPU), 256 above (the partials stay small)
 inline long long col_rows(long long rows) { return rows <= 65536 ? 64 : 256; }
 
-// partial[c][o] = sum_{r in chunk c} dz[r][o] for bf16 rows (d a multiple of 64),
-// 16-byte loads.  Block: 64
-// column groups of 16 bytes x 4 row lanes; each thread sums its group over every 4th row of
-// the chunk, then the 4 row lanes are added in a fixed order.
-template <typename V>
-__global__ void colsum_partial_kernel(const V* __restrict__ dz, long long rows, int d, int crows,
-                                      float* __restrict__ partial) {
-    constexpr int VEC = 16 / sizeof(V);
+// partial[c][o] = sum_{r in chunk c} dz[r][o] for bf16 rows (d a multiple of 64), 16-byte
+// loads.  Block: 64 column groups of 16 bytes x 4 row lanes; each thread sums its group over
+// every 4th row of the chunk, then the 4 row lanes are added in a fixed order.
+__global__ void colsum_partial_kernel(const __nv_bfloat16* __restrict__ dz, long long rows, int d,
+                                      int crows, float* __restrict__ partial) {
+    constexpr int VEC = 8;
     __shared__ float red[4][64][VEC + 1];
     // blockIdx.z selects one of several equally shaped matrices (layers)
     dz += (size_t)blockIdx.z * rows * d;
@@ -686,9 +679,9 @@ __global__ void colsum_partial_kernel(const V* __restrict__ dz, long long rows, 
         const uint4* src = reinterpret_cast<const uint4*>(dz) + g;
         for (long long r = r0 + threadIdx.y; r < r1; r += 4) {
             const uint4 q = src[(size_t)r * gpr];
-            const V* e = reinterpret_cast<const V*>(&q);
+            const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&q);
 #pragma unroll
-            for (int i = 0; i < VEC; ++i) acc[i] += to_f(e[i]);
+            for (int i = 0; i < VEC; ++i) acc[i] += __bfloat162float(e[i]);
         }
     }
 #pragma unroll
@@ -823,8 +816,8 @@ cudaError_t launch_relu_grad_mask_f32(const float* dy, const uint32_t* mask, flo
 cudaError_t launch_relu_grad_mask_bf16(const __nv_bfloat16* dy, const uint32_t* mask,
                                        __nv_bfloat16* dz, long long rows, int d,
                                        cudaStream_t st) {
-    relu_grad_mask_kernel<__nv_bfloat16>
-        <<<blocks_for((size_t)rows * d / 8, 256), 256, 0, st>>>(dy, mask, dz, rows, d);
+    relu_grad_mask_kernel<<<blocks_for((size_t)rows * d / 8, 256), 256, 0, st>>>(dy, mask, dz, rows,
+                                                                               d);
     return cudaGetLastError();
 }
 
@@ -949,30 +942,28 @@ size_t colsum_workspace_bytes(long long rows, int d) {
     return (size_t)(chunks < 1 ? 1 : chunks) * (size_t)d * sizeof(float);
 }
 
-template <typename V>
-static cudaError_t colsum(const V* dz, long long rows, int d, float* partial, float* out,
-                          cudaStream_t st, int batch = 1) {
+static cudaError_t colsum(const __nv_bfloat16* dz, long long rows, int d, float* partial,
+                          float* out, cudaStream_t st, int batch = 1) {
     const int crows = (int)col_rows(rows);
     const long long chunks = (rows + crows - 1) / crows;
     if (chunks == 0) {
         cudaError_t e = cudaMemsetAsync(out, 0, (size_t)batch * d * sizeof(float), st);
         return e;
     }
-    constexpr int VEC = 16 / sizeof(V);
-    dim3 grid((d / VEC + 63) / 64, (unsigned)chunks, (unsigned)batch);
-    colsum_partial_kernel<V><<<grid, dim3(64, 4), 0, st>>>(dz, rows, d, crows, partial);
+    dim3 grid((d / 8 + 63) / 64, (unsigned)chunks, (unsigned)batch);
+    colsum_partial_kernel<<<grid, dim3(64, 4), 0, st>>>(dz, rows, d, crows, partial);
     colsum_final_kernel<<<dim3((d + 31) / 32, batch), 1024, 0, st>>>(partial, (int)chunks, d, out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_colsum_bf16_batched(const __nv_bfloat16* dz, int batch, long long rows, int d,
                                        float* partial, float* out, cudaStream_t st) {
-    return colsum<__nv_bfloat16>(dz, rows, d, partial, out, st, batch);
+    return colsum(dz, rows, d, partial, out, st, batch);
 }
 
 cudaError_t launch_colsum_bf16(const __nv_bfloat16* dz, long long rows, int d, float* partial,
                                float* out, cudaStream_t st) {
-    return colsum<__nv_bfloat16>(dz, rows, d, partial, out, st);
+    return colsum(dz, rows, d, partial, out, st);
 }
 
 cudaError_t launch_splitk_reduce(const float* partial, int splits_max, int splits_self,
