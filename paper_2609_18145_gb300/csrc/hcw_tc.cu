@@ -1183,6 +1183,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                 constexpr bool fwd = decltype(fwd_tag)::value;
                 constexpr int RB = WCOLS * 2;                  // patch row bytes (128 or 64)
                 constexpr int SUB = WCOLS / 32;                // 32-column sub-chunks per patch
+                static_assert(SUB == 1 || SUB == 2, "mask words of a warp's columns");
                 RowUnit r = decode_row_unit(p, ul, STACKED, !fwd && MODE == MODE_FDX,
                                             STACKED && ly.shift > 0);
                 if (PAIR) r.t = 2 * r.t + (int)rank;
@@ -1396,6 +1397,19 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                     }
                     __syncwarp();
                 };
+                // FWD: the ReLU mask words.  A later launch reads them, so they go out after
+                // the signal, off the layer chain; in the fused launch its own input gradient
+                // does, which the signal has to order behind them.
+                auto store_mask = [&]() {
+                    if (fwd && ly.mout && tok_row >= 0) {
+                        uint32_t* m = ly.mout + (size_t)tok_row * wpr + (col0 >> 5);
+                        if constexpr (SUB == 2)   // (an even word of a row of whole pairs)
+                            *reinterpret_cast<uint2*>(m) = make_uint2(mbits[0], mbits[1]);
+                        else
+                            m[0] = mbits[0];
+                    }
+                    if (MODE == MODE_FDX) __syncwarp();
+                };
                 if (has_mprev) {
                     // the dz patch (the next layer's MMA operand) first
                     publish();
@@ -1464,6 +1478,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                             bulk_commit();
                         }
                     }
+                    if (MODE == MODE_FDX) store_mask();
                     if (signal) count(L.counters, 0);
                 }
                 // FWD z (layer API only): the pre-activation, from the accumulator
@@ -1500,13 +1515,7 @@ __global__ void __launch_bounds__(cta_threads(BN), 1)
                         bulk_commit();
                     }
                 }
-                // FWD: the ReLU mask words, read only by the input gradient (a later
-                // launch), after the signal so that they stay off the layer chain
-                if (fwd && ly.mout && tok_row >= 0) {
-#pragma unroll
-                    for (int h = 0; h < SUB; ++h)
-                        ly.mout[(size_t)tok_row * wpr + (col0 >> 5) + h] = mbits[h];
-                }
+                if (MODE != MODE_FDX) store_mask();
                 return true;
                 };
                 bool ok_unit;
