@@ -389,6 +389,9 @@ int hcw_set_stack_kernels(int mode);
  * Which family the bf16 stacked forward and input gradient of these sizes
  * would run on under the current setting (on the current device):
  * HCW_STACK_RESIDENT or HCW_STACK_STREAMING; -1 for invalid sizes or dtype.
+ * HCW_STACK_STREAMING also stands for the kernel that keeps 128 tokens on chip,
+ * whose results are the streaming kernels' (whether it runs depends on the
+ * layers and the direction too).
  */
 int hcw_stack_kernels_used(int B, int n, int d, int dtype);
 
@@ -523,8 +526,10 @@ int hcw_block_step(const int* ids, const hcw_block_params* params, const hcw_blo
  * is split across CTAs, and padded copies of operands whose rows TMA cannot read
  * (a K-major row not a multiple of 16 bytes, an MN-major one not a multiple of 64
  * elements, a pointer not 16-byte aligned): hcw_gemm_workspace_bytes gives the
- * size that allows the copies and the best split; a smaller one allows fewer
- * splits, NULL none.  Partial sums are added in split order.  Without room for
+ * size that allows the copies and the best split (no copies where M and N are
+ * multiples of 64 and K of 8: TMA reads such rows in every layout, whatever the
+ * pointer); a smaller one allows fewer splits, NULL none.  Partial sums are added
+ * in split order.  Without room for
  * the copies (and where they would not pay) such operands take a plain tiled
  * kernel.
  * Asynchronous on `stream`.
