@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(kRowWarps * 32)
 // takes rows w, w + 8, ..., eight at a time, whose sum in pairs joins its chain (at most
 // 16 such sums, where one row after the other made chains of 128), then the warps' sums
 // meet in shared memory in pairs.  33 passes of d = 512: 29 us with a column a lane and
-// 32 warps a CTA, 21 so.
+// 32 warps a CTA, 21 so with a chain of rows a warp; on its own and cold 18.0, in pairs 15.7.
 constexpr int kMaxLnJobs = 64;
 struct LnJob {
     const float* part;
