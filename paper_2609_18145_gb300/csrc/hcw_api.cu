@@ -398,15 +398,17 @@ double dw_cost(const WPlan& w, long long tokens, int d, int layers) {
 WPlan plan_dw(long long tokens, int d, unsigned flags, int layers = 1) {
     const int whole = whole_bn(d);
     WPlan best = split_dw(tokens, d, flags, layers, whole);
-    if (d % 256 == 0 || tokens <= 2048) return best;
+    // Fewer, wider tiles are split more often, with more partial sums: whole tiles decide
+    // which sizes fit the scratch of the call without a workspace.
+    auto fits = [&](const WPlan& w) {
+        return layers > 1 || dw_part_bytes(w, d) + align256(colsum_workspace_bytes(tokens, d)) <=
+                                 kNoAllocScratchBytes;
+    };
+    if (d % 256 == 0 || tokens <= 2048 || !fits(best)) return best;
     double least = 0;
     for (int bn = 64; bn <= 256 && bn < 2 * d; bn *= 2) {
         const WPlan w = split_dw(tokens, d, flags, layers, bn);
-        // Fewer, wider tiles are split more often, with more partial sums: sizes that fit
-        // the scratch of the call without a workspace with whole tiles keep fitting it.
-        if (layers == 1 && bn != whole &&
-            dw_part_bytes(w, d) + align256(colsum_workspace_bytes(tokens, d)) > kNoAllocScratchBytes)
-            continue;
+        if (!fits(w)) continue;
         const double c = dw_cost(w, tokens, d, layers);
         if (least == 0 || c <= least) {
             least = c;
